@@ -45,6 +45,12 @@ void launch_tail_inverse(cudaStream_t, int, int, const int32_t*, const int32_t*,
                          const double*, double*, double*, float*, float*);
 void launch_adj_values(cudaStream_t, int, const int32_t*, const double*, const double*,
                        const double*, double*, double*);
+void launch_branch_count(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
+                         const int32_t*, int32_t*);
+void launch_branch_cols(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
+                        const int32_t*, const Ell<double>&, int, const double*, const double*,
+                        const double*, const int32_t*, const int32_t*, const int32_t*,
+                        const int32_t*, int32_t*, double*, double*, double*);
 void launch_ext_rows(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
                      const int32_t*, const double*, const double*, const int32_t*, int32_t*,
                      double*, float*, double*, float*);
@@ -132,6 +138,10 @@ struct MatDev {
   int32_t* xrow = nullptr;
   double *xval = nullptr, *xdiag = nullptr;
   float *xval32 = nullptr, *xdiag32 = nullptr;
+  // the branches' columns in the complete factor (null without one)
+  int32_t *parent = nullptr, *br_ptr = nullptr, *br_row = nullptr;
+  double *br_fv = nullptr, *br_fm = nullptr, *br_sc = nullptr;
+  BranchCols cols() const { return BranchCols{br_ptr, br_row, br_fv, br_fm, br_sc}; }
   template <typename VT>
   DevMatT<VT> view(bool f16 = false) const;
 };
@@ -155,6 +165,7 @@ DevMatT<double> MatDev::view<double>(bool) const {
   M.w = w;
   M.c = c;
   M.xptr = xptr; M.xrow = xrow; M.xval = xval; M.xdiag = xdiag; M.xnb = xnb; M.xbr = xbr;
+  M.br = cols();
   return M;
 }
 template <>
@@ -181,6 +192,7 @@ DevMatT<float> MatDev::view<float>(bool f16) const {
   M.w = w;
   M.c = c;
   M.xptr = xptr; M.xrow = xrow; M.xval = xval32; M.xdiag = xdiag32; M.xnb = xnb; M.xbr = xbr;
+  M.br = cols();
   return M;
 }
 
@@ -452,6 +464,44 @@ static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w) {
   return GPCG_OK;
 }
 
+// The branches' columns of a complete factor whose values are built: rows
+// from the elimination tree (the parent of row i: the first entry after the
+// diagonal in its column), then values and scalars.  Synchronous.
+static gpcg_status build_branch_rows(gpcg_ctx* c, MatDev& M, std::vector<void*>& own) {
+  const MatrixPlan& P = M.plan;
+  const int m = c->m;
+  std::vector<int32_t> parent(std::max(P.n, 1), -1), ptr(m + 1, 0);
+  for (int i = 0; i < P.n; ++i)
+    if (P.U.ptr[i] + 1 < P.U.ptr[i + 1]) parent[i] = P.U.idx[P.U.ptr[i] + 1];
+  CUDA_TRY(upload(own, &M.parent, parent.data(), parent.size()));
+  CUDA_TRY(dalloc(own, &M.br_ptr, (size_t)m + 1));
+  launch_branch_count(0, m, c->G.f, c->G.t, M.row_of_bus, M.parent, M.br_ptr + 1);
+  CUDA_TRY(cudaMemcpy(ptr.data() + 1, M.br_ptr + 1, (size_t)m * 4, cudaMemcpyDeviceToHost));
+  size_t total = 0;
+  for (int l = 0; l < m; ++l) {
+    total += (size_t)ptr[l + 1];
+    ptr[l + 1] = (int32_t)total;
+  }
+  if (total > (size_t)INT32_MAX) {  // beyond the 32-bit positions: no columns
+    M.br_ptr = nullptr;
+    return GPCG_OK;
+  }
+  CUDA_TRY(cudaMemcpy(M.br_ptr, ptr.data(), ((size_t)m + 1) * 4, cudaMemcpyHostToDevice));
+  CUDA_TRY(dalloc(own, &M.br_row, total));
+  CUDA_TRY(dalloc(own, &M.br_fv, total));
+  CUDA_TRY(dalloc(own, &M.br_fm, total));
+  CUDA_TRY(dalloc(own, &M.br_sc, (size_t)m * SC_N));
+  return GPCG_OK;
+}
+
+static void launch_branch_values(const gpcg_ctx* c, const MatDev& M, const double* w,
+                                 cudaStream_t st) {
+  if (M.br_ptr)
+    launch_branch_cols(st, c->m, c->G.f, c->G.t, M.row_of_bus, M.parent, M.U.view<double>(),
+                       M.plan.n, M.inv_diag, w, M.c, c->G.pre, c->isl.br_lo, c->isl.br_cnt,
+                       M.br_ptr, M.br_row, M.br_fv, M.br_fm, M.br_sc);
+}
+
 static gpcg_status build_matrix(gpcg_ctx* c, MatDev& M, int which,
                                 const std::vector<uint8_t>& keep, double* w, double* cf,
                                 bool fill) {
@@ -516,7 +566,16 @@ static gpcg_status build_matrix(gpcg_ctx* c, MatDev& M, int which,
   }
   M.w = w;
   M.c = cf;
-  return fill_values(c, M, w);
+  M.br_ptr = nullptr;
+  gpcg_status st = fill_values(c, M, w);
+  if (st == GPCG_OK && fill) {
+    st = build_branch_rows(c, M, own);
+    if (st == GPCG_OK) {
+      launch_branch_values(c, M, w, 0);
+      CUDA_TRY(cudaGetLastError());
+    }
+  }
+  return st;
 }
 
 static gpcg_status build_matrices(gpcg_ctx* c) {
@@ -1018,7 +1077,10 @@ struct Layout {
   size_t vstride = 0, sstride = 0, vec_bytes = 0, bytes = 0;
 };
 
-static Layout make_layout(const gpcg_ctx* c, int T, int slots, size_t vt_size, bool zs = false) {
+// zs: z in shared memory; one: a single vector per slot (the reduced form of
+// the inner solve without extension rows), at wr
+static Layout make_layout(const gpcg_ctx* c, int T, int slots, size_t vt_size, bool zs = false,
+                          bool one = false) {
   Layout L;
   L.T = T;
   L.slots = slots;
@@ -1028,7 +1090,7 @@ static Layout make_layout(const gpcg_ctx* c, int T, int slots, size_t vt_size, b
   L.sstride = (size_t)c->n * T;
   L.vec_bytes = ((L.vstride * vt_size + 255) / 256) * 256;
   const size_t st_bytes = ((L.sstride * 8 + 255) / 256) * 256;
-  L.bytes = (size_t)slots * ((zs ? 4 : 5) * L.vec_bytes + 4 * st_bytes);
+  L.bytes = (size_t)slots * ((one ? 1 : zs ? 4 : 5) * L.vec_bytes + 4 * st_bytes);
   return L;
 }
 
@@ -1037,15 +1099,22 @@ static Layout make_layout(const gpcg_ctx* c, int T, int slots, size_t vt_size, b
 template <typename VT>
 static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, int slots,
                             bool f16 = false, bool zs = false) {
-  Layout Lo = make_layout(c, T, slots, sizeof(VT), zs);
+  const DevMatT<VT> MP = c->MP.view<VT>(f16), MQ = c->MQ.view<VT>(f16);
+  const bool red = !zs && reduced_form(P.precond, MP, MQ);
+  const bool one = red && !P.sc.gen_bus && !P.G.qmax;
+  Layout Lo = make_layout(c, T, slots, sizeof(VT), zs, one);
   gpcg_status s = ensure_work(c, Lo.bytes);
   if (s != GPCG_OK) return s;
   char* base = (char*)c->work;
   const size_t vb = (size_t)slots * Lo.vec_bytes;
   const size_t sb = (size_t)slots * (((Lo.sstride * 8 + 255) / 256) * 256);
-  const int nv = zs ? 4 : 5;
-  P.wx = base; P.wr = base + vb; P.wp = base + 2 * vb; P.wq = base + 3 * vb;
-  P.wz = zs ? nullptr : base + 4 * vb;
+  const int nv = one ? 1 : zs ? 4 : 5;
+  if (one) {
+    P.wr = base;
+  } else {
+    P.wx = base; P.wr = base + vb; P.wp = base + 2 * vb; P.wq = base + 3 * vb;
+    P.wz = zs ? nullptr : base + 4 * vb;
+  }
   P.vstride = Lo.vec_bytes / sizeof(VT);
   double* sbase = (double*)(base + nv * vb);
   const size_t ss = sb / slots / 8;
@@ -1054,8 +1123,7 @@ static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, i
   P.sstride = ss;
   P.tile_counter = c->d_counter;
   CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st));
-  CUDA_TRY(launch_fdpf<VT>(st, T, slots, P, c->MP.view<VT>(f16), c->MQ.view<VT>(f16),
-                           zs ? Lo.vec_bytes : 0));
+  CUDA_TRY(launch_fdpf<VT>(st, T, slots, P, MP, MQ, zs ? Lo.vec_bytes : 0));
   return GPCG_OK;
 }
 
@@ -1315,6 +1383,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
   const bool ext = gen || c->G.qmax != nullptr;
   const bool f16 = c->opt.precision == GPCG_BATCHED_FP32_F16;
   const bool f32 = c->opt.precision == GPCG_BATCHED_FP32 || f16;
+  const bool red = reduced_form(c->opt.precond, c->MP.view<float>(f16), c->MQ.view<float>(f16));
   // islanding for every outage (the autotuner's probes need it too)
   // (inside a stream capture the events become event-record nodes of the graph)
   auto record = [](cudaEvent_t ev, cudaStream_t s, bool cap) {
@@ -1337,8 +1406,8 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
   // CTAs per SM of tile width t, with z in shared memory or not (0: does not fit)
   auto blocks = [&](int t, bool z) {
     const size_t zb = z ? make_layout(c, t, 1, f32 ? 4 : 8, true).vec_bytes : 0;
-    return f32 ? fdpf_max_blocks_per_sm<float>(t, ext, zb)
-               : fdpf_max_blocks_per_sm<double>(t, ext, zb);
+    return f32 ? fdpf_max_blocks_per_sm<float>(t, ext, zb, red)
+               : fdpf_max_blocks_per_sm<double>(t, ext, zb, red);
   };
   auto use_zs = [&](int t) {
     return c->zs_allowed && !ext && (t == 2 || t == 4) && blocks(t, true) > 0;
@@ -1516,7 +1585,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
   } else if (mem == GPCG_MEM_DEVICE && !c->phase_on) {
     // device mode: islanding + solve as one CUDA graph, captured on the
     // context's own stream for this argument set and replayed on `st`
-    Layout Lo = make_layout(c, T, slots, f32 ? 4 : 8, zs);
+    Layout Lo = make_layout(c, T, slots, f32 ? 4 : 8, zs, red && !ext && !zs);
     s_ = ensure_work(c, Lo.bytes);
     if (s_ != GPCG_OK) { cleanup(); return s_; }
     std::vector<uintptr_t> key = {S, (uintptr_t)T, (uintptr_t)slots,

@@ -60,6 +60,22 @@ struct Ell {
   const VT* oval = nullptr;
 };
 
+// The branches' columns in the complete Cholesky factor M = L L^T of a
+// base-case matrix, built once per factor (reduced_cg in fdpf_ops.cuh says
+// what for).  For branch l with v = c e_from - e_to on the matrix's rows, and
+// v_m its part on the main island (v itself unless l is a bridge), the rows
+// where L^-1 v can be nonzero are the ancestors of its ends in the
+// elimination tree: positions [ptr[l], ptr[l + 1]) of row (ascending), with
+// fv = L^-1 v and fm = L^-1 v_m there.  sc holds SC_N scalars per branch.
+enum { SC_VY = 0, SC_MY, SC_VM2, SC_CA, SC_CB, SC_W, SC_N = 6 };
+struct BranchCols {
+  const int32_t *ptr = nullptr, *row = nullptr;
+  const double *fv = nullptr, *fm = nullptr;
+  // v.M^-1 v_m, v_m.M^-1 v_m, v_m.v_m, the entries of v_m at the from and the
+  // to end's rows (0: no row, or the island's end), and the branch's weight
+  const double* sc = nullptr;
+};
+
 // One fast-decoupled matrix (B' or B'') with its base-case factor.  VT is
 // the value type used by the solve kernels (float or double).  Vectors of
 // this matrix have n+1 rows per scenario: row n is kept at zero and is what
@@ -98,6 +114,7 @@ struct DevMatT {
   const int32_t* xnb = nullptr;  // the neighbour bus of each adjacency entry
   const int32_t* xbr = nullptr;  // the branch of each adjacency entry
   const VT *xval = nullptr, *xdiag = nullptr;
+  BranchCols br;  // null pointers: the factor is not the complete one
 };
 
 // Extension rows a lane may carry at once (see Ext in fdpf_ops.cuh): a

@@ -122,9 +122,9 @@ cudaError_t launch_fdpf(cudaStream_t st, int T, int grid, const FdpfParams& P,
 }
 
 template <typename VT>
-int fdpf_max_blocks_per_sm(int T, bool gen, size_t zbytes) {
-  if (gen) return zbytes ? 0 : fdpf_blocks_gen<VT>(T);
-  return fdpf_blocks_g<false, VT>(T, zbytes);
+int fdpf_max_blocks_per_sm(int T, bool gen, size_t zbytes, bool red) {
+  if (gen) return zbytes ? 0 : fdpf_blocks_gen<VT>(T, red);
+  return fdpf_blocks_g<false, VT>(T, zbytes, red);
 }
 
 template <typename VT>
@@ -145,8 +145,8 @@ template cudaError_t launch_fdpf<float>(cudaStream_t, int, int, const FdpfParams
                                         const DevMatT<float>&, const DevMatT<float>&, size_t);
 template cudaError_t launch_fdpf<double>(cudaStream_t, int, int, const FdpfParams&,
                                          const DevMatT<double>&, const DevMatT<double>&, size_t);
-template int fdpf_max_blocks_per_sm<float>(int, bool, size_t);
-template int fdpf_max_blocks_per_sm<double>(int, bool, size_t);
+template int fdpf_max_blocks_per_sm<float>(int, bool, size_t, bool);
+template int fdpf_max_blocks_per_sm<double>(int, bool, size_t, bool);
 template cudaError_t launch_apply<float>(cudaStream_t, int, const DevMatT<float>&, int, int,
                                          const int32_t*, const int32_t*, const int32_t*,
                                          const double*, double*, float*, size_t, int);

@@ -48,6 +48,13 @@ struct FdpfParams {
   const int32_t* misq_order = nullptr;  // B'' rows sorted by their bus's degree
 };
 
+// Whether the inner solves run in their reduced form (reduced.cuh): the
+// complete base-case factor, in the precision of the vectors.
+template <typename VT>
+inline bool reduced_form(int precond, const DevMatT<VT>& MP, const DevMatT<VT>& MQ) {
+  return precond == PREC_EXACT && MP.br.ptr && MQ.br.ptr && !MP.Lh && !MQ.Lh;
+}
+
 // The persistent N-1 kernel for tiles of T scenarios (2 to 32; generator
 // outages, P.sc.gen_bus set: 2, 4 or 8) on `grid` slots.  zbytes > 0 (branch
 // outages without reactive limits, T = 2 or 4): each tile's z vector in
@@ -56,13 +63,13 @@ template <typename VT>
 cudaError_t launch_fdpf(cudaStream_t st, int T, int grid, const FdpfParams& P,
                         const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes = 0);
 template <typename VT>
-int fdpf_max_blocks_per_sm(int T, bool gen = false, size_t zbytes = 0);
+int fdpf_max_blocks_per_sm(int T, bool gen, size_t zbytes, bool red);
 // the generator-outage kernel (fdpf_gen.cu)
 template <typename VT>
 cudaError_t launch_fdpf_gen(cudaStream_t st, int T, int grid, const FdpfParams& P,
                             const DevMatT<VT>& MP, const DevMatT<VT>& MQ);
 template <typename VT>
-int fdpf_blocks_gen(int T);
+int fdpf_blocks_gen(int T, bool red);
 template <typename VT>
 cudaError_t launch_apply(cudaStream_t st, int grid, const DevMatT<VT>& M, int op, int S,
                          const int32_t* outages, const int32_t* f, const int32_t* t,

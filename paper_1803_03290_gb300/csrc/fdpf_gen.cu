@@ -14,15 +14,15 @@ cudaError_t launch_fdpf_gen(cudaStream_t st, int T, int grid, const FdpfParams& 
 }
 
 template <typename VT>
-int fdpf_blocks_gen(int T) {
-  return fdpf_blocks_g<true, VT>(T);
+int fdpf_blocks_gen(int T, bool red) {
+  return fdpf_blocks_g<true, VT>(T, 0, red);
 }
 
 template cudaError_t launch_fdpf_gen<float>(cudaStream_t, int, int, const FdpfParams&,
                                             const DevMatT<float>&, const DevMatT<float>&);
 template cudaError_t launch_fdpf_gen<double>(cudaStream_t, int, int, const FdpfParams&,
                                              const DevMatT<double>&, const DevMatT<double>&);
-template int fdpf_blocks_gen<float>(int);
-template int fdpf_blocks_gen<double>(int);
+template int fdpf_blocks_gen<float>(int, bool);
+template int fdpf_blocks_gen<double>(int, bool);
 
 }  // namespace gpcg

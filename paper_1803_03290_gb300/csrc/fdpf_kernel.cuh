@@ -30,6 +30,7 @@
 #include "common.cuh"
 #include "fdpf.h"
 #include "fdpf_ops.cuh"
+#include "reduced.cuh"
 
 namespace gpcg {
 
@@ -362,14 +363,15 @@ __device__ __forceinline__ double v_ratio(VT dv, double e, double f) {
 }
 
 // theta += dtheta (P half-step) or |V| += dV (Q half-step) on the matrix's
-// rows, as moves of the rectangular voltage: (e, f) rotated through dtheta
+// rows, (scale: the lanes' factors of x, 0 for no step; null: x + xalpha p) as moves of the rectangular voltage: (e, f) rotated through dtheta
 // (theta kept beside it), or e and f both scaled by 1 + dV/|V|, so that
 // e + jf = |V| exp(j theta) holds to FP64 rounding; lanes two at a time.
 template <int T, typename VT, bool IS_P, bool GEN>
 __device__ GPCG_LOOP_INLINE void update_pass(const DevMatT<VT>& M, LaneState<T>& L,
                                              const VT* __restrict__ x,
                                              const VT* __restrict__ p, double* th,
-                                             double* EF, const SwitchState<T>* SW = nullptr) {
+                                             double* EF, const SwitchState<T>* SW = nullptr,
+                                             const double* scale = nullptr) {
   constexpr int LP = Geo<T>::LP;
   const Geo<T> g;
   bool any = false;
@@ -382,14 +384,26 @@ __device__ GPCG_LOOP_INLINE void update_pass(const DevMatT<VT>& M, LaneState<T>&
 #pragma unroll 1
     for (int jp = 0; jp < LP; jp += 2) {
       const int l0 = g.lane + jp, l1 = l0 + 1;
-      const bool on0 = L.active[l0] && !in_island(pr, L.lo[l0], L.cnt[l0]);
-      const bool on1 = L.active[l1] && !in_island(pr, L.lo[l1], L.cnt[l1]);
+      bool on0 = L.active[l0] && !in_island(pr, L.lo[l0], L.cnt[l0]);
+      bool on1 = L.active[l1] && !in_island(pr, L.lo[l1], L.cnt[l1]);
+      VT xa0, xa1;
+      if (scale) {
+        xa0 = (VT)scale[l0];
+        xa1 = (VT)scale[l1];
+        on0 = on0 && xa0 != (VT)0;
+        on1 = on1 && xa1 != (VT)0;
+      } else {
+        xa0 = (VT)L.xalpha[l0];
+        xa1 = (VT)L.xalpha[l1];
+      }
       if (!on0 && !on1) continue;
       const size_t o = (size_t)i * T + l0;
       Pair<VT> dx = ld2(x + (size_t)k * T + l0);
-      // the inner solve's deferred last step, x += alpha p
-      const VT xa0 = (VT)L.xalpha[l0], xa1 = (VT)L.xalpha[l1];
-      if (xa0 != (VT)0 || xa1 != (VT)0) {
+      if (scale) {
+        dx.a *= xa0;
+        dx.b *= xa1;
+      } else if (xa0 != (VT)0 || xa1 != (VT)0) {
+        // the inner solve's deferred last step, x += alpha p
         const Pair<VT> pv = ld2(p + (size_t)k * T + l0);
         dx.a = fma(xa0, pv.a, dx.a);  // as the solve's own step would take it
         dx.b = fma(xa1, pv.b, dx.b);
@@ -668,10 +682,20 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T>& 
 // rather than on L2 or DRAM; the CTA then takes rows x T x sizeof(VT) bytes
 // of shared memory (80 KB for FP32 tiles of two on a 10,000-bus grid), two
 // CTAs fit an SM, and the register budget is set for two.
-template <int T, typename VT, bool GEN, bool ZS = false>
+//
+// RED: the inner solves in their reduced form (reduced.cuh), for the complete
+// base-case factor: one vector per slot, P.wr.  With extension rows (GEN) the
+// Q solves stay with the PCG over five vectors.
+template <int T, typename VT, bool GEN, bool ZS = false, bool RED = false>
 __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
     fdpf_tiles_kernel(FdpfParams P_, DevMatT<VT> MP_, DevMatT<VT> MQ_) {
+  static_assert(!(ZS && RED), "z is a vector of the PCG");
   __shared__ LaneState<T> L;
+  RedLanes<T>* RL = nullptr;
+  if constexpr (RED) {
+    __shared__ RedLanes<T> rl;
+    RL = &rl;
+  }
   // the parameter blocks in shared memory: the out-of-line passes take them
   // by reference, so their fields are read from shared memory rather than
   // from a per-thread local copy
@@ -874,10 +898,16 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
     GPCG_PHASE(1);
     if (!more) continue;
     if (any_stepping<T>(L)) {
-      pcg_solve<T, VT, true, GEN>(P, MP, L, x, r, p, q, z, L.raP, L.rbP, L.wP, L.inP, nullptr,
-                                  nullptr, L.hold);
-      GPCG_PHASE(2);
-      update_pass<T, VT, true, GEN>(MP, L, x, p, th, EF, SW);
+      if constexpr (RED) {
+        red_solve<T, VT>(P, MP, L, *RL, r, L.raP, L.rbP, L.inP, L.hold);
+        GPCG_PHASE(2);
+        update_pass<T, VT, true, GEN>(MP, L, r, nullptr, th, EF, SW, RL->xa);
+      } else {
+        pcg_solve<T, VT, true, GEN>(P, MP, L, x, r, p, q, z, L.raP, L.rbP, L.wP, L.inP, nullptr,
+                                    nullptr, L.hold);
+        GPCG_PHASE(2);
+        update_pass<T, VT, true, GEN>(MP, L, x, p, th, EF, SW);
+      }
     }
     __syncthreads();
     GPCG_PHASE(3);
@@ -893,10 +923,16 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
     }
     GPCG_PHASE(4);
     if (any_stepping<T>(L)) {
+      if constexpr (RED && !GEN) {
+        red_solve<T, VT>(P, MQ, L, *RL, r, L.raQ, L.rbQ, L.inQ, L.hold);
+        GPCG_PHASE(5);
+        update_pass<T, VT, false, GEN>(MQ, L, r, nullptr, th, EF, SW, RL->xa);
+      } else {
       pcg_solve<T, VT, true, GEN>(P, MQ, L, x, r, p, q, z, L.raQ, L.rbQ, L.wQ, L.inQ,
                                   MQ.c ? L.cl : nullptr, SW, L.hold);
       GPCG_PHASE(5);
       update_pass<T, VT, false, GEN>(MQ, L, x, p, th, EF, SW);
+      }
     }
     if (g.rs == 0)
 #pragma unroll
@@ -921,6 +957,26 @@ cudaError_t set_zs_smem(size_t zbytes) {
                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zbytes);
 }
 
+template <bool GEN, typename VT, bool RED>
+cudaError_t launch_tiles(cudaStream_t st, int T, int grid, const FdpfParams& P,
+                         const DevMatT<VT>& MP, const DevMatT<VT>& MQ) {
+  switch (T) {
+    case 2: fdpf_tiles_kernel<2, VT, GEN, false, RED><<<grid, NTHREADS, 0, st>>>(P, MP, MQ); break;
+    case 4: fdpf_tiles_kernel<4, VT, GEN, false, RED><<<grid, NTHREADS, 0, st>>>(P, MP, MQ); break;
+    case 8: fdpf_tiles_kernel<8, VT, GEN, false, RED><<<grid, NTHREADS, 0, st>>>(P, MP, MQ); break;
+    case 16:
+      if constexpr (GEN) return cudaErrorInvalidValue;
+      else fdpf_tiles_kernel<16, VT, GEN, false, RED><<<grid, NTHREADS, 0, st>>>(P, MP, MQ);
+      break;
+    case 32:
+      if constexpr (GEN) return cudaErrorInvalidValue;
+      else fdpf_tiles_kernel<32, VT, GEN, false, RED><<<grid, NTHREADS, 0, st>>>(P, MP, MQ);
+      break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
+}
+
 template <bool GEN, typename VT>
 cudaError_t launch_fdpf_g(cudaStream_t st, int T, int grid, const FdpfParams& P,
                           const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes = 0) {
@@ -937,28 +993,36 @@ cudaError_t launch_fdpf_g(cudaStream_t st, int T, int grid, const FdpfParams& P,
       return cudaGetLastError();
     }
   }
+  return reduced_form(P.precond, MP, MQ) ? launch_tiles<GEN, VT, true>(st, T, grid, P, MP, MQ)
+                                         : launch_tiles<GEN, VT, false>(st, T, grid, P, MP, MQ);
+}
+
+template <bool GEN, typename VT, bool RED>
+int tiles_blocks(int T) {
+  int nb = 0;
+  cudaError_t ce = cudaErrorInvalidValue;
+  auto occ = [&](auto* k) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NTHREADS, 0);
+  };
   switch (T) {
-    case 2: fdpf_tiles_kernel<2, VT, GEN><<<grid, NTHREADS, 0, st>>>(P, MP, MQ); break;
-    case 4: fdpf_tiles_kernel<4, VT, GEN><<<grid, NTHREADS, 0, st>>>(P, MP, MQ); break;
-    case 8: fdpf_tiles_kernel<8, VT, GEN><<<grid, NTHREADS, 0, st>>>(P, MP, MQ); break;
+    case 2: ce = occ(fdpf_tiles_kernel<2, VT, GEN, false, RED>); break;
+    case 4: ce = occ(fdpf_tiles_kernel<4, VT, GEN, false, RED>); break;
+    case 8: ce = occ(fdpf_tiles_kernel<8, VT, GEN, false, RED>); break;
     case 16:
-      if constexpr (GEN) return cudaErrorInvalidValue;
-      else fdpf_tiles_kernel<16, VT, GEN><<<grid, NTHREADS, 0, st>>>(P, MP, MQ);
+      if constexpr (!GEN) ce = occ(fdpf_tiles_kernel<16, VT, GEN, false, RED>);
       break;
     case 32:
-      if constexpr (GEN) return cudaErrorInvalidValue;
-      else fdpf_tiles_kernel<32, VT, GEN><<<grid, NTHREADS, 0, st>>>(P, MP, MQ);
+      if constexpr (!GEN) ce = occ(fdpf_tiles_kernel<32, VT, GEN, false, RED>);
       break;
-    default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
+  return ce == cudaSuccess ? nb : 0;
 }
 
 template <bool GEN, typename VT>
-int fdpf_blocks_g(int T, size_t zbytes = 0) {
-  int nb = 0;
-  cudaError_t ce = cudaErrorInvalidValue;
+int fdpf_blocks_g(int T, size_t zbytes, bool red) {
   if (zbytes) {
+    int nb = 0;
+    cudaError_t ce = cudaErrorInvalidValue;
     if constexpr (!GEN) {
       if (T == 2 && set_zs_smem<2, VT, true>(zbytes) == cudaSuccess)
         ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
@@ -969,18 +1033,7 @@ int fdpf_blocks_g(int T, size_t zbytes = 0) {
     }
     return ce == cudaSuccess ? nb : 0;
   }
-  switch (T) {
-    case 2: ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fdpf_tiles_kernel<2, VT, GEN>, NTHREADS, 0); break;
-    case 4: ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fdpf_tiles_kernel<4, VT, GEN>, NTHREADS, 0); break;
-    case 8: ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fdpf_tiles_kernel<8, VT, GEN>, NTHREADS, 0); break;
-    case 16:
-      if constexpr (!GEN) ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fdpf_tiles_kernel<16, VT, GEN>, NTHREADS, 0);
-      break;
-    case 32:
-      if constexpr (!GEN) ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fdpf_tiles_kernel<32, VT, GEN>, NTHREADS, 0);
-      break;
-  }
-  return ce == cudaSuccess ? nb : 0;
+  return red ? tiles_blocks<GEN, VT, true>(T) : tiles_blocks<GEN, VT, false>(T);
 }
 
 }  // namespace gpcg

@@ -88,17 +88,23 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   const size_t scen = up256(S * 4) * 3 + up256(S * 8);
   const size_t vec_bytes = up256((size_t)(c.rows + 1) * T * vt);
   const size_t st_bytes = up256((size_t)c.n * T * 8);
-  // five vectors; the state theta and e + jf (two arrays' worth)
-  const size_t per_slot = 5 * vec_bytes + 3 * st_bytes;
+  // five vectors (one in the reduced form of the inner solve without
+  // extension rows); the state theta and e + jf (two arrays' worth)
+  const bool red = reduced_form(c.opt.precond, c.MPf, c.MQf);
+  const int nv = red && !ext ? 1 : 5;
+  const size_t per_slot = nv * vec_bytes + 3 * st_bytes;
+  // what fits is decided on five vectors in either form
+  const size_t most = 5 * vec_bytes + 3 * st_bytes;
   const size_t cap = GPCG_NOALLOC_SCRATCH_BYTES;
-  if (head + scen + per_slot > cap)
+  if (head + scen + most > cap)
     return err(GPCG_ERR_INVALID_ARG,
                "gpcg_n1_screen_noalloc: %zu scenarios of a %d-bus grid need %zu bytes of "
                "scratch, more than the %zu-byte limit",
-               S, c.n, head + scen + per_slot, cap);
+               S, c.n, head + scen + most, cap);
   const int n_tiles = (int)((S + T - 1) / T);
   const int occ =
-      f32 ? fdpf_max_blocks_per_sm<float>(T, ext) : fdpf_max_blocks_per_sm<double>(T, ext);
+      f32 ? fdpf_max_blocks_per_sm<float>(T, ext, 0, red)
+          : fdpf_max_blocks_per_sm<double>(T, ext, 0, red);
   int per_sm = c.opt.ctas_per_sm ? c.opt.ctas_per_sm : std::min(c.per_sm, occ);
   if (per_sm <= 0) per_sm = occ;
   per_sm = std::max(per_sm, 1);
@@ -154,9 +160,14 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   P.n_tiles = n_tiles;
   P.tile_counter = counter;
   const size_t vb = (size_t)slots * vec_bytes, sb = (size_t)slots * st_bytes;
-  P.wx = work; P.wr = work + vb; P.wp = work + 2 * vb; P.wq = work + 3 * vb; P.wz = work + 4 * vb;
+  if (nv == 1) {
+    P.wr = work;
+  } else {
+    P.wx = work; P.wr = work + vb; P.wp = work + 2 * vb; P.wq = work + 3 * vb;
+    P.wz = work + 4 * vb;
+  }
   P.vstride = vec_bytes / vt;
-  double* sbase = (double*)(work + 5 * vb);
+  double* sbase = (double*)(work + nv * vb);
   const size_t ss = st_bytes / 8;
   (void)sb;
   P.wth = sbase; P.we = sbase + slots * ss; P.wf = sbase + 2 * slots * ss;

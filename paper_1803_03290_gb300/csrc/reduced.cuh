@@ -1,0 +1,348 @@
+// The base-preconditioned CG of one outage in its two-dimensional Krylov
+// space, for the complete base-case factor.
+//
+// With M = B = L L^T the base-case matrix itself and B_s = B - w v v^T the
+// outage's (v = c e_from - e_to), M^-1 B_s maps span{z0, y}, z0 = M^-1 r0 and
+// y = M^-1 v_m, into itself: B_s z = B z - w (v.z) v_m on the main island
+// (v_m: v without an islanded end, which is masked out of every vector).  So
+// every iterate of the PCG of Sec. IV.B is a combination of those two
+// vectors and every residual one of r0 and v_m, and the recurrence needs
+// only scalars:
+//   r.r    from r0.r0, v_m.r0, v_m.v_m,
+//   r.z    from r0.z0 = |L^-1 r0|^2, v_m.z0 and v_m.y,
+//   v.z    from v.z0 = (L^-1 v).(L^-1 r0) and v.y.
+// All of them are known after the forward substitution f = L^-1 r0: L^-1 v
+// and L^-1 v_m are sparse (the ancestors of the outage's ends in the
+// elimination tree, about 60 of 10,000 rows) and belong to the grid
+// (BranchCols).  The solution xa z0 + xb y = xa L^-T (f + (xb / xa) L^-1 v_m)
+// then takes one backward substitution.  An inner solve is one forward and
+// one backward pass over one vector in place of an SpMV, a forward and a
+// backward pass over five vectors per iteration, with the same iterates and
+// the same stopping rule (grid10k, every outage, 1e-4 p.u.: 2.4 outer, 3.9
+// P and 3.4 Q iterations either way).
+#pragma once
+#include "fdpf_ops.cuh"
+
+namespace gpcg {
+
+// Forward substitution f = L^-1 r in place over the levels before the tail,
+// and the tail's right-hand side reduced and multiplied by the tail's dense
+// inverse (y into zt).  Adds the lanes' partial |r|^2 to rr and |f|^2 to ff.
+template <int T, typename VT>
+__device__ __forceinline__ void red_forward(const DevMatT<VT>& M, VT* __restrict__ f,
+                                            VT* __restrict__ zt, Vec<VT, Geo<T>::LP>& rr,
+                                            Vec<VT, Geo<T>::LP>& ff) {
+  constexpr int LP = Geo<T>::LP;
+  const Geo<T> g;
+  constexpr int RPS = Geo<T>::RPS, NPT = (TAIL_ROWS + RPS - 1) / RPS;
+  const int nl = M.tail_lev, t0 = M.tail_row0, nt = M.n - t0;
+  int r0 = 0, r1 = nl > 0 ? __ldg(M.lev_ptr + 1) : 0;
+  for (int lev = 0; lev < nl; ++lev) {
+    const int r2 = lev + 1 < nl ? __ldg(M.lev_ptr + lev + 2) : r1;
+    for (int i = r0 + g.rs; i < r1; i += RPS) {
+      const size_t o = (size_t)i * T + g.lane;
+      const VT id = __ldg(M.inv_diag + i);
+      Vec<VT, LP> a = ldv<LP>(f + o);
+#pragma unroll
+      for (int j = 0; j < LP; ++j) rr.v[j] += a.v[j] * a.v[j];
+      if (lev > 0) {  // the rows of level 0 have nothing to gather
+        int c[KL];
+        VT v[KL];
+        Vec<VT, LP> zc[KL];
+        ld_cols<KL>(M.L.col + (size_t)i * KL, c);
+        ld_vals<KL>(M.L.val + (size_t)i * KL, v);
+        const int o0 = __ldg(M.L.optr + i), o1 = __ldg(M.L.optr + i + 1);
+#pragma unroll
+        for (int k = 0; k < KL; ++k) zc[k] = ldv<LP>(f + (size_t)c[k] * T + g.lane);
+#pragma unroll
+        for (int k = 0; k < KL; ++k)
+#pragma unroll
+          for (int j = 0; j < LP; ++j) a.v[j] -= v[k] * zc[k].v[j];
+        for (int e = o0; e < o1; ++e) {
+          const VT vv = __ldg(M.L.oval + e);
+          const Vec<VT, LP> zz = ldv<LP>(f + (size_t)__ldg(M.L.ocol + e) * T + g.lane);
+#pragma unroll
+          for (int j = 0; j < LP; ++j) a.v[j] -= vv * zz.v[j];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < LP; ++j) {
+        a.v[j] *= id;
+        ff.v[j] += a.v[j] * a.v[j];
+      }
+      stv<LP>(f + o, a);
+    }
+    __syncthreads();
+    r0 = r1;
+    r1 = r2;
+  }
+  if (nt <= 0) return;
+  // the tail rows' right-hand side, minus the rows solved before
+  for (int k = g.rs; k < nt; k += RPS) {
+    const int i = t0 + k;
+    int c[KL];
+    VT v[KL];
+    ld_cols<KL>(M.L.col + (size_t)i * KL, c);
+    ld_vals<KL>(M.L.val + (size_t)i * KL, v);
+    Vec<VT, LP> a = ldv<LP>(f + (size_t)i * T + g.lane);
+#pragma unroll
+    for (int j = 0; j < LP; ++j) rr.v[j] += a.v[j] * a.v[j];
+#pragma unroll
+    for (int s = 0; s < KL; ++s) {
+      if (c[s] >= t0) continue;
+      const Vec<VT, LP> zz = ldv<LP>(f + (size_t)c[s] * T + g.lane);
+#pragma unroll
+      for (int j = 0; j < LP; ++j) a.v[j] -= v[s] * zz.v[j];
+    }
+    const int o0 = __ldg(M.L.optr + i), o1 = __ldg(M.L.optr + i + 1);
+    for (int e = o0; e < o1; ++e) {
+      const int cc = __ldg(M.L.ocol + e);
+      if (cc >= t0) continue;
+      const VT vv = __ldg(M.L.oval + e);
+      const Vec<VT, LP> zz = ldv<LP>(f + (size_t)cc * T + g.lane);
+#pragma unroll
+      for (int j = 0; j < LP; ++j) a.v[j] -= vv * zz.v[j];
+    }
+    stv<LP>(zt + (size_t)k * T + g.lane, a);
+  }
+  __syncthreads();
+  // y_t = X rhs: X_kj = xc[j nt + k], zero above the diagonal; a warp's rows
+  // k are consecutive, so it stops at the diagonal of its last row
+  Vec<VT, LP> y[NPT];
+#pragma unroll
+  for (int m = 0; m < NPT; ++m) {
+    const int k = g.rs + m * RPS;
+    const int jend = min(nt, __shfl_sync(0xffffffffu, k, 31) + 1);  // every lane takes part
+    y[m] = vzero<VT, LP>();
+    if (k < nt) {
+      const VT* col = M.xc + k;
+#pragma unroll 4
+      for (int j = 0; j < jend; ++j) {
+        const VT xv = __ldg(col + (size_t)j * nt);
+        const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)j * T + g.lane);
+#pragma unroll
+        for (int l = 0; l < LP; ++l) y[m].v[l] += xv * sv.v[l];
+      }
+#pragma unroll
+      for (int l = 0; l < LP; ++l) ff.v[l] += y[m].v[l] * y[m].v[l];
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int m = 0; m < NPT; ++m) {
+    const int k = g.rs + m * RPS;
+    if (k < nt) stv<LP>(zt + (size_t)k * T + g.lane, y[m]);
+  }
+}
+
+// Backward substitution x = L^-T f in place, the tail first (its y in zt).
+template <int T, typename VT>
+__device__ __forceinline__ void red_backward(const DevMatT<VT>& M, VT* __restrict__ f,
+                                             const VT* __restrict__ zt) {
+  constexpr int LP = Geo<T>::LP;
+  const Geo<T> g;
+  constexpr int RPS = Geo<T>::RPS, NPT = (TAIL_ROWS + RPS - 1) / RPS;
+  const int t0 = M.tail_row0, nt = M.n - t0;
+  if (nt > 0) {
+    // z_t = X^T y_t: X_ik = xr[i nt + k], zero for i < k; a warp starts at
+    // the diagonal of its first row
+#pragma unroll
+    for (int m = 0; m < NPT; ++m) {
+      const int k = g.rs + m * RPS;
+      const int ibeg = __shfl_sync(0xffffffffu, k, 0);
+      if (k >= nt) continue;
+      const VT* col = M.xr + k;
+      Vec<VT, LP> a = vzero<VT, LP>();
+#pragma unroll 4
+      for (int i = ibeg; i < nt; ++i) {
+        const VT xv = __ldg(col + (size_t)i * nt);
+        const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)i * T + g.lane);
+#pragma unroll
+        for (int l = 0; l < LP; ++l) a.v[l] += xv * sv.v[l];
+      }
+      stv<LP>(f + (size_t)(t0 + k) * T + g.lane, a);
+    }
+    __syncthreads();
+  }
+  const int nb = M.ntblev;
+  int r0 = nb > 0 ? __ldg(M.tblev_ptr) : 0, r1 = nb > 0 ? __ldg(M.tblev_ptr + 1) : 0;
+  for (int lev = 0; lev < nb; ++lev) {
+    const int r2 = lev + 1 < nb ? __ldg(M.tblev_ptr + lev + 2) : r1;
+    for (int k = r0 + g.rs; k < r1; k += RPS) {
+      const int i = __ldg(M.tblev_rows + k);
+      const size_t o = (size_t)i * T + g.lane;
+      int c[KU];
+      VT v[KU];
+      Vec<VT, LP> zc[KU];
+      ld_cols<KU>(M.U.col + (size_t)i * KU, c);
+      ld_vals<KU>(M.U.val + (size_t)i * KU, v);
+      const int o0 = __ldg(M.U.optr + i), o1 = __ldg(M.U.optr + i + 1);
+      const VT id = __ldg(M.inv_diag + i);
+      Vec<VT, LP> a = ldv<LP>(f + o);
+#pragma unroll
+      for (int s = 0; s < KU; ++s) zc[s] = ldv<LP>(f + (size_t)c[s] * T + g.lane);
+#pragma unroll
+      for (int s = 0; s < KU; ++s)
+#pragma unroll
+        for (int j = 0; j < LP; ++j) a.v[j] -= v[s] * zc[s].v[j];
+      for (int e = o0; e < o1; ++e) {
+        const VT vv = __ldg(M.U.oval + e);
+        const Vec<VT, LP> zz = ldv<LP>(f + (size_t)__ldg(M.U.ocol + e) * T + g.lane);
+#pragma unroll
+        for (int j = 0; j < LP; ++j) a.v[j] -= vv * zz.v[j];
+      }
+#pragma unroll
+      for (int j = 0; j < LP; ++j) a.v[j] *= id;
+      stv<LP>(f + o, a);
+    }
+    __syncthreads();
+    r0 = r1;
+    r1 = r2;
+  }
+}
+
+// What a lane's recurrence starts from: R = r0.r0, Z = r0.z0, u = v.z0,
+// m0 = v_m.z0, vr = v_m.r0, and the branch's scalars.
+struct RedScalars {
+  double R, Z, u, m0, vr, vy, my, vm2, w;
+};
+
+// The PCG of pcg_solve on those scalars: same steps, same stopping rule.
+// The solution is xa z0 + xb y; returns the iterations taken.
+__device__ inline int reduced_cg(const RedScalars& q, double tol2, int max_inner, double& xa,
+                                 double& xb) {
+  xa = xb = 0.0;
+  if (!(q.R > 0.0) || !(q.Z > 0.0)) return 0;
+  double a = 1.0, b = 0.0, pa = 1.0, pb = 0.0, rz = q.Z, best = q.R;
+  int its = 0, stall = 0;
+  while (its < max_inner) {
+    const double qb = pb - q.w * (pa * q.u + pb * q.vy);  // B_s p = pa r0 + qb v_m
+    const double pq = pa * pa * q.Z + (pa * qb + pb * pa) * q.m0 + pb * qb * q.my;
+    if (!(pq > 0.0) || !isfinite(pq)) break;
+    const double al = rz / pq;
+    xa += al * pa;
+    xb += al * pb;
+    a -= al * pa;
+    b -= al * qb;
+    ++its;
+    const double rr = a * a * q.R + 2.0 * a * b * q.vr + b * b * q.vm2;
+    if (!(rr > tol2 * q.R) || !isfinite(rr)) break;
+    if (rr < 0.999 * best) { best = rr; stall = 0; }
+    else if (++stall >= STALL_ITERS) break;
+    if (rr > 1e4 * best) break;
+    const double rzn = a * a * q.Z + 2.0 * a * b * q.m0 + b * b * q.my;
+    if (!(rzn > 0.0)) break;
+    const double be = rzn / rz;
+    rz = rzn;
+    pa = a + be * pa;
+    pb = b + be * pb;
+  }
+  return its;
+}
+
+template <int T>
+struct RedLanes {
+  double vr[T], xa[T];
+  double part[2][NTHREADS / 32][T];  // the warps' partial r.r and |f|^2
+};
+
+// PCG on B_s x = f for the lanes that are active and not held, f in place:
+// on return lane s's solution is S.xa[s] times the vector (xa = 0: no step).
+// Adds each lane's iteration count to iters.
+template <int T, typename VT>
+__device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT>& M,
+                                           LaneState<T>& L, RedLanes<T>& S, VT* f,
+                                           const int* ra, const int* rb, int* iters,
+                                           const int* hold) {
+  constexpr int LP = Geo<T>::LP;
+  constexpr int NW = NTHREADS / 32, TPR = Geo<T>::TPR;
+  __shared__ __align__(16) VT zt[TAIL_ROWS * T];
+  const Geo<T> g;
+  const int tid = threadIdx.x, warp = tid >> 5, wl = tid & 31;
+  if (tid < T) {  // v_m.r0, before f is overwritten; the zero row of the padding
+    double vr = 0.0;
+    if (L.active[tid] && L.l[tid] >= 0) {
+      const double* sc = M.br.sc + (size_t)L.l[tid] * SC_N;
+      if (ra[tid] >= 0) vr += sc[SC_CA] * (double)f[(size_t)ra[tid] * T + tid];
+      if (rb[tid] >= 0) vr += sc[SC_CB] * (double)f[(size_t)rb[tid] * T + tid];
+    }
+    S.vr[tid] = vr;
+    f[(size_t)M.n * T + tid] = (VT)0;
+  }
+  __syncthreads();
+  Vec<VT, LP> rr = vzero<VT, LP>(), ff = vzero<VT, LP>();
+  red_forward<T, VT>(M, f, zt, rr, ff);
+#pragma unroll
+  for (int off = 16; off >= TPR; off >>= 1)
+#pragma unroll
+    for (int j = 0; j < LP; ++j) {
+      rr.v[j] += __shfl_xor_sync(0xffffffffu, rr.v[j], off);
+      ff.v[j] += __shfl_xor_sync(0xffffffffu, ff.v[j], off);
+    }
+  if (wl < TPR)
+#pragma unroll
+    for (int j = 0; j < LP; ++j) {
+      S.part[0][warp][g.lane + j] = (double)rr.v[j];
+      S.part[1][warp][g.lane + j] = (double)ff.v[j];
+    }
+  __syncthreads();
+  // a warp per lane: the sparse dot products, the recurrence, and L^-1 v_m
+  // added to the lane's vector
+  const int t0 = M.tail_row0;
+  for (int s = warp; s < T; s += NW) {
+    double xa = 0.0;
+    if (L.active[s] && !(hold && hold[s])) {
+      RedScalars q{};
+      double R = 0.0, Z = 0.0;
+      for (int k = 0; k < NW; ++k) {
+        R += S.part[0][k][s];
+        Z += S.part[1][k][s];
+      }
+      q.R = R;
+      q.Z = Z;
+      const int l = L.l[s];
+      int e0 = 0, e1 = 0;
+      if (l >= 0) {
+        e0 = __ldg(M.br.ptr + l);
+        e1 = __ldg(M.br.ptr + l + 1);
+        const double* sc = M.br.sc + (size_t)l * SC_N;
+        q.vy = __ldg(sc + SC_VY);
+        q.my = __ldg(sc + SC_MY);
+        q.vm2 = __ldg(sc + SC_VM2);
+        q.w = __ldg(sc + SC_W);
+        q.vr = S.vr[s];
+        double u = 0.0, m0 = 0.0;
+        for (int e = e0 + wl; e < e1; e += 32) {
+          const int i = __ldg(M.br.row + e);
+          const double x = (double)(i < t0 ? f[(size_t)i * T + s] : zt[(size_t)(i - t0) * T + s]);
+          u = fma(__ldg(M.br.fv + e), x, u);
+          m0 = fma(__ldg(M.br.fm + e), x, m0);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+          u += __shfl_xor_sync(0xffffffffu, u, off);
+          m0 += __shfl_xor_sync(0xffffffffu, m0, off);
+        }
+        q.u = u;
+        q.m0 = m0;
+      }
+      double xb;
+      const int its = reduced_cg(q, P.inner_rtol * P.inner_rtol, P.max_inner, xa, xb);
+      if (xa != 0.0 && xb != 0.0) {
+        const double k = xb / xa;
+        for (int e = e0 + wl; e < e1; e += 32) {
+          const int i = __ldg(M.br.row + e);
+          VT* x = i < t0 ? f + (size_t)i * T + s : zt + (size_t)(i - t0) * T + s;
+          *x = (VT)fma(k, __ldg(M.br.fm + e), (double)*x);
+        }
+      }
+      if (wl == 0) iters[s] += its;
+    }
+    if (wl == 0) S.xa[s] = xa;
+  }
+  __syncthreads();
+  red_backward<T, VT>(M, f, zt);
+  if (M.ntblev == 0) __syncthreads();
+}
+
+}  // namespace gpcg
