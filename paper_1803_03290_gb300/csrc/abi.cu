@@ -25,8 +25,7 @@ namespace gpcg {
 void launch_branch_params(cudaStream_t, int, const double*, const double*, double*, double*,
                           double*, double*);
 void launch_ybus_diag(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
-                      const double*, const double*, const double*, const double*, double*,
-                      double*);
+                      const double*, const double*, const double*, const double*, double2*);
 void launch_laplacian_values(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
                              const int32_t*, const int32_t*, const double*, const int32_t*,
                              const double*, const int32_t*, const int32_t*, double*, int32_t*);
@@ -44,13 +43,15 @@ void launch_inv_diag(cudaStream_t, int, const int32_t*, const double*, double*, 
 void launch_tail_inverse(cudaStream_t, int, int, const int32_t*, const int32_t*, const double*,
                          const double*, double*, double*, float*, float*);
 void launch_adj_values(cudaStream_t, int, const int32_t*, const double*, const double*,
-                       const double*, double*, double*);
+                       const double*, double2*, double*, double*);
 void launch_branch_count(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
                          const int32_t*, int32_t*);
 void launch_branch_cols(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
                         const int32_t*, const Ell<double>&, int, const double*, const double*,
                         const double*, const int32_t*, const int32_t*, const int32_t*,
                         const int32_t*, int32_t*, double*, double*, double*);
+void launch_flow_values(cudaStream_t, int, const double*, const double*, const double*, double2*);
+void launch_gather_pair(cudaStream_t, int, const int4*, const double2*, double2*);
 void launch_ext_rows(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
                      const int32_t*, const double*, const double*, const int32_t*, int32_t*,
                      double*, float*, double*, float*);
@@ -217,7 +218,9 @@ struct gpcg_ctx {
   double* d_prefP = nullptr;   // [n + 1] prefix sums of a caller's injections
   int n_adj_slots = 0, n_adj_over = 0;
   std::vector<int32_t> deg;
-  int32_t *mis_order = nullptr, *misq_order = nullptr;
+  std::vector<double2> pq;  // (P_sched, Q_sched), internal numbering
+  BusTab tabP, tabQ;
+  double2* ef0 = nullptr;
   int32_t* d_bus_of_user = nullptr;  // caller's bus -> internal bus
   unsigned long long* phase = nullptr;  // diagnostics: [8 + 2 phase_cap]
   size_t phase_cap = 0;
@@ -612,17 +615,51 @@ static gpcg_status build_matrices(gpcg_ctx* c) {
     CUDA_TRY(cudaDeviceSynchronize());
   }
   {
-    const MatrixPlan& Q = c->MQ.plan;
-    std::vector<int32_t> order(Q.n);
-    for (int k = 0; k < Q.n; ++k) order[k] = k;
-    std::sort(order.begin(), order.end(),
-              [&](int a, int b) { return Q.bus_of_row[a] < Q.bus_of_row[b]; });
-    for (size_t w0 = 0; w0 < order.size(); w0 += 128)
-      std::stable_sort(order.begin() + w0, order.begin() + std::min(order.size(), w0 + 128),
-                       [&](int a, int b) {
-                         return c->deg[Q.bus_of_row[a]] > c->deg[Q.bus_of_row[b]];
-                       });
-    CUDA_TRY(upload(c->mat_owned, &c->misq_order, order.data(), order.size()));
+    // the half-steps' bus tables
+    auto& own = c->mat_owned;
+    for (int which = 0; which < 2; ++which) {
+      const MatrixPlan& P = which ? c->MQ.plan : c->MP.plan;
+      const int n = P.n;
+      std::vector<int32_t> order;
+      for (int b = 0; b < c->n; ++b)
+        if (P.row_of_bus[b] >= 0) order.push_back(b);
+      for (size_t w0 = 0; w0 < order.size(); w0 += MD_WINDOW)
+        std::stable_sort(order.begin() + w0, order.begin() + std::min(order.size(), w0 + MD_WINDOW),
+                         [&](int a, int b) {
+                           return c->deg[a] != c->deg[b] ? c->deg[a] > c->deg[b]
+                                                         : c->bus_type[a] < c->bus_type[b];
+                         });
+      std::vector<int4> md(n);
+      std::vector<int32_t> nbr((size_t)n * KG), br((size_t)n * KG);
+      std::vector<double2> pq(n);
+      for (int k = 0; k < n; ++k) {
+        const int b = order[k], a0 = c->bg.adj.ptr[b], deg = c->bg.adj.ptr[b + 1] - a0;
+        md[k] = make_int4(b, c->pre[b],
+                          std::min(deg, KG) | (c->bus_type[b] << MD_TYPE_SHIFT) |
+                              (deg > KG ? MD_OVER : 0),
+                          P.row_of_bus[b]);
+        for (int a = 0; a < KG; ++a) {
+          nbr[(size_t)a * n + k] = a < deg ? c->bg.adj.idx[a0 + a] : b;
+          br[(size_t)a * n + k] = a < deg ? c->bg.adj_branch[a0 + a] : -2;
+        }
+        pq[k] = c->pq[b];
+      }
+      BusTab& tab = which ? c->tabQ : c->tabP;
+      int4* d_md;
+      int32_t *d_nbr, *d_br;
+      double2 *d_gb, *d_yd, *d_pq;
+      CUDA_TRY(upload(own, &d_md, md.data(), md.size()));
+      CUDA_TRY(upload(own, &d_nbr, nbr.data(), nbr.size()));
+      CUDA_TRY(upload(own, &d_br, br.data(), br.size()));
+      CUDA_TRY(upload(own, &d_pq, pq.data(), pq.size()));
+      CUDA_TRY(dalloc(own, &d_gb, nbr.size()));
+      CUDA_TRY(dalloc(own, &d_yd, (size_t)n));
+      launch_adj_values(0, (int)br.size(), d_br, c->G.cf, c->G.g, c->G.by, d_gb, nullptr, nullptr);
+      launch_gather_pair(0, n, d_md, c->G.ydiag, d_yd);
+      CUDA_TRY(cudaGetLastError());
+      tab = BusTab{d_md, d_nbr, d_gb, d_yd, d_pq, n};
+    }
+    CUDA_TRY(cudaDeviceSynchronize());
   }
   c->planned_precond = c->opt.precond;
   return GPCG_OK;
@@ -885,30 +922,23 @@ extern "C" gpcg_status gpcg_create(const gpcg_grid* g, const gpcg_options* opt, 
     UP(G.adj_optr, E.optr.data(), E.optr.size());
     UP(G.adj_onbr, E.ocol.data(), E.ocol.size());
     UP(G.adj_obr, E.osrc.data(), E.osrc.size());
-    AL(G.adj_g, pad_nbr.size());
-    AL(G.adj_b, pad_nbr.size());
+    AL(G.adj_gb, pad_nbr.size());
     AL(G.adj_og, E.ocol.size());
     AL(G.adj_ob, E.ocol.size());
     c->n_adj_slots = (int)pad_nbr.size();
     c->n_adj_over = (int)E.ocol.size();
-    std::vector<int32_t> deg(n), order;
+    std::vector<int32_t> deg(n);
     for (int b = 0; b < n; ++b) deg[b] = std::min(c->bg.adj.ptr[b + 1] - c->bg.adj.ptr[b], KG);
-    for (int b = 0; b < n; ++b)
-      if (b != slack) order.push_back(b);
-    // bus order (neighbours close), degree-sorted inside windows of 128 rows
-    // so the threads of a warp mostly run neighbour loops of equal length
-    for (size_t w0 = 0; w0 < order.size(); w0 += 128)
-      std::stable_sort(order.begin() + w0, order.begin() + std::min(order.size(), w0 + 128),
-                       [&](int a, int b) { return deg[a] > deg[b]; });
     UP(G.adj_deg, deg.data(), n);
-    UP(c->mis_order, order.data(), order.size());
     c->deg = deg;
   }
   UP(G.sub, c->sub.data(), n);
   AL(G.g, m);
   AL(G.by, m);
-  AL(G.Gii, n);
-  AL(G.Bii, n);
+  AL(G.ybr, (size_t)2 * m);
+  AL(G.ydiag, n);
+  c->pq.resize(n);
+  for (int k = 0; k < n; ++k) c->pq[k] = make_double2(P_i[k], Q_i[k]);
   AL(c->wP, m);
   AL(c->wQ, m);
   AL(c->th0, n);
@@ -916,6 +946,7 @@ extern "C" gpcg_status gpcg_create(const gpcg_grid* g, const gpcg_options* opt, 
   AL(c->flow0, m);
   AL(c->c0, n);
   AL(c->s0, n);
+  AL(c->ef0, n);
   AL(c->d_counter, 1);
   AL(c->d_err, 1);
   AL(c->r0P, n);
@@ -935,9 +966,12 @@ extern "C" gpcg_status gpcg_create(const gpcg_grid* g, const gpcg_options* opt, 
 #undef UP
 #undef AL
   launch_branch_params(0, m, G.r, G.x, G.g, G.by, c->wP, c->wQ);
-  launch_ybus_diag(0, n, G.adj_ptr, G.adj_br, G.f, G.cf, G.g, G.by, G.b_sh, G.Gii, G.Bii);
-  launch_adj_values(0, c->n_adj_slots, G.adj_brl, G.cf, G.g, G.by, G.adj_g, G.adj_b);
-  launch_adj_values(0, c->n_adj_over, G.adj_obr, G.cf, G.g, G.by, G.adj_og, G.adj_ob);
+  launch_ybus_diag(0, n, G.adj_ptr, G.adj_br, G.f, G.cf, G.g, G.by, G.b_sh, G.ydiag);
+  launch_flow_values(0, m, G.cf, G.g, G.by, G.ybr);
+  launch_adj_values(0, c->n_adj_slots, G.adj_brl, G.cf, G.g, G.by, G.adj_gb, nullptr,
+                    nullptr);
+  launch_adj_values(0, c->n_adj_over, G.adj_obr, G.cf, G.g, G.by, nullptr, G.adj_og,
+                    G.adj_ob);
   if ((ce = cudaGetLastError()) != cudaSuccess) return fail_cuda(ce, "build kernels");
   st = build_matrices(c);
   if (st != GPCG_OK) {
@@ -1130,8 +1164,8 @@ static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, i
 static FdpfParams base_params(gpcg_ctx* c) {
   FdpfParams P;
   P.G = c->G;
-  P.mis_order = c->mis_order;
-  P.misq_order = c->misq_order;
+  P.tabP = c->tabP;
+  P.tabQ = c->tabQ;
   P.phase_cycles = c->phase_on ? c->phase : nullptr;
   P.tol = c->opt.tol;
   P.inner_rtol = c->opt.inner_rtol;
@@ -1195,7 +1229,7 @@ extern "C" gpcg_status gpcg_base_solve(gpcg_ctx* c, double* theta, double* vm, d
     return fail(GPCG_ERR_BASE_NOT_CONVERGED,
                 "base case did not converge (status %d after %d outer iterations)", hs, hit[0]);
   }
-  CUDA_TRY(launch_base_trig(0, c->n, c->th0, c->c0, c->s0));
+  CUDA_TRY(launch_base_trig(0, c->n, c->th0, c->V0, c->c0, c->s0, c->ef0));
   CUDA_TRY(launch_base_residual(0, c->G, c->V0, c->c0, c->s0, c->r0P, c->r0Q));
   CUDA_TRY(cudaDeviceSynchronize());
   c->base_flow.resize(c->m);
@@ -1374,6 +1408,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
   P.V0 = c->V0;
   P.c0 = c->c0;
   P.s0 = c->s0;
+  P.ef0 = c->ef0;
   P.out_theta = d_theta; P.out_vm = d_vm; P.out_flow = d_flow; P.out_maxload = d_ml;
   P.out_bus_map = c->d_bus_of_user;
   P.out_iters = d_iters; P.out_status = d_stat;
@@ -1462,7 +1497,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
           if (r != GPCG_OK) return r;
           FdpfParams Q = base_params(c);
           Q.sc = P.sc;
-          Q.th0 = P.th0; Q.V0 = P.V0; Q.c0 = P.c0; Q.s0 = P.s0;
+          Q.th0 = P.th0; Q.V0 = P.V0; Q.c0 = P.c0; Q.s0 = P.s0; Q.ef0 = P.ef0;
           // untimed: the first launch of a kernel variant, one tile of the
           // probe's lightest scenarios (the end of the scheduling order)
           const int nq = timed ? np : std::min(np, t);
@@ -2166,9 +2201,10 @@ bool ctx_view(const gpcg_ctx* c, CtxView* v) {
   v->V0 = c->V0;
   v->c0 = c->c0;
   v->s0 = c->s0;
-  v->mis_order = c->mis_order;
+  v->tabP = c->tabP;
+  v->tabQ = c->tabQ;
+  v->ef0 = c->ef0;
   v->bus_of_user = c->d_bus_of_user;
-  v->misq_order = c->misq_order;
   v->opt = c->opt;
   v->num_sms = c->num_sms;
   v->n = c->n;

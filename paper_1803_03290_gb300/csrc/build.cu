@@ -28,7 +28,7 @@ __global__ void ybus_diag_kernel(int n, const int32_t* __restrict__ adj_ptr,
                                  const int32_t* __restrict__ adj_br,
                                  const int32_t* __restrict__ from, const double* __restrict__ cf,
                                  const double* __restrict__ g, const double* __restrict__ by,
-                                 const double* __restrict__ b_sh, double* Gii, double* Bii) {
+                                 const double* __restrict__ b_sh, double2* ydiag) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double G = 0.0, B = 0.0;
@@ -38,8 +38,7 @@ __global__ void ybus_diag_kernel(int n, const int32_t* __restrict__ adj_ptr,
     G += c2 * g[e];
     B += c2 * (by[e] + 0.5 * b_sh[e]);
   }
-  Gii[i] = G;
-  Bii[i] = B;
+  ydiag[i] = make_double2(G, B);
 }
 
 // Values of a grounded sum of branch terms w v v^T, v = c e_from - e_to
@@ -216,10 +215,10 @@ void launch_branch_params(cudaStream_t st, int m, const double* r, const double*
 }
 void launch_ybus_diag(cudaStream_t st, int n, const int32_t* adj_ptr, const int32_t* adj_br,
                       const int32_t* from, const double* cf, const double* g, const double* by,
-                      const double* b_sh, double* Gii, double* Bii) {
+                      const double* b_sh, double2* ydiag) {
   if (n)
     ybus_diag_kernel<<<nblk(n, 256), 256, 0, st>>>(n, adj_ptr, adj_br, from, cf, g, by, b_sh,
-                                                   Gii, Bii);
+                                                   ydiag);
 }
 void launch_laplacian_values(cudaStream_t st, int nrows, const int32_t* bus_of_row,
                              const int32_t* row_of_bus, const int32_t* adj_ptr,
@@ -279,17 +278,48 @@ __global__ void inv_diag_kernel(int n, const int32_t* __restrict__ pos,
   inv32[i] = (float)d;
 }
 
-// Per-slot branch admittance of the mismatch adjacency (0 on padding).
+// Per-slot branch admittance of the mismatch adjacency (0 on padding), as
+// pairs (gb) or in two arrays.
 __global__ void adj_values_kernel(int n, const int32_t* __restrict__ br,
                                   const double* __restrict__ cf,
                                   const double* __restrict__ g, const double* __restrict__ by,
-                                  double* ag, double* ab) {
+                                  double2* gb, double* ag, double* ab) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const int e = br[k];
   // Y_ij = -c y for either end (c = 1 / turns ratio)
-  ag[k] = e >= 0 ? cf[e] * g[e] : 0.0;
-  ab[k] = e >= 0 ? cf[e] * by[e] : 0.0;
+  const double yg = e >= 0 ? cf[e] * g[e] : 0.0, yb = e >= 0 ? cf[e] * by[e] : 0.0;
+  if (gb) {
+    gb[k] = make_double2(yg, yb);
+  } else {
+    ag[k] = yg;
+    ab[k] = yb;
+  }
+}
+
+// The admittances the branch flows take (DevGrid::ybr).
+__global__ void flow_values_kernel(int m, const double* __restrict__ cf,
+                                   const double* __restrict__ g, const double* __restrict__ by,
+                                   double2* ybr) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= m) return;
+  const double c = cf[k];
+  ybr[2 * (size_t)k] = make_double2(g[k] * c * c, g[k] * c);
+  ybr[2 * (size_t)k + 1] = make_double2(by[k] * c, g[k]);
+}
+void launch_flow_values(cudaStream_t st, int m, const double* cf, const double* g,
+                        const double* by, double2* ybr) {
+  if (m > 0) flow_values_kernel<<<(m + 255) / 256, 256, 0, st>>>(m, cf, g, by, ybr);
+}
+
+__global__ void gather_pair_kernel(int n, const int4* __restrict__ md,
+                                   const double2* __restrict__ src, double2* dst) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) dst[k] = src[md[k].x];
+}
+void launch_gather_pair(cudaStream_t st, int n, const int4* md, const double2* src,
+                        double2* dst) {
+  if (n > 0) gather_pair_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, md, src, dst);
 }
 
 void launch_gather_val(cudaStream_t st, int n, const int32_t* src, const double* csr, double* dst,
@@ -346,8 +376,8 @@ void launch_tail_inverse(cudaStream_t st, int t0, int nt, const int32_t* l_ptr,
 }
 
 void launch_adj_values(cudaStream_t st, int n, const int32_t* br, const double* cf,
-                       const double* g, const double* by, double* ag, double* ab) {
-  if (n > 0) adj_values_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, br, cf, g, by, ag, ab);
+                       const double* g, const double* by, double2* gb, double* ag, double* ab) {
+  if (n > 0) adj_values_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, br, cf, g, by, gb, ag, ab);
 }
 
 }  // namespace gpcg

@@ -37,15 +37,16 @@ struct DevGrid {
   double* cf = nullptr;                      // 1 / turns ratio at the from end (1: a line)
   double *qmin = nullptr, *qmax = nullptr;   // PV generators' reactive limits (null: none)
   double *g = nullptr, *by = nullptr;        // series admittance g + j b_y
+  double2* ybr = nullptr;                    // per branch (c^2 g, c g), (c b_y, g), c = cf
   int32_t *adj_ptr = nullptr, *adj_idx = nullptr, *adj_br = nullptr;  // CSR adjacency
-  double *Gii = nullptr, *Bii = nullptr;     // bus admittance diagonal
+  double2* ydiag = nullptr;                  // bus admittance diagonal (G_ii, B_ii)
   int32_t *pre = nullptr, *sub = nullptr;    // depth-first preorder, subtree size
   int32_t* user_of_bus = nullptr;            // internal bus index -> caller's index
-  // padded adjacency for the mismatch: neighbour, branch, -g, -b_y per slot,
+  // padded adjacency for the mismatch: neighbour, branch, (c g, c b_y) per slot,
   // slot-major (slot a of bus i at a * n + i: a warp taking consecutive buses
   // reads consecutive entries)
   int32_t *adj_nbr = nullptr, *adj_brl = nullptr, *adj_deg = nullptr;  // deg = used slots
-  double *adj_g = nullptr, *adj_b = nullptr;
+  double2* adj_gb = nullptr;
   int32_t *adj_optr = nullptr, *adj_onbr = nullptr, *adj_obr = nullptr;
   double *adj_og = nullptr, *adj_ob = nullptr;
 };

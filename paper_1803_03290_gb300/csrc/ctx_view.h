@@ -3,6 +3,7 @@
 #pragma once
 #include "../../include/gpcg.h"
 #include "common.cuh"
+#include "fdpf.h"
 
 namespace gpcg {
 
@@ -11,7 +12,8 @@ struct CtxView {
   DevMatT<float> MPf, MQf;
   DevMatT<double> MPd, MQd;
   const double *th0 = nullptr, *V0 = nullptr, *c0 = nullptr, *s0 = nullptr;
-  const int32_t *mis_order = nullptr, *misq_order = nullptr;
+  BusTab tabP, tabQ;
+  const double2* ef0 = nullptr;
   const int32_t* bus_of_user = nullptr;  // caller's bus -> internal bus
   gpcg_options opt{};
   int num_sms = 0, n = 0, m = 0, slack = -1, rows = 0, tile = 0, slack_user = -1;

@@ -79,11 +79,13 @@ __global__ void base_residual_kernel(DevGrid G, const double* __restrict__ V0,
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= G.n) return;
   const double ei = V0[i] * c0[i], fi = V0[i] * s0[i];
-  double re = fma(G.Gii[i], ei, -G.Bii[i] * fi), im = fma(G.Gii[i], fi, G.Bii[i] * ei);
+  const double2 yd = G.ydiag[i];
+  double re = fma(yd.x, ei, -yd.y * fi), im = fma(yd.x, fi, yd.y * ei);
   const int deg = G.adj_deg[i];
   for (int a = 0; a < deg; ++a) {
     const int j = G.adj_nbr[(size_t)a * G.n + i];
-    const double gv = G.adj_g[(size_t)a * G.n + i], bv = G.adj_b[(size_t)a * G.n + i];
+    const double2 gb = G.adj_gb[(size_t)a * G.n + i];
+    const double gv = gb.x, bv = gb.y;
     const double ej = V0[j] * c0[j], fj = V0[j] * s0[j];
     re = fma(-gv, ej, fma(bv, fj, re));
     im = fma(-gv, fj, fma(-bv, ej, im));
@@ -104,10 +106,16 @@ cudaError_t launch_base_residual(cudaStream_t st, const DevGrid& G, const double
   return cudaGetLastError();
 }
 
-// Base-case cos/sin per bus, shared by every scenario's warm start.
-__global__ void base_trig_kernel(int n, const double* th, double* c, double* s) {
+// Base-case cos/sin and e + jf per bus, shared by every scenario's warm start.
+__global__ void base_trig_kernel(int n, const double* th, const double* V, double* c, double* s,
+                                 double2* ef) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) sincos(th[i], &s[i], &c[i]);
+  if (i >= n) return;
+  double sn, cs;
+  sincos(th[i], &sn, &cs);
+  c[i] = cs;
+  s[i] = sn;
+  ef[i] = make_double2(V[i] * cs, V[i] * sn);
 }
 
 // ----------------------------------------------------------- launchers
@@ -136,8 +144,9 @@ cudaError_t launch_apply(cudaStream_t st, int grid, const DevMatT<VT>& M, int op
   return cudaGetLastError();
 }
 
-cudaError_t launch_base_trig(cudaStream_t st, int n, const double* th, double* c, double* s) {
-  base_trig_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, th, c, s);
+cudaError_t launch_base_trig(cudaStream_t st, int n, const double* th, const double* V, double* c,
+                             double* s, double2* ef) {
+  base_trig_kernel<<<(n + 255) / 256, 256, 0, st>>>(n, th, V, c, s, ef);
   return cudaGetLastError();
 }
 

@@ -12,12 +12,31 @@ constexpr double DIVERGE_LIMIT = 1.0e4;   // p.u.: a larger mismatch is divergen
 constexpr double DIVERGE_GROWTH = 10.0;   // as is growth to this multiple of the best
 enum { PREC_IC0 = 0, PREC_JACOBI = 1, PREC_EXACT = 2 };
 
+constexpr int MD_DEG = 0xff, MD_TYPE_SHIFT = 8, MD_TYPE = 3, MD_OVER = 1 << 10;
+
+// The buses of a half-step in the order its mismatch and update passes visit
+// them, with what they need to know of each in that order, so that a warp's
+// loads coalesce: md = {bus, preorder, degree in the padded adjacency (MD_DEG)
+// | bus type | MD_OVER: overflow entries, row of the half-step's matrix}, the
+// neighbour and (c g, c b_y) of each slot (slot a of entry k at a * n + k), the
+// admittance diagonal and the scheduled injections.  Bus order, sorted by
+// degree and type inside windows of MD_WINDOW entries: the threads of a warp
+// run neighbour loops of equal length.
+constexpr int MD_WINDOW = 512;
+struct BusTab {
+  const int4* md = nullptr;
+  const int32_t* nbr = nullptr;
+  const double2 *gb = nullptr, *yd = nullptr, *pq = nullptr;
+  int n = 0;
+};
+
 struct FdpfParams {
   DevGrid G;
   int S = 0, n_tiles = 0;
   ScenInfo sc;
   const double *th0 = nullptr, *V0 = nullptr;  // warm start (bus order)
   const double *c0 = nullptr, *s0 = nullptr;   // cos, sin of th0
+  const double2* ef0 = nullptr;                // V0 (c0, s0)
   const double *r0P = nullptr, *r0Q = nullptr; // base-case mismatch per bus (null: not used)
   int flat_start = 0;
   double tol = 1e-4, inner_rtol = 3e-3;
@@ -44,8 +63,7 @@ struct FdpfParams {
   // diagnostics, or null: [8] per-phase SM cycles summed over CTAs, then per
   // scenario the global timer (ns) when a lane took it and when it retired
   unsigned long long* phase_cycles = nullptr;
-  const int32_t* mis_order = nullptr;   // non-slack buses sorted by degree
-  const int32_t* misq_order = nullptr;  // B'' rows sorted by their bus's degree
+  BusTab tabP, tabQ;  // non-slack buses, rows of B'; PQ buses, rows of B''
 };
 
 // Whether the inner solves run in their reduced form (reduced.cuh): the
@@ -74,7 +92,8 @@ template <typename VT>
 cudaError_t launch_apply(cudaStream_t st, int grid, const DevMatT<VT>& M, int op, int S,
                          const int32_t* outages, const int32_t* f, const int32_t* t,
                          const double* X, double* Y, VT* wbuf, size_t vstride, int precond);
-cudaError_t launch_base_trig(cudaStream_t st, int n, const double* th, double* c, double* s);
+cudaError_t launch_base_trig(cudaStream_t st, int n, const double* th, const double* V, double* c,
+                             double* s, double2* ef);
 cudaError_t launch_base_residual(cudaStream_t st, const DevGrid& G, const double* V0,
                                  const double* c0, const double* s0, double* r0P, double* r0Q);
 

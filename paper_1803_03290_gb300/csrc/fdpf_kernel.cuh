@@ -48,7 +48,7 @@ __device__ __forceinline__ float inv_vmag<float>(double e, double f) {
 }
 template <>
 __device__ __forceinline__ double inv_vmag<double>(double e, double f) {
-  return 1.0 / sqrt(fma(e, e, f * f));
+  return rsqrt(fma(e, e, f * f));  // 7 FP64 instructions, 1 / sqrt takes 15
 }
 
 // ------------------------------------------------------------ mismatch
@@ -58,12 +58,6 @@ __device__ __forceinline__ double inv_vmag<double>(double e, double f) {
 template <int T>
 __device__ __forceinline__ size_t ef_at(int bus, int lane) {
   return ((size_t)bus * T + lane) * 2;
-}
-
-// The neighbour slots of bus i (slot-major adjacency).
-__device__ __forceinline__ void ld_nbrs(const DevGrid& G, int i, int (&nb)[KG]) {
-#pragma unroll
-  for (int a = 0; a < KG; ++a) nb[a] = __ldg(G.adj_nbr + (size_t)a * G.n + i);
 }
 
 // I_i = sum_j Y_ij V_j at bus i for lane ln, the lane's outaged branch left
@@ -77,7 +71,8 @@ __device__ __forceinline__ double2 bus_current(const DevGrid& G, const LaneState
   for (int a = 0; a < deg; ++a) {
     if (__ldg(G.adj_brl + (size_t)a * G.n + i) == br) continue;
     const int j = __ldg(G.adj_nbr + (size_t)a * G.n + i);
-    const double gv = __ldg(G.adj_g + (size_t)a * G.n + i), bv = __ldg(G.adj_b + (size_t)a * G.n + i);
+    const double2 gb = __ldg(G.adj_gb + (size_t)a * G.n + i);
+    const double gv = gb.x, bv = gb.y;
     const double2 u = *reinterpret_cast<const double2*>(EF + ef_at<T>(j, ln));
     re = fma(-gv, u.x, fma(bv, u.y, re));
     im = fma(-gv, u.y, fma(-bv, u.x, im));
@@ -92,7 +87,8 @@ __device__ __forceinline__ double2 bus_current(const DevGrid& G, const LaneState
     im = fma(-gw, u.y, fma(-bw, u.x, im));
   }
   const double2 v = *reinterpret_cast<const double2*>(EF + ef_at<T>(i, ln));
-  double Gii = __ldg(G.Gii + i), Bii = __ldg(G.Bii + i);
+  const double2 yd = __ldg(G.ydiag + i);
+  double Gii = yd.x, Bii = yd.y;
   if (i == L.fb[ln] || i == L.tb[ln]) {
     const double c2 = i == L.fb[ln] ? L.cl[ln] * L.cl[ln] : 1.0;
     Gii -= c2 * L.gl[ln];
@@ -105,176 +101,176 @@ __device__ __forceinline__ double2 bus_current(const DevGrid& G, const LaneState
 // I = Y V, P + jQ = V conj(I).  The outaged branch is left out of the
 // neighbour sum and of the diagonal.  WITH_P: the P half-step (writes
 // dP/V into the B' right-hand side and tracks max|dP| and max|dQ| for the
-// convergence test); otherwise writes dQ/V into the B'' right-hand side.
-// A thread takes a bus and its lanes two at a time: each neighbour's
+// convergence test, L.emax); otherwise writes dQ/V into the B'' right-hand
+// side.  A thread takes a bus and its lanes two at a time: each neighbour's
 // admittance and the pair's voltages are loaded once for the two lanes.
+//
+// FP64 bound: about 4 (degree + 1) + 3 fused multiply-adds per bus and lane
+// at 2 per SM and clock.  Everything that can be is kept off that pipe (maxima
+// and island tests on integers, conversions by cvt_f32), a lane without
+// re-dispatch skips its term, and the buses an outage or a switch changes are
+// found by one bit test per bus.  What a row needs to know comes in one
+// descriptor and one 16-byte load per neighbour slot, in the order of the
+// visit (BusTab).
 template <int T, typename VT, bool WITH_P, bool GEN>
-__device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMatT<VT>& MP,
-                                               const DevMatT<VT>& MQ, LaneState<T>& L,
-                                               const double* __restrict__ EF,
+__device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMatT<VT>& MQ,
+                                               LaneState<T>& L, const double* __restrict__ EF,
                                                VT* __restrict__ rhs,
-                                               Vec<unsigned long long, Geo<T>::LP>& errP_,
-                                               Vec<unsigned long long, Geo<T>::LP>& errQ_,
                                                SwitchState<T>* SW = nullptr) {
   constexpr int LP = Geo<T>::LP;
+  static_assert(LP == 2, "lanes come in pairs");
   const Geo<T> g;
   const DevGrid& G = P.G;
-  // the running maxima in registers through the row loop (the caller's
-  // copies sit in its local memory)
-  Vec<unsigned long long, LP> errP = errP_, errQ = errQ_;
-  // rows are visited in order of bus degree, so the threads of a warp run
-  // neighbour loops of equal length and no FP64 work is spent on padding
-  const int nrows = WITH_P ? G.n - 1 : MQ.n;
-  const int32_t* order = WITH_P ? P.mis_order : P.misq_order;
-  int kn = 0, nbn[KG];
-  if (g.rs < nrows) {
-    kn = __ldg(order + g.rs);
-    ld_nbrs(G, WITH_P ? kn : __ldg(MQ.bus_of_row + kn), nbn);
+  const BusTab& tab = WITH_P ? P.tabP : P.tabQ;
+  const int nrows = tab.n;
+  const int l0 = g.lane, l1 = g.lane + 1;
+  const bool act0 = L.active[l0] != 0, act1 = L.active[l1] != 0;
+  const int lo0 = L.lo[l0], cnt0 = L.cnt[l0], lo1 = L.lo[l1], cnt1 = L.cnt[l1];
+  // a lane's first P half-step away from the ends of its outaged branch: the
+  // base-case mismatch holds (the state is the base case there)
+  const bool first0 = WITH_P && P.r0P && L.outer[l0] == 0;
+  const bool first1 = WITH_P && P.r0P && L.outer[l1] == 0;
+  // lanes with an injection to re-dispatch
+  const bool red0 = WITH_P && __double_as_longlong(L.coef[l0]) != 0;
+  const bool red1 = WITH_P && __double_as_longlong(L.coef[l1]) != 0;
+  // the buses that are not as in the base case, as bits (bus & 63)
+  unsigned long long filt = 0ull;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int ln = l0 + j;
+    if (L.fb[ln] >= 0) filt |= 1ull << (L.fb[ln] & 63);
+    if (L.tb[ln] >= 0) filt |= 1ull << (L.tb[ln] & 63);
+    if (GEN && WITH_P) {
+      if (L.gb[ln] >= 0) filt |= 1ull << (L.gb[ln] & 63);
+      for (int s = 0; s < SW->nx[ln]; ++s) filt |= 1ull << (SW->xb[ln][s] & 63);
+    }
   }
   for (int kk = g.rs; kk < nrows; kk += Geo<T>::RPS) {
-    const int k = kn;
-    int nb[KG];
-#pragma unroll
-    for (int a = 0; a < KG; ++a) nb[a] = nbn[a];
-    if (kk + Geo<T>::RPS < nrows) {
-      kn = __ldg(order + kk + Geo<T>::RPS);
-      ld_nbrs(G, WITH_P ? kn : __ldg(MQ.bus_of_row + kn), nbn);
-    }
-    const int i = WITH_P ? k : __ldg(MQ.bus_of_row + k);
-    const int pr = __ldg(G.pre + i);
-    const int deg = __ldg(G.adj_deg + i);
+    const int4 d = __ldg(tab.md + kk);
+    const int i = d.x;
+    const bool on0 = act0 && !in_island(d.y, lo0, cnt0);
+    const bool on1 = act1 && !in_island(d.y, lo1, cnt1);
     Vec<VT, LP> out = vzero<VT, LP>();
-#pragma unroll 1
-    for (int jp = 0; jp < LP; jp += 2) {
-      const int l0 = g.lane + jp, l1 = l0 + 1;
-      const bool on0 = L.active[l0] && !in_island(pr, L.lo[l0], L.cnt[l0]);
-      const bool on1 = L.active[l1] && !in_island(pr, L.lo[l1], L.cnt[l1]);
-      if (!(on0 || on1)) continue;
-      // a lane's first P half-step away from the ends of its outaged branch:
-      // the base-case mismatch holds (the state is the base case there)
-      bool w0 = false, w1 = false;
-      if (WITH_P && P.r0P) {
-        w0 = on0 && L.outer[l0] == 0 && i != L.fb[l0] && i != L.tb[l0];
-        w1 = on1 && L.outer[l1] == 0 && i != L.fb[l1] && i != L.tb[l1];
-      }
+    if (on0 || on1) {
+      const bool hit = (filt >> (i & 63)) & 1ull;
+      const bool end0 = hit && (i == L.fb[l0] || i == L.tb[l0]);
+      const bool end1 = hit && (i == L.fb[l1] || i == L.tb[l1]);
+      const bool w0 = on0 && first0 && !end0, w1 = on1 && first1 && !end1;
       const bool n0 = on0 && !w0, n1 = on1 && !w1;  // lanes that sum the neighbours
+      const double2* own = reinterpret_cast<const double2*>(EF + ef_at<T>(i, l0));
+      const double2 ev0 = own[0], ev1 = own[1];
       // -sum over the neighbours of Y_ij V_j, both lanes of the pair
       double re0 = 0.0, im0 = 0.0, re1 = 0.0, im1 = 0.0;
       if (n0 || n1) {
-#pragma unroll
-      for (int a0 = 0; a0 < KG; a0 += MIS_GROUP) {
-        double2 u0[MIS_GROUP], u1[MIS_GROUP];
-        double gv[MIS_GROUP], bv[MIS_GROUP];
-#pragma unroll
-        for (int a = 0; a < MIS_GROUP; ++a)
-          if (a0 + a < deg) {
-            const double2* q2 = reinterpret_cast<const double2*>(EF + ef_at<T>(nb[a0 + a], l0));
-            u0[a] = q2[0];
-            u1[a] = q2[1];
-            gv[a] = __ldg(G.adj_g + (size_t)(a0 + a) * G.n + i);
-            bv[a] = __ldg(G.adj_b + (size_t)(a0 + a) * G.n + i);
+        const int deg = d.z & MD_DEG;
+        const int32_t* nbr = tab.nbr + kk;
+        const double2* gbp = tab.gb + kk;
+#pragma unroll 2
+        for (int a = 0; a < deg; ++a) {
+          const double2* q2 =
+              reinterpret_cast<const double2*>(EF + ef_at<T>(__ldg(nbr + (size_t)a * nrows), l0));
+          const double2 gb = __ldg(gbp + (size_t)a * nrows);
+          const double2 u0 = q2[0], u1 = q2[1];
+          if (n0) {
+            re0 = fma(-gb.x, u0.x, fma(gb.y, u0.y, re0));
+            im0 = fma(-gb.x, u0.y, fma(-gb.y, u0.x, im0));
           }
-#pragma unroll
-        for (int a = 0; a < MIS_GROUP; ++a)
-          if (a0 + a < deg) {
+          if (n1) {
+            re1 = fma(-gb.x, u1.x, fma(gb.y, u1.y, re1));
+            im1 = fma(-gb.x, u1.y, fma(-gb.y, u1.x, im1));
+          }
+        }
+        if (d.z & MD_OVER) {
+          const int o1 = __ldg(G.adj_optr + i + 1);
+          for (int e = __ldg(G.adj_optr + i); e < o1; ++e) {
+            const int jn = __ldg(G.adj_onbr + e);
+            const double gw = __ldg(G.adj_og + e), bw = __ldg(G.adj_ob + e);
+            const double2* q2 = reinterpret_cast<const double2*>(EF + ef_at<T>(jn, l0));
+            const double2 v0 = q2[0], v1 = q2[1];
             if (n0) {
-              re0 = fma(-gv[a], u0[a].x, fma(bv[a], u0[a].y, re0));
-              im0 = fma(-gv[a], u0[a].y, fma(-bv[a], u0[a].x, im0));
+              re0 = fma(-gw, v0.x, fma(bw, v0.y, re0));
+              im0 = fma(-gw, v0.y, fma(-bw, v0.x, im0));
             }
             if (n1) {
-              re1 = fma(-gv[a], u1[a].x, fma(bv[a], u1[a].y, re1));
-              im1 = fma(-gv[a], u1[a].y, fma(-bv[a], u1[a].x, im1));
+              re1 = fma(-gw, v1.x, fma(bw, v1.y, re1));
+              im1 = fma(-gw, v1.y, fma(-bw, v1.x, im1));
             }
           }
-      }
-      const int o0 = __ldg(G.adj_optr + i), o1 = __ldg(G.adj_optr + i + 1);
-      for (int e = o0; e < o1; ++e) {
-        const int jn = __ldg(G.adj_onbr + e);
-        const double gw = __ldg(G.adj_og + e), bw = __ldg(G.adj_ob + e);
-        const double2* q2 = reinterpret_cast<const double2*>(EF + ef_at<T>(jn, l0));
-        const double2 v0 = q2[0], v1 = q2[1];
-        if (n0) {
-          re0 = fma(-gw, v0.x, fma(bw, v0.y, re0));
-          im0 = fma(-gw, v0.y, fma(-bw, v0.x, im0));
         }
-        if (n1) {
-          re1 = fma(-gw, v1.x, fma(bw, v1.y, re1));
-          im1 = fma(-gw, v1.y, fma(-bw, v1.x, im1));
-        }
-      }
-      // the outaged branch's term back out at its two end buses
+        // the outaged branch's terms back out at its two end buses
+        if (end0 || end1) {
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int ln = j ? l1 : l0;
-        if (!(j ? n1 : n0) || (i != L.fb[ln] && i != L.tb[ln])) continue;
-        const int e = i == L.fb[ln] ? 0 : 1;
-        const double2 v = *reinterpret_cast<const double2*>(
-            EF + ef_at<T>(e ? L.fb[ln] : L.tb[ln], ln));
-        const double go = L.og[ln][e], bo = L.ob[ln][e];
-        double& re = j ? re1 : re0;
-        double& im = j ? im1 : im0;
-        re -= fma(-go, v.x, bo * v.y);
-        im -= fma(-go, v.y, -bo * v.x);
-      }
+          for (int j = 0; j < 2; ++j) {
+            const int ln = l0 + j;
+            if (!(j ? n1 && end1 : n0 && end0)) continue;
+            const int e = i == L.fb[ln] ? 0 : 1;
+            const double2 v = *reinterpret_cast<const double2*>(
+                EF + ef_at<T>(e ? L.fb[ln] : L.tb[ln], ln));
+            const double go = L.og[ln][e], bo = L.ob[ln][e];
+            double& re = j ? re1 : re0;
+            double& im = j ? im1 : im0;
+            re -= fma(-go, v.x, bo * v.y);
+            im -= fma(-go, v.y, -bo * v.x);
+            // and its share of the diagonal
+            const double c2 = e ? 1.0 : L.cl[ln] * L.cl[ln];
+            const double gs = c2 * L.gl[ln], bs = c2 * L.bl[ln];
+            const double eo = j ? ev1.x : ev0.x, fo = j ? ev1.y : ev0.y;
+            re -= fma(gs, eo, -bs * fo);
+            im -= fma(gs, fo, bs * eo);
+          }
+        }
       }
       // own voltage, the diagonal term and the mismatch of each lane
-      const double2* own = reinterpret_cast<const double2*>(EF + ef_at<T>(i, l0));
-      const double2 ev0 = own[0], ev1 = own[1];
-      const int bt = G.bus_type[i];
-      const double Gii = __ldg(G.Gii + i), Bii = __ldg(G.Bii + i), qs = __ldg(G.Q_sched + i);
-      double Ps = 0.0, pg = 0.0, Pgr = 0.0;
-      if (WITH_P) {
-        Ps = __ldg(G.P_sched + i);
-        if (bt == 1) {
-          Pgr = __ldg(G.P_gen + i);
-          pg = fmax(Pgr, 0.0);  // generators with P_gen > 0 take it
-        }
-      }
+      const int bt = (d.z >> MD_TYPE_SHIFT) & MD_TYPE;
+      const double2 yd = __ldg(tab.yd + kk), pq = __ldg(tab.pq + kk);
+      const double qs = pq.y;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
         if (!(j ? on1 : on0)) continue;
-        const int ln = j ? l1 : l0;
+        const int ln = l0 + j;
+        const double ei = j ? ev1.x : ev0.x, fi = j ? ev1.y : ev0.y;
+        const VT iv = inv_vmag<VT>(ei, fi);
         // a tripped generator's bus keeps only its load and takes no share
         // of the re-dispatch; a bus with an extension row (that one, or a PV
         // bus held at a reactive limit) is PQ with the injection qx
-        const bool tr = GEN && WITH_P && i == L.gb[ln];
-        const double pgl = tr ? 0.0 : pg;
-        bool xe = false;
+        bool tr = false, xe = false;
         double qx = qs;
         int xr = -1;  // the bus's extension row
-        if (GEN && WITH_P)
+        if (GEN && WITH_P && hit) {
+          tr = i == L.gb[ln];
           for (int s = 0; s < SW->nx[ln]; ++s)
             if (SW->xb[ln][s] == i) { xe = true; qx = SW->xq[ln][s]; xr = s; }
+        }
+        // ps with the bus's share of the re-dispatch: generators with P_gen > 0
+        // take it (kept in branches with loads of their own, so that the rows
+        // without a share spend nothing on it)
+        auto redispatched = [&](double ps) {
+          if (GEN && tr) {
+            ps -= __ldg(G.P_gen + i);
+          } else if (bt == 1 && (j ? red1 : red0)) {
+            ps = fma(L.coef[ln], fmax(__ldg(G.P_gen + i), 0.0), ps);
+          }
+          return ps;
+        };
         if (j ? w1 : w0) {
           // the base-case state here: the base case is within the reactive limits
-          const double dP = fma(L.coef[ln], pgl, __ldg(P.r0P + i)) - (tr ? Pgr : 0.0);
-          upd_max_bits(errP.v[jp + j], dP);
+          const double dP = redispatched(__ldg(P.r0P + i));
+          upd_max_shared<Geo<T>::TPR == 1>(&L.emax[0][ln], dP);
           if (bt == 0 || xe) {
             const double q0 = __ldg(P.r0Q + i);
-            upd_max_bits(errQ.v[jp + j], xe ? q0 + (qx - qs) : q0);
+            upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], xe ? q0 + (qx - qs) : q0);
           }
-          out.v[jp + j] = to_vt<VT>(dP) * (j ? inv_vmag<VT>(ev1.x, ev1.y)
-                                             : inv_vmag<VT>(ev0.x, ev0.y));
+          out.v[j] = to_vt<VT>(dP) * iv;
           continue;
         }
-        const double ei = j ? ev1.x : ev0.x, fi = j ? ev1.y : ev0.y;
-        const VT iv = inv_vmag<VT>(ei, fi);
-        double Gd = Gii, Bd = Bii;
-        if (i == L.fb[ln] || i == L.tb[ln]) {  // the outaged branch's share
-          const double c2 = i == L.fb[ln] ? L.cl[ln] * L.cl[ln] : 1.0;
-          Gd -= c2 * L.gl[ln];
-          Bd -= c2 * L.bl[ln];
-        }
         // I_i = Y_ii V_i + sum_j Y_ij V_j
-        const double re = fma(Gd, ei, fma(-Bd, fi, j ? re1 : re0));
-        const double im = fma(Gd, fi, fma(Bd, ei, j ? im1 : im0));
+        const double re = fma(yd.x, ei, fma(-yd.y, fi, j ? re1 : re0));
+        const double im = fma(yd.x, fi, fma(yd.y, ei, j ? im1 : im0));
         // dQ = Q_sched - Im(V_i conj(I_i)); dP = P_sched + re-dispatch - Re(...)
-        VT res;
         if (WITH_P) {
-          const double dP =
-              fma(-ei, re, fma(-fi, im, fma(L.coef[ln], pgl, tr ? Ps - Pgr : Ps)));
-          upd_max_bits(errP.v[jp + j], dP);
-          if (bt == 0 || xe) upd_max_bits(errQ.v[jp + j], fma(-fi, re, fma(ei, im, qx)));
+          const double dP = fma(-ei, re, fma(-fi, im, redispatched(pq.x)));
+          upd_max_shared<Geo<T>::TPR == 1>(&L.emax[0][ln], dP);
+          if (bt == 0 || xe) upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], fma(-fi, re, fma(ei, im, qx)));
           if (GEN && bt == 1 && !xe && G.qmax) {
             // a PV generator's output Q(V) - Q_sched = -dQ against its limits:
             // a violation is a candidate for the switch to PQ at that limit
@@ -297,17 +293,15 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
             if ((side > 0 && vm > vs) || (side < 0 && vm < vs))
               atomicOr(&SW->bk[ln], 1u << xr);
           }
-          res = to_vt<VT>(dP) * iv;
+          out.v[j] = to_vt<VT>(dP) * iv;
         } else {
           const double dQ = fma(-fi, re, fma(ei, im, qs));
-          upd_max_bits(errQ.v[jp + j], dQ);  // decides whether the Q step is taken
-          res = to_vt<VT>(dQ) * iv;
+          upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], dQ);  // decides whether the Q step is taken
+          out.v[j] = to_vt<VT>(dQ) * iv;
         }
-        out.v[jp + j] = res;
       }
     }
-    if (WITH_P) stv<LP>(rhs + (size_t)__ldg(MP.row_of_bus + i) * T + g.lane, out);
-    else stv<LP>(rhs + (size_t)k * T + g.lane, out);
+    stv<LP>(rhs + (size_t)d.w * T + g.lane, out);
   }
   // the B'' extension rows: dQ/V at their buses, with the reactive
   // injection each holds
@@ -321,25 +315,31 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
         const double2 I = bus_current<T>(G, L, EF, b, ln);
         const double2 v = *reinterpret_cast<const double2*>(EF + ef_at<T>(b, ln));
         const double dQ = fma(-v.y, I.x, fma(v.x, I.y, SW->xq[ln][s]));
-        upd_max_bits(errQ.v[j], dQ);
+        upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], dQ);
         rhs[(size_t)(MQ.n + 1 + s) * T + ln] = to_vt<VT>(dQ) * inv_vmag<VT>(v.x, v.y);
       }
     }
-  errP_ = errP;
-  errQ_ = errQ;
 }
 
 // (e, f) rotated through the angle d, in FP64:
 //   e' = e cos d - f sin d = e - (e a + f b),  f' = f - (f a - e b),
-// with a = 1 - cos d and b = sin d.  For |d| <= 0.02 both come from their
-// Taylor series in u = d^2 (a = u/2 - u^2/24 + u^3/720, b = d - d^3/6 +
-// d^5/120; the first dropped terms are below 3e-16 there), larger steps call
-// sincos.  The rotation is exact to FP64 rounding, so the state (e, f) stays
-// at the angle theta and modulus |V| that the kernel reports: the state whose
-// mismatch the convergence test evaluated is the state that is returned.
-__device__ __forceinline__ void rotate_ef(double d, double& e, double& f) {
+// with a = 1 - cos d and b = sin d from their Taylor series.  For |d| <= 1e-4,
+// where most buses are after a scenario's first step, a = d^2/2 and
+// b = d - d^3/6 (d a / 3 = d^3/6; the first dropped terms are below 5e-18); for
+// |d| <= 0.02 two more terms in u = d^2 (dropped terms below 3e-16); larger
+// steps call sincos.  The rotation is exact to FP64 rounding, so the state
+// (e, f) stays at the angle theta and modulus |V| that the kernel reports: the
+// state whose mismatch the convergence test evaluated is the state that is
+// returned.  x: the step in the inner solve's precision, which decides the
+// branch off the FP64 pipe; d: the same in FP64.
+template <typename VT>
+__device__ __forceinline__ void rotate_ef(VT x, double d, double& e, double& f) {
   double a, b;
-  if (fabs(d) <= 0.02) {
+  const VT ax = fabs(x);
+  if (ax <= (VT)1e-4) {
+    a = d * to_f64((VT)0.5 * x);
+    b = fma(d * a, -1.0 / 3.0, d);
+  } else if (ax <= (VT)0.02) {
     const double u = d * d;
     a = u * fma(u, fma(u, 1.0 / 720.0, -1.0 / 24.0), 0.5);
     b = fma(d * u, fma(u, 1.0 / 120.0, -1.0 / 6.0), d);
@@ -363,79 +363,73 @@ __device__ __forceinline__ double v_ratio(VT dv, double e, double f) {
 }
 
 // theta += dtheta (P half-step) or |V| += dV (Q half-step) on the matrix's
-// rows, (scale: the lanes' factors of x, 0 for no step; null: x + xalpha p) as moves of the rectangular voltage: (e, f) rotated through dtheta
-// (theta kept beside it), or e and f both scaled by 1 + dV/|V|, so that
-// e + jf = |V| exp(j theta) holds to FP64 rounding; lanes two at a time.
+// rows, as moves of the rectangular voltage: (e, f) rotated through dtheta
+// (theta kept beside it when it is an output), or e and f both scaled by
+// 1 + dV/|V|, so that e + jf = |V| exp(j theta) holds to FP64 rounding; lanes
+// two at a time.  scale: the lanes' factors of x (0: no step); null: the step
+// is x + xalpha p, the inner solve's deferred last step.  In bus order, so that
+// the state (48 bytes read and written per bus and pair of lanes) streams and
+// only the 8 bytes of x are gathered.
 template <int T, typename VT, bool IS_P, bool GEN>
-__device__ GPCG_LOOP_INLINE void update_pass(const DevMatT<VT>& M, LaneState<T>& L,
-                                             const VT* __restrict__ x,
-                                             const VT* __restrict__ p, double* th,
-                                             double* EF, const SwitchState<T>* SW = nullptr,
+__device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<VT>& M,
+                                             LaneState<T>& L, const VT* __restrict__ x,
+                                             const VT* __restrict__ p, double* th, double* EF,
+                                             const SwitchState<T>* SW = nullptr,
                                              const double* scale = nullptr) {
   constexpr int LP = Geo<T>::LP;
   const Geo<T> g;
-  bool any = false;
-#pragma unroll
-  for (int j = 0; j < LP; ++j) any |= L.active[g.lane + j] != 0;
-  if (!any) return;
-  for (int k = g.rs; k < M.n; k += Geo<T>::RPS) {
-    const int pr = __ldg(M.pre_of_row + k);
-    const int i = __ldg(M.bus_of_row + k);
-#pragma unroll 1
-    for (int jp = 0; jp < LP; jp += 2) {
-      const int l0 = g.lane + jp, l1 = l0 + 1;
-      bool on0 = L.active[l0] && !in_island(pr, L.lo[l0], L.cnt[l0]);
-      bool on1 = L.active[l1] && !in_island(pr, L.lo[l1], L.cnt[l1]);
-      VT xa0, xa1;
-      if (scale) {
-        xa0 = (VT)scale[l0];
-        xa1 = (VT)scale[l1];
-        on0 = on0 && xa0 != (VT)0;
-        on1 = on1 && xa1 != (VT)0;
-      } else {
-        xa0 = (VT)L.xalpha[l0];
-        xa1 = (VT)L.xalpha[l1];
-      }
-      if (!on0 && !on1) continue;
-      const size_t o = (size_t)i * T + l0;
-      Pair<VT> dx = ld2(x + (size_t)k * T + l0);
-      if (scale) {
-        dx.a *= xa0;
-        dx.b *= xa1;
-      } else if (xa0 != (VT)0 || xa1 != (VT)0) {
-        // the inner solve's deferred last step, x += alpha p
-        const Pair<VT> pv = ld2(p + (size_t)k * T + l0);
-        dx.a = fma(xa0, pv.a, dx.a);  // as the solve's own step would take it
-        dx.b = fma(xa1, pv.b, dx.b);
-      }
-      double2* ef = reinterpret_cast<double2*>(EF + ef_at<T>(i, l0));
-      double2 u0 = ef[0], u1 = ef[1];
-      if (IS_P) {
-        Pair<double> t = ld2(th + o);
-        if (on0) {
-          const double d = to_f64(dx.a);
-          t.a += d;
-          rotate_ef(d, u0.x, u0.y);
-        }
-        if (on1) {
-          const double d = to_f64(dx.b);
-          t.b += d;
-          rotate_ef(d, u1.x, u1.y);
-        }
-        st2(th + o, t);
-      } else {
-        if (on0) {
-          const double r = v_ratio<VT>(dx.a, u0.x, u0.y);
-          u0 = make_double2(fma(u0.x, r, u0.x), fma(u0.y, r, u0.y));
-        }
-        if (on1) {
-          const double r = v_ratio<VT>(dx.b, u1.x, u1.y);
-          u1 = make_double2(fma(u1.x, r, u1.x), fma(u1.y, r, u1.y));
-        }
-      }
-      ef[0] = u0;
-      ef[1] = u1;
+  const int l0 = g.lane, l1 = g.lane + 1;
+  bool act0 = L.active[l0] != 0, act1 = L.active[l1] != 0;
+  const VT xa0 = (VT)(scale ? scale[l0] : L.xalpha[l0]);
+  const VT xa1 = (VT)(scale ? scale[l1] : L.xalpha[l1]);
+  if (scale) {
+    act0 = act0 && xa0 != (VT)0;
+    act1 = act1 && xa1 != (VT)0;
+  }
+  if (!act0 && !act1) return;
+  const int lo0 = L.lo[l0], cnt0 = L.cnt[l0], lo1 = L.lo[l1], cnt1 = L.cnt[l1];
+  const int4* __restrict__ md = IS_P ? P.tabP.md : P.tabQ.md;
+  const bool keep_th = IS_P && P.out_theta;
+  for (int kk = g.rs; kk < M.n; kk += Geo<T>::RPS) {
+    const int4 d = __ldg(md + kk);
+    const bool on0 = act0 && !in_island(d.y, lo0, cnt0);
+    const bool on1 = act1 && !in_island(d.y, lo1, cnt1);
+    if (!on0 && !on1) continue;
+    const size_t ox = (size_t)d.w * T + l0;
+    Pair<VT> dx = ld2(x + ox);
+    double2* ef = reinterpret_cast<double2*>(EF + ef_at<T>(d.x, l0));
+    double2 u0 = ef[0], u1 = ef[1];
+    if (scale) {
+      dx.a *= xa0;
+      dx.b *= xa1;
+    } else if (xa0 != (VT)0 || xa1 != (VT)0) {
+      const Pair<VT> pv = ld2(p + ox);
+      dx.a = fma(xa0, pv.a, dx.a);  // as the solve's own step would take it
+      dx.b = fma(xa1, pv.b, dx.b);
     }
+    if (IS_P) {
+      const double d0 = to_f64(dx.a), d1 = to_f64(dx.b);
+      if (on0) rotate_ef<VT>(dx.a, d0, u0.x, u0.y);
+      if (on1) rotate_ef<VT>(dx.b, d1, u1.x, u1.y);
+      if (keep_th) {
+        const size_t o = (size_t)d.x * T + l0;
+        Pair<double> t = ld2(th + o);
+        if (on0) t.a += d0;
+        if (on1) t.b += d1;
+        st2(th + o, t);
+      }
+    } else {
+      if (on0) {
+        const double r = v_ratio<VT>(dx.a, u0.x, u0.y);
+        u0 = make_double2(fma(u0.x, r, u0.x), fma(u0.y, r, u0.y));
+      }
+      if (on1) {
+        const double r = v_ratio<VT>(dx.b, u1.x, u1.y);
+        u1 = make_double2(fma(u1.x, r, u1.x), fma(u1.y, r, u1.y));
+      }
+    }
+    ef[0] = u0;
+    ef[1] = u1;
   }
   // |V| of the extension rows' buses
   if (GEN && !IS_P && M.xptr && g.rs == 0)
@@ -498,8 +492,8 @@ __device__ __forceinline__ void setup_lane(const FdpfParams& P, const DevMatT<VT
     const int dg = G.adj_deg[x];
     for (int a = 0; a < dg && !hit; ++a)
       if (G.adj_brl[(size_t)a * G.n + x] == l) {
-        L.og[ln][e] = G.adj_g[(size_t)a * G.n + x];
-        L.ob[ln][e] = G.adj_b[(size_t)a * G.n + x];
+        L.og[ln][e] = G.adj_gb[(size_t)a * G.n + x].x;
+        L.ob[ln][e] = G.adj_gb[(size_t)a * G.n + x].y;
         hit = true;
       }
     for (int k = G.adj_optr[x]; k < G.adj_optr[x + 1] && !hit; ++k)
@@ -545,19 +539,16 @@ __device__ GPCG_PASS_INLINE void init_pass(const FdpfParams& P, LaneState<T>& L,
   for (int j = 0; j < LP; ++j) fresh |= (L.fresh[g.lane + j] != 0) << j;
   if (!fresh) return;
   for (int i = g.rs; i < G.n; i += Geo<T>::RPS) {
-    double t0, v0, c0, s0;
-    if (P.flat_start) { t0 = 0.0; v0 = G.V_set[i]; c0 = 1.0; s0 = 0.0; }
-    else { t0 = P.th0[i]; v0 = P.V0[i]; c0 = P.c0[i]; s0 = P.s0[i]; }
+    const double2 u = P.flat_start ? make_double2(G.V_set[i], 0.0) : __ldg(P.ef0 + i);
+    const double t0 = P.flat_start || !P.out_theta ? 0.0 : P.th0[i];
     const int pr = G.pre[i];
 #pragma unroll
     for (int j = 0; j < LP; ++j) {
       if (!((fresh >> j) & 1)) continue;
       const int ln = g.lane + j;
-      const size_t o = (size_t)i * T + ln;
       const bool isl = in_island(pr, L.lo[ln], L.cnt[ln]);
-      th[o] = isl ? 0.0 : t0;
-      reinterpret_cast<double2*>(EF + ef_at<T>(i, ln))[0] =
-          isl ? make_double2(0.0, 0.0) : make_double2(v0 * c0, v0 * s0);
+      if (P.out_theta) th[(size_t)i * T + ln] = isl ? 0.0 : t0;
+      reinterpret_cast<double2*>(EF + ef_at<T>(i, ln))[0] = isl ? make_double2(0.0, 0.0) : u;
     }
   }
 }
@@ -603,8 +594,9 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T>& 
     for (int k = g.rs; k < G.m; k += Geo<T>::RPS) {
       const int a = __ldg(G.f + k), b = __ldg(G.t + k);
       const int pa = __ldg(G.pre + a), pb = __ldg(G.pre + b);
-      const double gk = __ldg(G.g + k), bk = __ldg(G.by + k), ir = __ldg(G.inv_rating + k);
-      const double ck = __ldg(G.cf + k);  // 1 / turns ratio at a (1 for a line)
+      // c^2 g, c g, c b and g, c = 1 / turns ratio at a (1 for a line)
+      const double2 y0 = __ldg(G.ybr + 2 * (size_t)k), y1 = __ldg(G.ybr + 2 * (size_t)k + 1);
+      const double ir = __ldg(G.inv_rating + k);
 #pragma unroll 1
       for (int jp = 0; jp < LP; jp += 2) {
         if (!((dn >> jp) & 3)) continue;
@@ -622,10 +614,10 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T>& 
             // P_ba = g |V_b|^2 - c (g Re(V_a conj V_b) - b Im(V_a conj V_b)),
             // c = 1 / turns ratio at a (the pi-model sees V_a c)
             const double ea = va[h].x, fa = va[h].y, eb = vb[h].x, fb = vb[h].y;
-            const double cr = ck * fma(ea, eb, fa * fb), sr = ck * fma(fa, eb, -ea * fb);
-            const double gc = gk * cr;
-            Pab = fma(gk * ck * ck, fma(ea, ea, fa * fa), -fma(bk, sr, gc));
-            const double Pba = fma(gk, fma(eb, eb, fb * fb), fma(bk, sr, -gc));
+            const double cr = fma(ea, eb, fa * fb), sr = fma(fa, eb, -ea * fb);
+            const double gc = y0.y * cr;
+            Pab = fma(y0.x, fma(ea, ea, fa * fa), -fma(y1.x, sr, gc));
+            const double Pba = fma(y1.y, fma(eb, eb, fb * fb), fma(y1.x, sr, -gc));
             // loading max(|P_ab|, |P_ba|) / rating: the larger end picked on
             // the bit patterns, one multiplication
             const unsigned long long u = abs_bits(Pab), v = abs_bits(Pba);
@@ -766,7 +758,7 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
 
   for (;;) {
     // retire finished lanes, then refill empty lanes from the queue
-    if (any_lane<T>(L, L.done)) retire_pass<T>(P, L, th, EF);
+    if (any_lane<T>(L.done)) retire_pass<T>(P, L, th, EF);
     GPCG_PHASE(7);
     if (tid == 0 && !L.drained) {
       int need = 0;
@@ -793,7 +785,10 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
     __syncthreads();
     init_pass<T>(P, L, th, EF);
     __syncthreads();
-    if (tid < T) L.fresh[tid] = 0;
+    if (tid < T) {
+      L.fresh[tid] = 0;
+      L.emax[0][tid] = L.emax[1][tid] = 0ull;
+    }
     if constexpr (GEN) {
       // lanes that sat out the last outer iteration after a switch
       if (tid < T && SW->skip[tid]) {
@@ -803,21 +798,19 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
       __syncthreads();
     }
     GPCG_PHASE(0);
-    if (!any_lane<T>(L, L.active)) {
+    if (!any_lane<T>(L.active)) {
       if (L.drained) break;
       continue;
     }
     // P half-step: mismatch + convergence test
-    Vec<unsigned long long, LP> eP = vzero<unsigned long long, LP>(), eQ = eP;
-    mismatch_pass<T, VT, true, GEN>(P, MP, MQ, L, EF, r, eP, eQ, SW);
-    const Vec<unsigned long long, LP> bP = lane_max_bits<T, RS_ERRP>(L, eP);
-    const Vec<unsigned long long, LP> bQ = lane_max_bits<T, RS_ERRQ>(L, eQ);
-    if (g.rs == 0) {
-#pragma unroll
-      for (int j = 0; j < LP; ++j) {
-        const int ln = g.lane + j;
-        if (!L.active[ln]) continue;
-        const double a = from_bits(bP.v[j]), b = from_bits(bQ.v[j]);
+    mismatch_pass<T, VT, true, GEN>(P, MQ, L, EF, r, SW);
+    __syncthreads();
+    if (tid < T) {
+      {
+        const int ln = tid;
+        const double a = from_bits(L.emax[0][ln]), b = from_bits(L.emax[1][ln]);
+        L.emax[1][ln] = 0ull;
+        if (L.active[ln]) {
         const double e2 = (a != a || b != b) ? INFINITY : fmax(a, b);
         L.err[ln] = e2;
         int st = -1;
@@ -892,46 +885,42 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
         }
         // a P mismatch already within the tolerance takes no P step
         L.hold[ln] = a <= P.tol;
+        }
       }
     }
-    const bool more = any_lane<T>(L, L.active);
+    const bool more = any_lane<T>(L.active);
     GPCG_PHASE(1);
     if (!more) continue;
     if (any_stepping<T>(L)) {
       if constexpr (RED) {
         red_solve<T, VT>(P, MP, L, *RL, r, L.raP, L.rbP, L.inP, L.hold);
         GPCG_PHASE(2);
-        update_pass<T, VT, true, GEN>(MP, L, r, nullptr, th, EF, SW, RL->xa);
+        update_pass<T, VT, true, GEN>(P, MP, L, r, nullptr, th, EF, SW, RL->xa);
       } else {
         pcg_solve<T, VT, true, GEN>(P, MP, L, x, r, p, q, z, L.raP, L.rbP, L.wP, L.inP, nullptr,
                                     nullptr, L.hold);
         GPCG_PHASE(2);
-        update_pass<T, VT, true, GEN>(MP, L, x, p, th, EF, SW);
+        update_pass<T, VT, true, GEN>(P, MP, L, x, p, th, EF, SW);
       }
     }
     __syncthreads();
     GPCG_PHASE(3);
     // Q half-step: the Q mismatch after the P step; a lane whose Q mismatch
     // is within the tolerance takes no Q step
-    Vec<unsigned long long, LP> d0 = vzero<unsigned long long, LP>(), d1 = d0;
-    mismatch_pass<T, VT, false, GEN>(P, MP, MQ, L, EF, r, d0, d1, SW);
-    {
-      const Vec<unsigned long long, LP> bQ2 = lane_max_bits<T, RS_ERRQ>(L, d1);
-      if (g.rs == 0)
-#pragma unroll
-        for (int j = 0; j < LP; ++j) L.hold[g.lane + j] = from_bits(bQ2.v[j]) <= P.tol;
-    }
+    mismatch_pass<T, VT, false, GEN>(P, MQ, L, EF, r, SW);
+    __syncthreads();
+    if (tid < T) L.hold[tid] = from_bits(L.emax[1][tid]) <= P.tol;
     GPCG_PHASE(4);
     if (any_stepping<T>(L)) {
       if constexpr (RED && !GEN) {
         red_solve<T, VT>(P, MQ, L, *RL, r, L.raQ, L.rbQ, L.inQ, L.hold);
         GPCG_PHASE(5);
-        update_pass<T, VT, false, GEN>(MQ, L, r, nullptr, th, EF, SW, RL->xa);
+        update_pass<T, VT, false, GEN>(P, MQ, L, r, nullptr, th, EF, SW, RL->xa);
       } else {
       pcg_solve<T, VT, true, GEN>(P, MQ, L, x, r, p, q, z, L.raQ, L.rbQ, L.wQ, L.inQ,
                                   MQ.c ? L.cl : nullptr, SW, L.hold);
       GPCG_PHASE(5);
-      update_pass<T, VT, false, GEN>(MQ, L, x, p, th, EF, SW);
+      update_pass<T, VT, false, GEN>(P, MQ, L, x, p, th, EF, SW);
       }
     }
     if (g.rs == 0)

@@ -19,10 +19,6 @@ constexpr int LP_MAX = FDPF_LP;  // scenario lanes a thread holds, at most
 #define FDPF_UNROLL 1
 #endif
 constexpr int UNR = FDPF_UNROLL;  // rows per thread in flight in the SpMV
-#ifndef FDPF_MIS_GROUP
-#define FDPF_MIS_GROUP 1
-#endif
-constexpr int MIS_GROUP = FDPF_MIS_GROUP;  // neighbours loaded together in the mismatch
 // Large passes are kept out of line by default (separate register
 // allocation); -DGPCG_PASS_INLINE=__forceinline__ inlines them.
 #ifndef GPCG_PASS_INLINE
@@ -219,8 +215,8 @@ struct SwitchState {
   int skip[T];
 };
 
-constexpr int NRED_SITES = 10;  // reduction sites with a buffer of their own
-enum RedSite { RS_BB = 0, RS_RZ0, RS_PQ, RS_RR, RS_RZ, RS_ERRP, RS_ERRQ, RS_LOAD, RS_RQ, RS_QQ };
+constexpr int NRED_SITES = 8;   // reduction sites with a buffer of their own
+enum RedSite { RS_BB = 0, RS_RZ0, RS_PQ, RS_RR, RS_RZ, RS_LOAD, RS_RQ, RS_QQ };
 
 template <int T>
 struct LaneState {
@@ -242,7 +238,8 @@ struct LaneState {
   double xalpha[T];          // a deferred last step x += alpha p of the inner solve
   // one small buffer per reduction site (see lane_sum): [site][warp][lane]
   double red2[NRED_SITES * (NTHREADS / 32) * T];
-  int flag;
+  // running maxima of |dP| [0] and |dQ| [1] (abs_bits patterns)
+  unsigned long long emax[2][T];
   int drained;
 };
 
@@ -276,37 +273,17 @@ __device__ __forceinline__ Pair<double> lane_reduce(double* red, double v0, doub
 
 // True when some active lane is not held (block-uniform).
 template <int T>
-__device__ __forceinline__ bool any_stepping(LaneState<T>& L) {
+__device__ __forceinline__ bool any_stepping(const LaneState<T>& L) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int any = 0;
-    for (int s = 0; s < T; ++s) any |= (L.active[s] != 0 && L.hold[s] == 0);
-    L.flag = any;
-  }
-  __syncthreads();
-  const bool r = L.flag != 0;
-  __syncthreads();
-  return r;
+  return __syncthreads_or(threadIdx.x < T && L.active[threadIdx.x] != 0 &&
+                          L.hold[threadIdx.x] == 0);
 }
 
 // True when some lane has a nonzero flag (block-uniform).
 template <int T, typename F>
-__device__ __forceinline__ bool any_lane(LaneState<T>& L, const F* flags) {
+__device__ __forceinline__ bool any_lane(const F* flags) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int any = 0;
-    for (int s = 0; s < T; ++s) any |= (flags[s] != 0);
-    L.flag = any;
-  }
-  __syncthreads();
-  const bool r = L.flag != 0;
-  __syncthreads();
-  return r;
-}
-
-__device__ __forceinline__ void upd_max(double& m, double d) {
-  const double a = fabs(d);
-  if (!(a <= m)) m = (a == a) ? a : INFINITY;
+  return __syncthreads_or(threadIdx.x < T && flags[threadIdx.x] != 0);
 }
 
 // |d| as an unsigned 64-bit pattern: for non-negative doubles the integer
@@ -318,6 +295,19 @@ __device__ __forceinline__ unsigned long long abs_bits(double d) {
 __device__ __forceinline__ void upd_max_bits(unsigned long long& m, double d) {
   const unsigned long long a = abs_bits(d);
   m = a > m ? a : m;
+}
+// A running maximum in shared memory: the compare of the high words against
+// the maximum seen so far keeps all but a few values of a pass from the atomic,
+// and the loop that calls it needs no registers for maxima.  WARP: the warp's
+// threads share the maximum (one thread per row), and of those that got past
+// the compare the largest by high word will do.
+template <bool WARP>
+__device__ __forceinline__ void upd_max_shared(unsigned long long* m, double d) {
+  const unsigned long long a = abs_bits(d);
+  const unsigned hi = (unsigned)(a >> 32);
+  if (hi >= reinterpret_cast<const volatile unsigned*>(m)[1] && a) {
+    if (!WARP || hi == __reduce_max_sync(__activemask(), hi)) atomicMax(m, a);
+  }
 }
 // A loading (non-negative) above 1, infinity included and NaN not, decided on
 // the bit pattern (the order of non-negative doubles is their integer order).

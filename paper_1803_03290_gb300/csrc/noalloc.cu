@@ -141,8 +141,8 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
 
   FdpfParams P;
   P.G = c.G;
-  P.mis_order = c.mis_order;
-  P.misq_order = c.misq_order;
+  P.tabP = c.tabP;
+  P.tabQ = c.tabQ;
   P.r0P = c.r0P;
   P.r0Q = c.r0Q;
   P.tol = c.opt.tol;
@@ -151,7 +151,7 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   P.max_inner = c.opt.max_inner;
   P.precond = c.opt.precond;
   P.sc = ScenInfo{const_cast<int32_t*>(outages), lo, cnt, coef, nogen};
-  P.th0 = c.th0; P.V0 = c.V0; P.c0 = c.c0; P.s0 = c.s0;
+  P.th0 = c.th0; P.V0 = c.V0; P.c0 = c.c0; P.s0 = c.s0; P.ef0 = c.ef0;
   P.out_theta = theta; P.out_vm = vm; P.out_flow = flow; P.out_maxload = max_loading;
   P.out_iters = iters; P.out_status = status;
   P.out_nover = n_overload; P.out_ovmask = overload;

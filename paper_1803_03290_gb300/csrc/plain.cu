@@ -170,7 +170,8 @@ __device__ double2 current_at(const DevGrid& G, const Scen& c, const double2* __
   for (int a = 0; a < deg; ++a) {
     if (__ldg(G.adj_brl + (size_t)a * G.n + i) == c.l) continue;
     const int j = __ldg(G.adj_nbr + (size_t)a * G.n + i);
-    const double gv = __ldg(G.adj_g + (size_t)a * G.n + i), bv = __ldg(G.adj_b + (size_t)a * G.n + i);
+    const double2 gb = __ldg(G.adj_gb + (size_t)a * G.n + i);
+    const double gv = gb.x, bv = gb.y;
     const double2 u = EF[j];
     re = fma(-gv, u.x, fma(bv, u.y, re));
     im = fma(-gv, u.y, fma(-bv, u.x, im));
@@ -185,7 +186,8 @@ __device__ double2 current_at(const DevGrid& G, const Scen& c, const double2* __
     im = fma(-gw, u.y, fma(-bw, u.x, im));
   }
   const double2 v = EF[i];
-  double Gd = __ldg(G.Gii + i), Bd = __ldg(G.Bii + i);
+  const double2 yd = __ldg(G.ydiag + i);
+  double Gd = yd.x, Bd = yd.y;
   if (i == c.fb || i == c.tb) {  // the outaged branch's share of the diagonal
     const double c2 = i == c.fb ? c.cl * c.cl : 1.0;
     Gd -= c2 * c.gl;
@@ -421,7 +423,7 @@ __global__ void __launch_bounds__(PT) plain_fdpf_kernel(FdpfParams P, DevMatT<do
         const double d = W.x[k];
         W.th[i] += d;
         double2 u = EF[i];
-        rotate_ef(d, u.x, u.y);
+        rotate_ef<double>(d, d, u.x, u.y);
         EF[i] = u;
       }
       if (!grid_barrier(W)) return;
