@@ -1786,6 +1786,13 @@ static gpcg_status ensure_adj_matrix(gpcg_ctx* c) {
     CUDA_TRY(dalloc(own, &M.xc32, nt * nt));
     CUDA_TRY(dalloc(own, &M.xr32, nt * nt));
   }
+  if (M.br_ptr) {  // the branches' columns: rows shared, values its own
+    int32_t total = 0;
+    CUDA_TRY(cudaMemcpy(&total, M.br_ptr + c->m, sizeof total, cudaMemcpyDeviceToHost));
+    CUDA_TRY(dalloc(own, &M.br_fv, (size_t)total));
+    CUDA_TRY(dalloc(own, &M.br_fm, (size_t)total));
+    CUDA_TRY(dalloc(own, &M.br_sc, (size_t)c->m * SC_N));
+  }
   for (EllDev* E : {&M.A, &M.L, &M.U}) {
     CUDA_TRY(dalloc(own, &E->val, E->nslot));
     CUDA_TRY(dalloc(own, &E->val32, E->nslot));
@@ -1862,6 +1869,7 @@ extern "C" gpcg_status gpcg_n1_adjoint(gpcg_ctx* c, const int32_t* outages, int3
   // base-case B' with the given susceptances, and its factor
   s_ = fill_values(c, c->MA, db);
   if (s_ != GPCG_OK) { cleanup(); return s_; }
+  launch_branch_values(c, c->MA, db, st);
   // outputs (device staging in host mode)
   double *oL = nullptr, *oP = nullptr, *ob = nullptr;
   if (mem == GPCG_MEM_DEVICE) { oL = loss; oP = dL_dP; ob = dL_db; }
@@ -1872,9 +1880,11 @@ extern "C" gpcg_status gpcg_n1_adjoint(gpcg_ctx* c, const int32_t* outages, int3
   }
   const int T = 2;
   const int n_tiles = (int)((S + T - 1) / T);
-  const int per_sm = std::max(1, adjoint_max_blocks_per_sm());
+  const bool red = reduced_form(c->opt.precond, c->MA.view<double>(), c->MA.view<double>());
+  const int per_sm = std::max(1, adjoint_max_blocks_per_sm(red));
   const int slots = std::max(1, std::min(n_tiles, c->num_sms * per_sm));
-  const size_t acc_bytes = (size_t)slots * ((size_t)n + m + 1) * 8;
+  // per slot: gradient sums, loss, and dL/df of its two scenarios
+  const size_t acc_bytes = (size_t)slots * ((size_t)n + m + 1 + 2 * (size_t)m) * 8 + 16;
   if (acc_bytes > c->adj_acc_bytes) {
     if (c->adj_acc) cudaFree(c->adj_acc);
     c->adj_acc = nullptr;
@@ -1886,6 +1896,8 @@ extern "C" gpcg_status gpcg_n1_adjoint(gpcg_ctx* c, const int32_t* outages, int3
   double* accP = c->adj_acc;
   double* accb = accP + (size_t)slots * n;
   double* accL = accb + (size_t)slots * m;
+  // (16-byte aligned: read in pairs)
+  double* accg = accP + ((size_t)slots * ((size_t)n + m + 1) + 1) / 2 * 2;
   if (S) {
     CUDA_TRY_C(cudaMemcpyAsync(c->d_outages, hout.data(), S * 4, cudaMemcpyHostToDevice, st));
     ce = launch_islands(st, (int)S, n, c->d_outages, c->isl, P_in ? dPu : nullptr, c->d_prefP,
@@ -1912,7 +1924,7 @@ extern "C" gpcg_status gpcg_n1_adjoint(gpcg_ctx* c, const int32_t* outages, int3
     P.sstride = ss;
     P.tile_counter = c->d_counter;
     CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st));
-    AdjParamsView A{dPi, db, accP, accb, accL};
+    AdjParamsView A{dPi, db, accP, accb, accL, accg};
     ce = launch_adjoint(st, slots, P, A, c->MA.view<double>());
     if (ce == cudaSuccess) ce = launch_slot_sum(st, 1, slots, accL, nullptr, oL);
     if (ce == cudaSuccess && oP) ce = launch_slot_sum(st, n, slots, accP, c->G.user_of_bus, oP);

@@ -117,10 +117,11 @@ struct AdjParamsView {
   const double* P;   // [n] injections, internal bus order
   const double* b;   // [m] branch susceptances
   double *gP, *gb, *loss;  // per-slot sums: [slots][n], [slots][m], [slots]
+  double* g;               // [slots][m][2] scratch: dL/df of a slot's scenarios
 };
 cudaError_t launch_adjoint(cudaStream_t st, int grid, const FdpfParams& P, const AdjParamsView& A,
                            const DevMatT<double>& M);
-int adjoint_max_blocks_per_sm();
+int adjoint_max_blocks_per_sm(bool red);
 
 // Inputs and outputs of the DC (P-theta) quick screen.
 struct DcParamsView {
