@@ -220,6 +220,7 @@ struct gpcg_ctx {
   std::vector<int32_t> deg;
   std::vector<double2> pq;  // (P_sched, Q_sched), internal numbering
   BusTab tabP, tabQ;
+  int2 *row_pre = nullptr, *br_rows = nullptr;  // the DC screen's output maps
   double2* ef0 = nullptr;
   int32_t* d_bus_of_user = nullptr;  // caller's bus -> internal bus
   unsigned long long* phase = nullptr;  // diagnostics: [8 + 2 phase_cap]
@@ -659,6 +660,12 @@ static gpcg_status build_matrices(gpcg_ctx* c) {
       CUDA_TRY(cudaGetLastError());
       tab = BusTab{d_md, d_nbr, d_gb, d_yd, d_pq, n};
     }
+    std::vector<int2> rp(c->n), ends(c->m);
+    const std::vector<int32_t>& row = c->MP.plan.row_of_bus;
+    for (int b = 0; b < c->n; ++b) rp[c->user_of[b]] = make_int2(row[b], c->pre[b]);
+    for (int k = 0; k < c->m; ++k) ends[k] = make_int2(row[c->f[k]], row[c->t[k]]);
+    CUDA_TRY(upload(own, &c->row_pre, rp.data(), rp.size()));
+    CUDA_TRY(upload(own, &c->br_rows, ends.data(), ends.size()));
     CUDA_TRY(cudaDeviceSynchronize());
   }
   c->planned_precond = c->opt.precond;
@@ -2022,7 +2029,13 @@ extern "C" gpcg_status gpcg_n1_dc_screen(gpcg_ctx* c, const int32_t* outages, in
   const bool f32 = c->opt.precision == GPCG_BATCHED_FP32 || f16;
   const int T = 2;
   const int n_tiles = (int)((S + T - 1) / T);
-  const int per_sm = std::max(1, f32 ? dc_max_blocks_per_sm<float>() : dc_max_blocks_per_sm<double>());
+  // FP64 solves with the complete factor: direct, unless the iterations of the
+  // PCG are asked for
+  const DevMatT<double> M64 = c->MP.view<double>();
+  const bool direct = !f32 && !d_it && reduced_form(c->opt.precond, M64, M64);
+  const int per_sm = std::max(1, direct ? dc_direct_max_blocks_per_sm()
+                                 : f32 ? dc_max_blocks_per_sm<float>()
+                                       : dc_max_blocks_per_sm<double>());
   const int slots = std::max(1, std::min(n_tiles, c->num_sms * per_sm));
   FdpfParams P = base_params(c);
   P.phase_cycles = nullptr;  // the diagnostics cover the AC screens
@@ -2045,8 +2058,10 @@ extern "C" gpcg_status gpcg_n1_dc_screen(gpcg_ctx* c, const int32_t* outages, in
   P.wth = sbase; P.wV = sbase + slots * ss; P.we = sbase + 2 * slots * ss;
   P.wf = sbase + 3 * slots * ss;
   P.sstride = ss;
-  DcParamsView D{dPi, c->G.user_of_bus, d_th, d_fl, d_ml, d_it, d_st, d_nov, d_ovm};
-  ce = f32 ? launch_dc<float>(st, slots, P, D, c->MP.view<float>(f16), c->MP.view<double>())
+  DcParamsView D{dPi, c->G.user_of_bus, d_th, d_fl, d_ml, d_it, d_st, d_nov, d_ovm,
+                 c->row_pre, c->br_rows};
+  ce = direct ? launch_dc_direct(st, slots, P, D, M64, (double*)P.wx)
+       : f32 ? launch_dc<float>(st, slots, P, D, c->MP.view<float>(f16), c->MP.view<double>())
            : launch_dc<double>(st, slots, P, D, c->MP.view<double>(), c->MP.view<double>());
   if (ce != cudaSuccess) { cleanup(); return fail(GPCG_ERR_CUDA, "dc screen: %s", cudaGetErrorString(ce)); }
   if (mem == GPCG_MEM_HOST) {

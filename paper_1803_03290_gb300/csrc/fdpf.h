@@ -134,12 +134,19 @@ struct DcParamsView {
   int32_t* status;              // [S], or null
   int32_t* nover;               // [S] branches loaded above their rating, or null
   uint32_t* ovmask;             // [S][(m + 31) / 32] those branches as bits, or null
+  const int2* row_pre;          // [n] caller's bus -> row of B' (-1: slack), preorder
+  const int2* br_rows;          // [m] rows of B' of the from and the to end
 };
 template <typename VT>
 cudaError_t launch_dc(cudaStream_t st, int grid, const FdpfParams& P, const DcParamsView& D,
                       const DevMatT<VT>& M, const DevMatT<double>& M64);
 template <typename VT>
 int dc_max_blocks_per_sm();
+// The same for the complete factor with FP64 solves and no iteration counts
+// asked for; f0: 2 (rows + 1) doubles of scratch.
+cudaError_t launch_dc_direct(cudaStream_t st, int grid, const FdpfParams& P,
+                             const DcParamsView& D, const DevMatT<double>& M, double* f0);
+int dc_direct_max_blocks_per_sm();
 cudaError_t launch_slot_sum(cudaStream_t st, int n, int slots, const double* acc,
                             const int32_t* map, double* out);
 cudaError_t launch_gather_perm(cudaStream_t st, int n, const int32_t* idx, const double* src,
