@@ -117,8 +117,33 @@ Ell<double> EllDev::view<double>() const { return Ell<double>{col, val, optr, oc
 template <>
 Ell<float> EllDev::view<float>() const { return Ell<float>{col, val32, optr, ocol, oval32}; }
 
+// A substitution's rows in visiting order (SubTab): structure from the host,
+// values gathered on the device through `src` (CSR positions, -1: none).
+struct SubDev {
+  int n = 0, nc = 0;  // rows, further chunks
+  int4 *rc = nullptr, *col = nullptr, *ccol = nullptr;
+  int32_t *src = nullptr, *dsrc = nullptr, *csrc = nullptr;  // positions of the values
+  double *val = nullptr, *id = nullptr, *cval = nullptr;
+  float *val32 = nullptr, *id32 = nullptr, *cval32 = nullptr;
+  template <typename VT>
+  SubTab<VT> view() const;
+};
+template <>
+SubTab<double> SubDev::view<double>() const {
+  return SubTab<double>{rc, col, val, id, ccol, cval};
+}
+template <>
+SubTab<float> SubDev::view<float>() const {
+  return SubTab<float>{rc, col, val32, id32, ccol, cval32};
+}
+
 struct MatDev {
   MatrixPlan plan;
+  SubDev fwd, bwd;
+  int32_t *th_ptr = nullptr, *th_col = nullptr, *th_src = nullptr;  // see DevMatT
+  double* th_val = nullptr;
+  float* th_val32 = nullptr;
+  int n_th = 0;
   int32_t *bus_of_row = nullptr, *row_of_bus = nullptr, *pre_of_row = nullptr, *visit = nullptr;
   int32_t *a_ptr = nullptr, *a_idx = nullptr, *a_diag = nullptr;
   int32_t *l_ptr = nullptr, *l_idx = nullptr, *l_diag = nullptr;
@@ -167,6 +192,8 @@ DevMatT<double> MatDev::view<double>(bool) const {
   M.c = c;
   M.xptr = xptr; M.xrow = xrow; M.xval = xval; M.xdiag = xdiag; M.xnb = xnb; M.xbr = xbr;
   M.br = cols();
+  M.fwd = fwd.view<double>(); M.bwd = bwd.view<double>();
+  M.th_ptr = th_ptr; M.th_col = th_col; M.th_val = th_val;
   return M;
 }
 template <>
@@ -194,6 +221,8 @@ DevMatT<float> MatDev::view<float>(bool f16) const {
   M.c = c;
   M.xptr = xptr; M.xrow = xrow; M.xval = xval32; M.xdiag = xdiag32; M.xnb = xnb; M.xbr = xbr;
   M.br = cols();
+  M.fwd = fwd.view<float>(); M.bwd = bwd.view<float>();
+  M.th_ptr = th_ptr; M.th_col = th_col; M.th_val = th_val32;
   return M;
 }
 
@@ -394,6 +423,63 @@ static void ell_fill(cudaStream_t st, EllDev& D, const double* csr_val) {
   launch_gather_val(st, D.nover, D.osrc, csr_val, D.oval, D.oval32);
 }
 
+// The table of a substitution that visits `order` (rows level by level; ptr:
+// the levels' bounds in it): entries of row i are the positions [ptr_[i], ...)
+// of `A` without the diagonal, val_of maps them to positions of L's values.
+template <typename Entries>
+static cudaError_t sub_upload(std::vector<void*>& own, const std::vector<int32_t>& rows,
+                              const std::vector<int32_t>& ptr, int pad, const MatrixPlan& P,
+                              Entries entries, SubDev& D) {
+  const int n = (int)rows.size();
+  std::vector<int32_t> order(rows);
+  std::vector<std::pair<int, int>> ent;
+  std::vector<int32_t> cnt(P.n, 0);
+  for (int i : rows) { entries(i, ent); cnt[i] = (int32_t)ent.size(); }
+  for (size_t k = 0; k + 1 < ptr.size(); ++k)
+    std::stable_sort(order.begin() + ptr[k], order.begin() + ptr[k + 1],
+                     [&](int a, int b) { return cnt[a] > cnt[b]; });
+  std::vector<int4> rc(n), col, ccol;
+  std::vector<int32_t> src, dsrc(n), csrc;
+  auto chunk = [&](size_t from, std::vector<int4>& cols, std::vector<int32_t>& pos) {
+    int c[SUB_K];
+    for (size_t a = 0; a < SUB_K; ++a) {
+      const bool have = from + a < ent.size();
+      c[a] = have ? ent[from + a].first : pad;
+      pos.push_back(have ? ent[from + a].second : -1);
+    }
+    cols.push_back(make_int4(c[0], c[1], c[2], c[3]));
+  };
+  for (int k = 0; k < n; ++k) {
+    const int i = order[k];
+    entries(i, ent);
+    rc[k] = make_int4(i, cnt[i], (int)ccol.size(), 0);
+    chunk(0, col, src);
+    for (size_t a = SUB_K; a < ent.size(); a += SUB_K) chunk(a, ccol, csrc);
+    dsrc[k] = i;
+  }
+  D.n = n;
+  D.nc = (int)ccol.size();
+  cudaError_t ce;
+  if ((ce = upload(own, &D.rc, rc.data(), rc.size())) != cudaSuccess) return ce;
+  if ((ce = upload(own, &D.col, col.data(), col.size())) != cudaSuccess) return ce;
+  if ((ce = upload(own, &D.src, src.data(), src.size())) != cudaSuccess) return ce;
+  if ((ce = upload(own, &D.dsrc, dsrc.data(), dsrc.size())) != cudaSuccess) return ce;
+  if ((ce = upload(own, &D.ccol, ccol.data(), ccol.size())) != cudaSuccess) return ce;
+  if ((ce = upload(own, &D.csrc, csrc.data(), csrc.size())) != cudaSuccess) return ce;
+  if ((ce = dalloc(own, &D.cval, csrc.size())) != cudaSuccess) return ce;
+  if ((ce = dalloc(own, &D.cval32, csrc.size())) != cudaSuccess) return ce;
+  if ((ce = dalloc(own, &D.val, src.size())) != cudaSuccess) return ce;
+  if ((ce = dalloc(own, &D.val32, src.size())) != cudaSuccess) return ce;
+  if ((ce = dalloc(own, &D.id, dsrc.size())) != cudaSuccess) return ce;
+  return dalloc(own, &D.id32, dsrc.size());
+}
+
+static void sub_fill(cudaStream_t st, SubDev& D, const double* l_val, const double* inv_diag) {
+  launch_gather_val(st, D.n * SUB_K, D.src, l_val, D.val, D.val32);
+  launch_gather_val(st, D.nc * SUB_K, D.csrc, l_val, D.cval, D.cval32);
+  launch_gather_val(st, D.n, D.dsrc, inv_diag, D.id, D.id32);
+}
+
 // Values of a matrix whose structure is built: the weighted Laplacian
 // (weights w per branch), its factor on the planned pattern, diagonals and
 // padded-row values.  Synchronous.
@@ -411,6 +497,32 @@ static gpcg_status alloc_tail(gpcg_ctx* c, MatDev& M, int which, int cap) {
   M.tblev_rows = nullptr;
   if (!P.tblev_rows.empty())
     CUDA_TRY(upload(own, &M.tblev_rows, P.tblev_rows.data(), P.tblev_rows.size()));
+  {
+    std::vector<int32_t> pos(P.L.nnz());  // position in U -> position in L
+    for (int k = 0; k < P.L.nnz(); ++k) pos[P.l_to_u[k]] = k;
+    CUDA_TRY(sub_upload(own, P.tblev_rows, P.tblev_ptr, P.n, P,
+                        [&](int i, std::vector<std::pair<int, int>>& e) {
+                          e.clear();
+                          for (int k = P.U.ptr[i] + 1; k < P.U.ptr[i + 1]; ++k)
+                            e.push_back({P.U.idx[k], pos[k]});
+                        },
+                        M.bwd));
+    std::vector<int32_t> tp(1, 0), tc, ts;
+    for (int i = P.tail_row0; i < P.n; ++i) {
+      for (int k = P.L.ptr[i]; k < P.L.ptr[i + 1]; ++k)
+        if (P.L.idx[k] < P.tail_row0) {
+          tc.push_back(P.L.idx[k]);
+          ts.push_back(k);
+        }
+      tp.push_back((int32_t)tc.size());
+    }
+    M.n_th = (int)tc.size();
+    CUDA_TRY(upload(own, &M.th_ptr, tp.data(), tp.size()));
+    CUDA_TRY(upload(own, &M.th_col, tc.data(), tc.size()));
+    CUDA_TRY(upload(own, &M.th_src, ts.data(), ts.size()));
+    CUDA_TRY(dalloc(own, &M.th_val, tc.size()));
+    CUDA_TRY(dalloc(own, &M.th_val32, tc.size()));
+  }
   const size_t nt = (size_t)(P.n - P.tail_row0);
   CUDA_TRY(dalloc(own, &M.xc, nt * nt));
   CUDA_TRY(dalloc(own, &M.xr, nt * nt));
@@ -423,8 +535,10 @@ static gpcg_status alloc_tail(gpcg_ctx* c, MatDev& M, int which, int cap) {
 
 // The tail block's inverse from the factor's values: of the FP16-stored
 // factor first (M.xc as FP64 scratch), then of the factor itself.
-static void launch_tail_inverses(const MatDev& M, cudaStream_t st) {
+static void launch_tail_inverses(MatDev& M, cudaStream_t st) {
   const MatrixPlan& P = M.plan;
+  sub_fill(st, M.bwd, M.l_val, M.inv_diag);
+  launch_gather_val(st, M.n_th, M.th_src, M.l_val, M.th_val, M.th_val32);
   if (M.lsc && M.xch)
     launch_tail_inverse(st, P.tail_row0, P.n - P.tail_row0, M.l_ptr, M.l_idx, M.l_val, M.lsc,
                         M.xc, nullptr, M.xch, M.xrh);
@@ -449,6 +563,7 @@ static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w) {
   ell_fill(st, M.A, M.a_val);
   ell_fill(st, M.L, M.l_val);
   ell_fill(st, M.U, M.l_val);
+  sub_fill(st, M.fwd, M.l_val, M.inv_diag);
   if (M.lsc) {
     launch_scale_factor(st, P.n, M.l_ptr, M.l_idx, M.l_val, M.lsc, M.inv_d2, M.inv_d2_32);
     for (EllDev* E : {&M.L, &M.U}) {
@@ -563,6 +678,10 @@ static gpcg_status build_matrix(gpcg_ctx* c, MatDev& M, int which,
     CUDA_TRY(ell_upload(own, ell_from_rows(ra, KA, P.n), M.A));
     CUDA_TRY(ell_upload(own, ell_from_rows(rl, KL, P.n), M.L));
     CUDA_TRY(ell_upload(own, ell_from_rows(ru, KU, P.n), M.U));
+    std::vector<int32_t> rows(P.n);
+    for (int i = 0; i < P.n; ++i) rows[i] = i;
+    CUDA_TRY(sub_upload(own, rows, P.lev_ptr, P.n, P,
+                        [&](int i, std::vector<std::pair<int, int>>& e) { e = rl[i]; }, M.fwd));
     for (EllDev* E : {&M.L, &M.U}) {
       CUDA_TRY(dalloc(own, &E->valh, E->nslot));
       CUDA_TRY(dalloc(own, &E->ovalh, E->nover));
@@ -1139,7 +1258,7 @@ static Layout make_layout(const gpcg_ctx* c, int T, int slots, size_t vt_size, b
 // vector's bytes of it) instead of the work buffer.
 template <typename VT>
 static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, int slots,
-                            bool f16 = false, bool zs = false) {
+                            bool f16 = false, bool zs = false, int nt = NTHREADS) {
   const DevMatT<VT> MP = c->MP.view<VT>(f16), MQ = c->MQ.view<VT>(f16);
   const bool red = !zs && reduced_form(P.precond, MP, MQ);
   const bool one = red && !P.sc.gen_bus && !P.G.qmax;
@@ -1163,8 +1282,12 @@ static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, i
   P.wf = sbase + 3 * slots * ss;
   P.sstride = ss;
   P.tile_counter = c->d_counter;
+  if (!P.fill) P.fill = T;
+  const size_t rows = (size_t)std::max(c->MP.plan.n, c->MQ.plan.n) + 1;
+  const size_t wide = one ? wide_shared(nt, rows * T * sizeof(VT)) : 0;
+  if (wide) P.wr = nullptr;
   CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st));
-  CUDA_TRY(launch_fdpf<VT>(st, T, slots, P, MP, MQ, zs ? Lo.vec_bytes : 0));
+  CUDA_TRY(launch_fdpf<VT>(st, T, slots, P, MP, MQ, zs ? Lo.vec_bytes : 0, nt, wide));
   return GPCG_OK;
 }
 
@@ -1215,7 +1338,7 @@ extern "C" gpcg_status gpcg_base_solve(gpcg_ctx* c, double* theta, double* vm, d
   CUDA_TRY(cudaMalloc(&d_iters3, 3 * sizeof(int32_t)));
   P.out_iters = d_iters3;
   P.out_status = d_stat;
-  s = run_fdpf<double>(c, st, P, 2, 1);
+  s = run_fdpf<double>(c, st, P, 2, 1, false, false, wide_launch(1, c->num_sms, c->MP.plan.n, true).nt);
   int32_t hs = -1, hit[3] = {0, 0, 0};
   if (s == GPCG_OK) {
     cudaError_t ce = cudaDeviceSynchronize();
@@ -1445,6 +1568,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
   gpcg_status rs = GPCG_OK;
   int T = 2, slots = 1;
   bool zs = false;
+  int nt = NTHREADS;
   // CTAs per SM of tile width t, with z in shared memory or not (0: does not fit)
   auto blocks = [&](int t, bool z) {
     const size_t zb = z ? make_layout(c, t, 1, f32 ? 4 : 8, true).vec_bytes : 0;
@@ -1571,6 +1695,13 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
     T = c->opt.tile ? c->opt.tile : (c->tile ? c->tile : 2);
     if (ext) T = std::min(T, 8);  // the kernel with extension rows: tiles of 2, 4, 8
     zs = use_zs(T);
+    // few scenarios, no knob asked for by the caller (a fixed tile width promises
+    // the same sums for any number of scenarios): wide CTAs
+    WideLaunch wl{NTHREADS, 0, T};
+    if (red && !ext && !zs && !c->opt.tile && !c->opt.ctas_per_sm) {
+      wl = wide_launch((int)S, c->num_sms, c->MP.plan.n, !f32);
+      if (wl.nt != NTHREADS) T = 2;
+    }
     const int n_tiles = (int)((S + T - 1) / T);
     int per_sm = c->opt.ctas_per_sm ? c->opt.ctas_per_sm : c->per_sm;
     if (!c->opt.ctas_per_sm && per_sm > blocks(T, zs)) per_sm = blocks(T, zs);
@@ -1578,6 +1709,11 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
     per_sm = std::max(per_sm, 1);
     c->per_sm_used = per_sm;
     slots = std::max(1, std::min(n_tiles, c->num_sms * per_sm));
+    if (wl.nt != NTHREADS) {
+      nt = wl.nt;
+      slots = wl.grid;
+      P.fill = wl.fill;
+    }
     P.S = (int)S;
     P.n_tiles = n_tiles;
     P.order = c->d_order;
@@ -1636,7 +1772,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
                                   (uintptr_t)d_flow, (uintptr_t)d_lab, (uintptr_t)d_iters,
                                   (uintptr_t)d_stat, (uintptr_t)d_ml, (uintptr_t)d_nov,
                                   (uintptr_t)d_ovm, (uintptr_t)c->d_outages,
-                                  (uintptr_t)c->d_order, (uintptr_t)c->d_lo, (uintptr_t)gen,
+                                  (uintptr_t)c->d_order, (uintptr_t)c->d_lo, (uintptr_t)gen, (uintptr_t)nt,
                                   (uintptr_t)zs};
     {
       double opts[3] = {c->opt.tol, c->opt.inner_rtol, 0.0};
@@ -1651,8 +1787,8 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
       CUDA_TRY_C(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
       cudaError_t e = enqueue_islands(c->cap_stream, true);
       if (e == cudaSuccess) {
-        rs = f32 ? run_fdpf<float>(c, c->cap_stream, P, T, slots, f16, zs)
-                 : run_fdpf<double>(c, c->cap_stream, P, T, slots, false, zs);
+        rs = f32 ? run_fdpf<float>(c, c->cap_stream, P, T, slots, f16, zs, nt)
+                 : run_fdpf<double>(c, c->cap_stream, P, T, slots, false, zs, nt);
         if (rs == GPCG_OK) e = record(c->ev[2], c->cap_stream, true);
       }
       cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &gr);
@@ -1669,8 +1805,8 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
     return GPCG_OK;
   } else {
     CUDA_TRY_C(enqueue_islands(st));
-    rs = f32 ? run_fdpf<float>(c, st, P, T, slots, f16, zs)
-             : run_fdpf<double>(c, st, P, T, slots, false, zs);
+    rs = f32 ? run_fdpf<float>(c, st, P, T, slots, f16, zs, nt)
+             : run_fdpf<double>(c, st, P, T, slots, false, zs, nt);
   }
   if (rs != GPCG_OK) { cleanup(); return rs; }
   CUDA_TRY_C(cudaEventRecord(c->ev[2], st));
@@ -1691,7 +1827,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
     if (!plain) {
       unsigned long long sub[3];
       CUDA_TRY_C(cudaMemcpy(sub, c->phase + 8 + 2 * S, sizeof sub, cudaMemcpyDeviceToHost));
-      std::fprintf(stderr, "gpcg inner-solve cycles: spmv=%.1f%% fwd=%.1f%% bwd=%.1f%% of all\n",
+      std::fprintf(stderr, "gpcg inner-solve cycles: spmv or recurrence=%.1f%% fwd=%.1f%% bwd=%.1f%% of all\n",
                    100.0 * sub[0] / tot, 100.0 * sub[1] / tot, 100.0 * sub[2] / tot);
     }
   }
@@ -1799,6 +1935,16 @@ static gpcg_status ensure_adj_matrix(gpcg_ctx* c) {
     CUDA_TRY(dalloc(own, &M.br_fv, (size_t)total));
     CUDA_TRY(dalloc(own, &M.br_fm, (size_t)total));
     CUDA_TRY(dalloc(own, &M.br_sc, (size_t)c->m * SC_N));
+  }
+  CUDA_TRY(dalloc(own, &M.th_val, M.n_th));
+  CUDA_TRY(dalloc(own, &M.th_val32, M.n_th));
+  for (SubDev* D : {&M.fwd, &M.bwd}) {
+    CUDA_TRY(dalloc(own, &D->val, (size_t)D->n * SUB_K));
+    CUDA_TRY(dalloc(own, &D->val32, (size_t)D->n * SUB_K));
+    CUDA_TRY(dalloc(own, &D->cval, (size_t)D->nc * SUB_K));
+    CUDA_TRY(dalloc(own, &D->cval32, (size_t)D->nc * SUB_K));
+    CUDA_TRY(dalloc(own, &D->id, D->n));
+    CUDA_TRY(dalloc(own, &D->id32, D->n));
   }
   for (EllDev* E : {&M.A, &M.L, &M.U}) {
     CUDA_TRY(dalloc(own, &E->val, E->nslot));

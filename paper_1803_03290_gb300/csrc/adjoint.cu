@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(NTHREADS, RED ? 3 : FDPF_MIN_BLOCKS)
     const int br0 = L.l[l0], br1 = L.l[l1];
     const bool v0 = L.scen[l0] >= 0, v1 = L.scen[l1] >= 0;
     auto solve = [&]() {
-      if constexpr (RED) red_solve<T, VT>(P, M, L, *RL, r, L.raP, L.rbP, L.inP, nullptr);
+      if constexpr (RED) red_solve<T, NTHREADS, VT>(P, M, L, *RL, r, L.raP, L.rbP, L.inP, nullptr);
       else pcg_solve<T, VT>(P, M, L, x, r, p, q, z, L.raP, L.rbP, L.wP, L.inP);
     };
     // the solution at matrix row k (-1: the slack)

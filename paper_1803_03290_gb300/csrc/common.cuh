@@ -77,6 +77,24 @@ struct BranchCols {
   const double* sc = nullptr;
 };
 
+// The rows of a substitution in the order it visits them -- level by level,
+// the rows of a level by falling number of entries, so that the threads of a
+// warp have equally many and none gathers padding -- with what a row needs in
+// that order, so that a warp's loads coalesce: rc = {row, entries, first further
+// chunk, 0}, the first SUB_K columns and values, and 1 / L_ii.  The entries
+// beyond are in chunks of SUB_K (ccol, cval; padding has value 0), so that a long
+// row waits on one memory latency per SUB_K entries.
+constexpr int SUB_K = 4;
+template <typename VT>
+struct SubTab {
+  const int4* rc = nullptr;
+  const int4* col = nullptr;
+  const VT* val = nullptr;  // [n][SUB_K]
+  const VT* id = nullptr;
+  const int4* ccol = nullptr;
+  const VT* cval = nullptr;  // [chunks][SUB_K]
+};
+
 // One fast-decoupled matrix (B' or B'') with its base-case factor.  VT is
 // the value type used by the solve kernels (float or double).  Vectors of
 // this matrix have n+1 rows per scenario: row n is kept at zero and is what
@@ -116,6 +134,11 @@ struct DevMatT {
   const int32_t* xbr = nullptr;  // the branch of each adjacency entry
   const VT *xval = nullptr, *xdiag = nullptr;
   BranchCols br;  // null pointers: the factor is not the complete one
+  // forward: all levels (lev_ptr); backward: the rows before the tail (tblev_ptr)
+  SubTab<VT> fwd, bwd;
+  // the tail rows' factor entries on the rows before the tail (CSR by tail row)
+  const int32_t *th_ptr = nullptr, *th_col = nullptr;
+  const VT* th_val = nullptr;
 };
 
 // Extension rows a lane may carry at once (see Ext in fdpf_ops.cuh): a

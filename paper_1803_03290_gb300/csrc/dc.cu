@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(NTHREADS) dc_base_kernel(DevMatT<double> M, De
   }
   __syncthreads();
   Vec<double, 2> rr = vzero<double, 2>(), ff = vzero<double, 2>();
-  red_forward<T, double>(M, f, zt, rr, ff);
+  red_forward<T, NTHREADS, 2, double>(M, f, zt, rr, ff);
   __syncthreads();
   for (int k = M.tail_row0 + g.rs; k < M.n; k += Geo<T>::RPS)
     st2(f + (size_t)k * T, ld2(zt + (size_t)(k - M.tail_row0) * T));
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(NTHREADS, FDPF_MIN_BLOCKS)
       }
     }
     __syncthreads();
-    red_backward<T, double>(M, f, zt);
+    red_backward<T, NTHREADS, 2, double>(M, f, zt);
     if (M.ntblev == 0) __syncthreads();
     // theta in the caller's bus order (slack and islanded buses 0)
     if (D.theta)

@@ -121,12 +121,13 @@ __global__ void base_trig_kernel(int n, const double* th, const double* V, doubl
 // ----------------------------------------------------------- launchers
 template <typename VT>
 cudaError_t launch_fdpf(cudaStream_t st, int T, int grid, const FdpfParams& P,
-                        const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes) {
+                        const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes, int nt,
+                        size_t wide_bytes) {
   if (P.sc.gen_bus || P.G.qmax) {
     if (zbytes) return cudaErrorInvalidValue;
     return launch_fdpf_gen<VT>(st, T, grid, P, MP, MQ);
   }
-  return launch_fdpf_g<false, VT>(st, T, grid, P, MP, MQ, zbytes);
+  return launch_fdpf_g<false, VT>(st, T, grid, P, MP, MQ, zbytes, nt, wide_bytes);
 }
 
 template <typename VT>
@@ -151,9 +152,9 @@ cudaError_t launch_base_trig(cudaStream_t st, int n, const double* th, const dou
 }
 
 template cudaError_t launch_fdpf<float>(cudaStream_t, int, int, const FdpfParams&,
-                                        const DevMatT<float>&, const DevMatT<float>&, size_t);
+                                        const DevMatT<float>&, const DevMatT<float>&, size_t, int, size_t);
 template cudaError_t launch_fdpf<double>(cudaStream_t, int, int, const FdpfParams&,
-                                         const DevMatT<double>&, const DevMatT<double>&, size_t);
+                                         const DevMatT<double>&, const DevMatT<double>&, size_t, int, size_t);
 template int fdpf_max_blocks_per_sm<float>(int, bool, size_t, bool);
 template int fdpf_max_blocks_per_sm<double>(int, bool, size_t, bool);
 template cudaError_t launch_apply<float>(cudaStream_t, int, const DevMatT<float>&, int, int,

@@ -1,5 +1,7 @@
 // Parameters and launchers of the persistent N-1 kernel (fdpf.cu).
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace gpcg {
@@ -33,6 +35,7 @@ struct BusTab {
 struct FdpfParams {
   DevGrid G;
   int S = 0, n_tiles = 0;
+  int fill = 0;                // lanes of a tile that take scenarios (at most T)
   ScenInfo sc;
   const double *th0 = nullptr, *V0 = nullptr;  // warm start (bus order)
   const double *c0 = nullptr, *s0 = nullptr;   // cos, sin of th0
@@ -73,13 +76,45 @@ inline bool reduced_form(int precond, const DevMatT<VT>& MP, const DevMatT<VT>& 
   return precond == PREC_EXACT && MP.br.ptr && MQ.br.ptr && !MP.Lh && !MQ.Lh;
 }
 
+// A launch of S scenarios too few to fill the GPU: threads per CTA, CTAs and
+// lanes per tile (tiles of two, reduced inner solves without extension rows).
+// A pass over the rows then lasts as long as its chain of loads times the rows
+// per thread, so the threads that other tiles do not need go to this one; and
+// while there are SMs to spare a tile takes one scenario, which halves the FP64
+// work an SM has to do for it.
+struct WideLaunch {
+  int nt, grid, fill;
+};
+// Dynamic shared memory a wide CTA may take for the vector of its solves (the
+// substitutions' gathers then wait on shared memory): what one CTA of 1,024
+// threads or two of 512 leave of an SM's 227 KB beside their own arrays.
+inline size_t wide_shared(int nt, size_t vec_bytes) {
+  const size_t room = nt == 1024 ? 200u << 10 : nt == 512 ? 88u << 10 : 0;
+  return vec_bytes <= room ? vec_bytes : 0;
+}
+// Grids of fewer rows than threads gain nothing (FP64 solves do from 512: the
+// dense tail's terms are split over the threads).  Kernel times for tolerance
+// 1e-10, CTAs of 256 / 512 / 1,024 threads: 97 outages of a 2,000-bus grid 2.04 /
+// 1.58 / 1.48 ms (one scenario a tile; two: - / 1.76 / 1.65), 300 outages 2.02 / 1.75
+// / 1.65 ms, 600 outages 3.72 / 2.89 / 3.06 ms; 180 outages of 120 buses 1.57 / 1.82 /
+// 2.07 ms; base case of 10,000 buses 16.2 / 12.5 / 11.3 ms.
+inline WideLaunch wide_launch(int S, int num_sms, int rows, bool fp64) {
+  const int most = rows >= 1024 ? 1024 : rows >= 512 || fp64 ? 512 : NTHREADS;
+  const WideLaunch w = S <= num_sms       ? WideLaunch{std::min(1024, most), S, 1}
+                       : S <= 2 * num_sms ? WideLaunch{std::min(1024, most), (S + 1) / 2, 2}
+                       : S <= 4 * num_sms ? WideLaunch{std::min(512, most), (S + 1) / 2, 2}
+                                          : WideLaunch{NTHREADS, 0, 2};
+  return w.nt == NTHREADS ? WideLaunch{NTHREADS, 0, 2} : w;
+}
+
 // The persistent N-1 kernel for tiles of T scenarios (2 to 32; generator
 // outages, P.sc.gen_bus set: 2, 4 or 8) on `grid` slots.  zbytes > 0 (branch
 // outages without reactive limits, T = 2 or 4): each tile's z vector in
 // zbytes of dynamic shared memory, P.wz unused.
 template <typename VT>
 cudaError_t launch_fdpf(cudaStream_t st, int T, int grid, const FdpfParams& P,
-                        const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes = 0);
+                        const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes = 0,
+                        int nt = NTHREADS, size_t wide_bytes = 0);
 template <typename VT>
 int fdpf_max_blocks_per_sm(int T, bool gen, size_t zbytes, bool red);
 // the generator-outage kernel (fdpf_gen.cu)

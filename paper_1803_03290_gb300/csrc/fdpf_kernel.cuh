@@ -62,8 +62,8 @@ __device__ __forceinline__ size_t ef_at(int bus, int lane) {
 
 // I_i = sum_j Y_ij V_j at bus i for lane ln, the lane's outaged branch left
 // out (off the diagonal and its share of it), summed like mismatch_pass.
-template <int T>
-__device__ __forceinline__ double2 bus_current(const DevGrid& G, const LaneState<T>& L,
+template <int T, int NT>
+__device__ __forceinline__ double2 bus_current(const DevGrid& G, const LaneState<T, NT>& L,
                                                const double* __restrict__ EF, int i, int ln) {
   double re = 0.0, im = 0.0;
   const int br = L.l[ln];
@@ -112,14 +112,14 @@ __device__ __forceinline__ double2 bus_current(const DevGrid& G, const LaneState
 // found by one bit test per bus.  What a row needs to know comes in one
 // descriptor and one 16-byte load per neighbour slot, in the order of the
 // visit (BusTab).
-template <int T, typename VT, bool WITH_P, bool GEN>
+template <int T, int NT, typename VT, bool WITH_P, bool GEN>
 __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMatT<VT>& MQ,
-                                               LaneState<T>& L, const double* __restrict__ EF,
+                                               LaneState<T, NT>& L, const double* __restrict__ EF,
                                                VT* __restrict__ rhs,
                                                SwitchState<T>* SW = nullptr) {
-  constexpr int LP = Geo<T>::LP;
+  constexpr int LP = Geo<T, NT>::LP;
   static_assert(LP == 2, "lanes come in pairs");
-  const Geo<T> g;
+  const Geo<T, NT> g;
   const DevGrid& G = P.G;
   const BusTab& tab = WITH_P ? P.tabP : P.tabQ;
   const int nrows = tab.n;
@@ -145,7 +145,7 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
       for (int s = 0; s < SW->nx[ln]; ++s) filt |= 1ull << (SW->xb[ln][s] & 63);
     }
   }
-  for (int kk = g.rs; kk < nrows; kk += Geo<T>::RPS) {
+  for (int kk = g.rs; kk < nrows; kk += Geo<T, NT>::RPS) {
     const int4 d = __ldg(tab.md + kk);
     const int i = d.x;
     const bool on0 = act0 && !in_island(d.y, lo0, cnt0);
@@ -255,10 +255,10 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
         if (j ? w1 : w0) {
           // the base-case state here: the base case is within the reactive limits
           const double dP = redispatched(__ldg(P.r0P + i));
-          upd_max_shared<Geo<T>::TPR == 1>(&L.emax[0][ln], dP);
+          upd_max_shared<Geo<T, NT>::TPR == 1>(&L.emax[0][ln], dP);
           if (bt == 0 || xe) {
             const double q0 = __ldg(P.r0Q + i);
-            upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], xe ? q0 + (qx - qs) : q0);
+            upd_max_shared<Geo<T, NT>::TPR == 1>(&L.emax[1][ln], xe ? q0 + (qx - qs) : q0);
           }
           out.v[j] = to_vt<VT>(dP) * iv;
           continue;
@@ -269,8 +269,8 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
         // dQ = Q_sched - Im(V_i conj(I_i)); dP = P_sched + re-dispatch - Re(...)
         if (WITH_P) {
           const double dP = fma(-ei, re, fma(-fi, im, redispatched(pq.x)));
-          upd_max_shared<Geo<T>::TPR == 1>(&L.emax[0][ln], dP);
-          if (bt == 0 || xe) upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], fma(-fi, re, fma(ei, im, qx)));
+          upd_max_shared<Geo<T, NT>::TPR == 1>(&L.emax[0][ln], dP);
+          if (bt == 0 || xe) upd_max_shared<Geo<T, NT>::TPR == 1>(&L.emax[1][ln], fma(-fi, re, fma(ei, im, qx)));
           if (GEN && bt == 1 && !xe && G.qmax) {
             // a PV generator's output Q(V) - Q_sched = -dQ against its limits:
             // a violation is a candidate for the switch to PQ at that limit
@@ -296,7 +296,7 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
           out.v[j] = to_vt<VT>(dP) * iv;
         } else {
           const double dQ = fma(-fi, re, fma(ei, im, qs));
-          upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], dQ);  // decides whether the Q step is taken
+          upd_max_shared<Geo<T, NT>::TPR == 1>(&L.emax[1][ln], dQ);  // decides whether the Q step is taken
           out.v[j] = to_vt<VT>(dQ) * iv;
         }
       }
@@ -312,10 +312,10 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
       if (!L.active[ln]) continue;
       for (int s = 0; s < SW->nx[ln]; ++s) {
         const int b = SW->xb[ln][s];
-        const double2 I = bus_current<T>(G, L, EF, b, ln);
+        const double2 I = bus_current<T, NT>(G, L, EF, b, ln);
         const double2 v = *reinterpret_cast<const double2*>(EF + ef_at<T>(b, ln));
         const double dQ = fma(-v.y, I.x, fma(v.x, I.y, SW->xq[ln][s]));
-        upd_max_shared<Geo<T>::TPR == 1>(&L.emax[1][ln], dQ);
+        upd_max_shared<Geo<T, NT>::TPR == 1>(&L.emax[1][ln], dQ);
         rhs[(size_t)(MQ.n + 1 + s) * T + ln] = to_vt<VT>(dQ) * inv_vmag<VT>(v.x, v.y);
       }
     }
@@ -370,14 +370,14 @@ __device__ __forceinline__ double v_ratio(VT dv, double e, double f) {
 // is x + xalpha p, the inner solve's deferred last step.  In bus order, so that
 // the state (48 bytes read and written per bus and pair of lanes) streams and
 // only the 8 bytes of x are gathered.
-template <int T, typename VT, bool IS_P, bool GEN>
+template <int T, int NT, typename VT, bool IS_P, bool GEN>
 __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<VT>& M,
-                                             LaneState<T>& L, const VT* __restrict__ x,
+                                             LaneState<T, NT>& L, const VT* __restrict__ x,
                                              const VT* __restrict__ p, double* th, double* EF,
                                              const SwitchState<T>* SW = nullptr,
                                              const double* scale = nullptr) {
-  constexpr int LP = Geo<T>::LP;
-  const Geo<T> g;
+  constexpr int LP = Geo<T, NT>::LP;
+  const Geo<T, NT> g;
   const int l0 = g.lane, l1 = g.lane + 1;
   bool act0 = L.active[l0] != 0, act1 = L.active[l1] != 0;
   const VT xa0 = (VT)(scale ? scale[l0] : L.xalpha[l0]);
@@ -390,7 +390,7 @@ __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<
   const int lo0 = L.lo[l0], cnt0 = L.cnt[l0], lo1 = L.lo[l1], cnt1 = L.cnt[l1];
   const int4* __restrict__ md = IS_P ? P.tabP.md : P.tabQ.md;
   const bool keep_th = IS_P && P.out_theta;
-  for (int kk = g.rs; kk < M.n; kk += Geo<T>::RPS) {
+  for (int kk = g.rs; kk < M.n; kk += Geo<T, NT>::RPS) {
     const int4 d = __ldg(md + kk);
     const bool on0 = act0 && !in_island(d.y, lo0, cnt0);
     const bool on1 = act1 && !in_island(d.y, lo1, cnt1);
@@ -458,9 +458,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Scenario info of a lane taking scenario s (thread `ln`, one per lane).
-template <int T, typename VT>
+template <int T, int NT, typename VT>
 __device__ __forceinline__ void setup_lane(const FdpfParams& P, const DevMatT<VT>& MP,
-                                           const DevMatT<VT>& MQ, LaneState<T>& L, int ln,
+                                           const DevMatT<VT>& MQ, LaneState<T, NT>& L, int ln,
                                            SwitchState<T>* SW) {
   const DevGrid& G = P.G;
   const int s = L.scen[ln];
@@ -528,17 +528,17 @@ __device__ __forceinline__ void setup_lane(const FdpfParams& P, const DevMatT<VT
 
 // Warm start (Sec. III.B) of the lanes flagged `fresh`: the base-case state,
 // zero on islanded buses.  Other lanes keep their state.
-template <int T>
-__device__ GPCG_PASS_INLINE void init_pass(const FdpfParams& P, LaneState<T>& L, double* th,
+template <int T, int NT>
+__device__ GPCG_PASS_INLINE void init_pass(const FdpfParams& P, LaneState<T, NT>& L, double* th,
                                            double* EF) {
-  constexpr int LP = Geo<T>::LP;
-  const Geo<T> g;
+  constexpr int LP = Geo<T, NT>::LP;
+  const Geo<T, NT> g;
   const DevGrid& G = P.G;
   int fresh = 0;
 #pragma unroll
   for (int j = 0; j < LP; ++j) fresh |= (L.fresh[g.lane + j] != 0) << j;
   if (!fresh) return;
-  for (int i = g.rs; i < G.n; i += Geo<T>::RPS) {
+  for (int i = g.rs; i < G.n; i += Geo<T, NT>::RPS) {
     const double2 u = P.flat_start ? make_double2(G.V_set[i], 0.0) : __ldg(P.ef0 + i);
     const double t0 = P.flat_start || !P.out_theta ? 0.0 : P.th0[i];
     const int pr = G.pre[i];
@@ -555,17 +555,17 @@ __device__ GPCG_PASS_INLINE void init_pass(const FdpfParams& P, LaneState<T>& L,
 
 // Outputs of the lanes flagged `done`: state, branch flows and loading
 // (Sec. I: overload screening), status and iteration counts.
-template <int T>
-__device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T>& L,
+template <int T, int NT>
+__device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T, NT>& L,
                                              const double* th, const double* EF) {
-  constexpr int LP = Geo<T>::LP;
-  const Geo<T> g;
+  constexpr int LP = Geo<T, NT>::LP;
+  const Geo<T, NT> g;
   const DevGrid& G = P.G;
   int dn = 0;
 #pragma unroll
   for (int j = 0; j < LP; ++j) dn |= (L.done[g.lane + j] != 0) << j;
   if ((P.out_theta || P.out_vm) && dn) {
-    for (int iu = g.rs; iu < G.n; iu += Geo<T>::RPS) {
+    for (int iu = g.rs; iu < G.n; iu += Geo<T, NT>::RPS) {
       const int i = P.out_bus_map ? __ldg(P.out_bus_map + iu) : iu;
 #pragma unroll
       for (int j = 0; j < LP; ++j) {
@@ -584,14 +584,14 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T>& 
   Vec<int, LP> nov = vzero<int, LP>();  // branches loaded above their rating
   const int nw = (G.m + 31) >> 5;       // words of a scenario's overload mask
   if (P.out_ovmask && dn) {
-    for (int w = g.rs; w < nw; w += Geo<T>::RPS)
+    for (int w = g.rs; w < nw; w += Geo<T, NT>::RPS)
 #pragma unroll
       for (int j = 0; j < LP; ++j)
         if ((dn >> j) & 1) P.out_ovmask[(size_t)L.scen[g.lane + j] * nw + w] = 0u;
     __syncthreads();  // the rows are cleared before any bit is set
   }
   if (dn) {
-    for (int k = g.rs; k < G.m; k += Geo<T>::RPS) {
+    for (int k = g.rs; k < G.m; k += Geo<T, NT>::RPS) {
       const int a = __ldg(G.f + k), b = __ldg(G.t + k);
       const int pa = __ldg(G.pre + a), pb = __ldg(G.pre + b);
       // c^2 g, c g, c b and g, c = 1 / turns ratio at a (1 for a line)
@@ -678,14 +678,17 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T>& 
 // RED: the inner solves in their reduced form (reduced.cuh), for the complete
 // base-case factor: one vector per slot, P.wr.  With extension rows (GEN) the
 // Q solves stay with the PCG over five vectors.
-template <int T, typename VT, bool GEN, bool ZS = false, bool RED = false>
-__global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
+//
+// NT threads a CTA: NTHREADS when the tiles fill the GPU at five CTAs per SM;
+// wide_threads (fdpf.h) says when fewer, wider CTAs take them.
+template <int T, typename VT, bool GEN, bool ZS = false, bool RED = false, int NT = NTHREADS>
+__global__ void __launch_bounds__(NT, ZS ? 2 : NT == NTHREADS ? FDPF_MIN_BLOCKS : 1024 / NT)
     fdpf_tiles_kernel(FdpfParams P_, DevMatT<VT> MP_, DevMatT<VT> MQ_) {
   static_assert(!(ZS && RED), "z is a vector of the PCG");
-  __shared__ LaneState<T> L;
-  RedLanes<T>* RL = nullptr;
+  __shared__ LaneState<T, NT> L;
+  RedLanes<T, NT>* RL = nullptr;
   if constexpr (RED) {
-    __shared__ RedLanes<T> rl;
+    __shared__ RedLanes<T, NT> rl;
     RL = &rl;
   }
   // the parameter blocks in shared memory: the out-of-line passes take them
@@ -709,13 +712,15 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
   const FdpfParams& P = *reinterpret_cast<const FdpfParams*>(pbuf);
   const DevMatT<VT>& MP = *reinterpret_cast<const DevMatT<VT>*>(mbuf[0]);
   const DevMatT<VT>& MQ = *reinterpret_cast<const DevMatT<VT>*>(mbuf[1]);
-  constexpr int LP = Geo<T>::LP;
-  const Geo<T> g;
+  constexpr int LP = Geo<T, NT>::LP;
+  const Geo<T, NT> g;
   VT* x = (VT*)P.wx + (size_t)blockIdx.x * P.vstride;
-  VT* r = (VT*)P.wr + (size_t)blockIdx.x * P.vstride;
+  // (wide CTAs: the solves' vector in dynamic shared memory where it fits)
+  extern __shared__ __align__(16) unsigned char zdyn[];
+  VT* r = NT > NTHREADS && !P.wr ? reinterpret_cast<VT*>(zdyn)
+                                 : (VT*)P.wr + (size_t)blockIdx.x * P.vstride;
   VT* p = (VT*)P.wp + (size_t)blockIdx.x * P.vstride;
   VT* q = (VT*)P.wq + (size_t)blockIdx.x * P.vstride;
-  extern __shared__ __align__(16) unsigned char zdyn[];
   VT* z = ZS ? reinterpret_cast<VT*>(zdyn) : (VT*)P.wz + (size_t)blockIdx.x * P.vstride;
   const size_t so = (size_t)blockIdx.x * P.sstride;
   // E and F regions of the slots taken together: [slot][bus][lane][e, f]
@@ -758,15 +763,15 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
 
   for (;;) {
     // retire finished lanes, then refill empty lanes from the queue
-    if (any_lane<T>(L.done)) retire_pass<T>(P, L, th, EF);
+    if (any_lane<T>(L.done)) retire_pass<T, NT>(P, L, th, EF);
     GPCG_PHASE(7);
     if (tid == 0 && !L.drained) {
       int need = 0;
-      for (int s = 0; s < T; ++s) need += (L.scen[s] < 0);
+      for (int s = 0; s < P.fill; ++s) need += (L.scen[s] < 0);
       if (need) {
         const int base = atomicAdd(P.tile_counter, need);
         int j = 0;
-        for (int s = 0; s < T; ++s) {
+        for (int s = 0; s < P.fill; ++s) {
           if (L.scen[s] >= 0) continue;
           const int qi = base + j++;
           if (qi < P.S) {
@@ -779,11 +784,11 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
     }
     __syncthreads();
     if (tid < T && L.fresh[tid]) {
-      setup_lane<T, VT>(P, MP, MQ, L, tid, SW);
+      setup_lane<T, NT, VT>(P, MP, MQ, L, tid, SW);
       if (tim) P.phase_cycles[8 + 2 * (size_t)L.scen[tid]] = global_ns();
     }
     __syncthreads();
-    init_pass<T>(P, L, th, EF);
+    init_pass<T, NT>(P, L, th, EF);
     __syncthreads();
     if (tid < T) {
       L.fresh[tid] = 0;
@@ -803,7 +808,7 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
       continue;
     }
     // P half-step: mismatch + convergence test
-    mismatch_pass<T, VT, true, GEN>(P, MQ, L, EF, r, SW);
+    mismatch_pass<T, NT, VT, true, GEN>(P, MQ, L, EF, r, SW);
     __syncthreads();
     if (tid < T) {
       {
@@ -891,36 +896,36 @@ __global__ void __launch_bounds__(NTHREADS, ZS ? 2 : FDPF_MIN_BLOCKS)
     const bool more = any_lane<T>(L.active);
     GPCG_PHASE(1);
     if (!more) continue;
-    if (any_stepping<T>(L)) {
+    if (any_stepping(L)) {
       if constexpr (RED) {
-        red_solve<T, VT>(P, MP, L, *RL, r, L.raP, L.rbP, L.inP, L.hold);
+        red_solve<T, NT, VT>(P, MP, L, *RL, r, L.raP, L.rbP, L.inP, L.hold);
         GPCG_PHASE(2);
-        update_pass<T, VT, true, GEN>(P, MP, L, r, nullptr, th, EF, SW, RL->xa);
-      } else {
+        update_pass<T, NT, VT, true, GEN>(P, MP, L, r, nullptr, th, EF, SW, RL->xa);
+      } else if constexpr (NT == NTHREADS) {
         pcg_solve<T, VT, true, GEN>(P, MP, L, x, r, p, q, z, L.raP, L.rbP, L.wP, L.inP, nullptr,
                                     nullptr, L.hold);
         GPCG_PHASE(2);
-        update_pass<T, VT, true, GEN>(P, MP, L, x, p, th, EF, SW);
+        update_pass<T, NT, VT, true, GEN>(P, MP, L, x, p, th, EF, SW);
       }
     }
     __syncthreads();
     GPCG_PHASE(3);
     // Q half-step: the Q mismatch after the P step; a lane whose Q mismatch
     // is within the tolerance takes no Q step
-    mismatch_pass<T, VT, false, GEN>(P, MQ, L, EF, r, SW);
+    mismatch_pass<T, NT, VT, false, GEN>(P, MQ, L, EF, r, SW);
     __syncthreads();
     if (tid < T) L.hold[tid] = from_bits(L.emax[1][tid]) <= P.tol;
     GPCG_PHASE(4);
-    if (any_stepping<T>(L)) {
+    if (any_stepping(L)) {
       if constexpr (RED && !GEN) {
-        red_solve<T, VT>(P, MQ, L, *RL, r, L.raQ, L.rbQ, L.inQ, L.hold);
+        red_solve<T, NT, VT>(P, MQ, L, *RL, r, L.raQ, L.rbQ, L.inQ, L.hold);
         GPCG_PHASE(5);
-        update_pass<T, VT, false, GEN>(P, MQ, L, r, nullptr, th, EF, SW, RL->xa);
-      } else {
+        update_pass<T, NT, VT, false, GEN>(P, MQ, L, r, nullptr, th, EF, SW, RL->xa);
+      } else if constexpr (NT == NTHREADS) {
       pcg_solve<T, VT, true, GEN>(P, MQ, L, x, r, p, q, z, L.raQ, L.rbQ, L.wQ, L.inQ,
                                   MQ.c ? L.cl : nullptr, SW, L.hold);
       GPCG_PHASE(5);
-      update_pass<T, VT, false, GEN>(P, MQ, L, x, p, th, EF, SW);
+      update_pass<T, NT, VT, false, GEN>(P, MQ, L, x, p, th, EF, SW);
       }
     }
     if (g.rs == 0)
@@ -966,9 +971,25 @@ cudaError_t launch_tiles(cudaStream_t st, int T, int grid, const FdpfParams& P,
   return cudaGetLastError();
 }
 
+// Wide CTAs, the solves' vector in wide_bytes of dynamic shared memory (0: in
+// global memory).
+template <typename VT, int NT>
+cudaError_t launch_wide(cudaStream_t st, int grid, const FdpfParams& P, const DevMatT<VT>& MP,
+                        const DevMatT<VT>& MQ, size_t wide_bytes) {
+  auto* k = fdpf_tiles_kernel<2, VT, false, false, true, NT>;
+  if (wide_bytes) {
+    const cudaError_t ce =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide_bytes);
+    if (ce != cudaSuccess) return ce;
+  }
+  k<<<grid, NT, wide_bytes, st>>>(P, MP, MQ);
+  return cudaGetLastError();
+}
+
 template <bool GEN, typename VT>
 cudaError_t launch_fdpf_g(cudaStream_t st, int T, int grid, const FdpfParams& P,
-                          const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes = 0) {
+                          const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes = 0,
+                          int nt = NTHREADS, size_t wide_bytes = 0) {
   if (zbytes) {
     if constexpr (GEN) return cudaErrorInvalidValue;
     else {
@@ -981,6 +1002,11 @@ cudaError_t launch_fdpf_g(cudaStream_t st, int T, int grid, const FdpfParams& P,
         return ce;
       return cudaGetLastError();
     }
+  }
+  if constexpr (!GEN) {
+    if (nt != NTHREADS && T == 2 && reduced_form(P.precond, MP, MQ))
+      return nt == 512 ? launch_wide<VT, 512>(st, grid, P, MP, MQ, wide_bytes)
+                       : launch_wide<VT, 1024>(st, grid, P, MP, MQ, wide_bytes);
   }
   return reduced_form(P.precond, MP, MQ) ? launch_tiles<GEN, VT, true>(st, T, grid, P, MP, MQ)
                                          : launch_tiles<GEN, VT, false>(st, T, grid, P, MP, MQ);

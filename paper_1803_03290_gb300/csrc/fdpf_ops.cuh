@@ -186,11 +186,12 @@ __device__ __forceinline__ void ld_halfs(const __half* p, double (&v)[K]) {
 }
 
 // ------------------------------------------------------------ geometry
-template <int T>
+// NT: threads of the CTA
+template <int T, int NT = NTHREADS>
 struct Geo {
   static constexpr int LP = T < LP_MAX ? T : LP_MAX;  // lanes per thread
   static constexpr int TPR = T / LP;                  // threads per row
-  static constexpr int RPS = NTHREADS / TPR;          // rows per step
+  static constexpr int RPS = NT / TPR;                // rows per step
   int rs, lane;                                       // row slot, first lane
   __device__ Geo() : rs(threadIdx.x / TPR), lane((threadIdx.x % TPR) * LP) {}
 };
@@ -218,7 +219,7 @@ struct SwitchState {
 constexpr int NRED_SITES = 8;   // reduction sites with a buffer of their own
 enum RedSite { RS_BB = 0, RS_RZ0, RS_PQ, RS_RR, RS_RZ, RS_LOAD, RS_RQ, RS_QQ };
 
-template <int T>
+template <int T, int NT = NTHREADS>
 struct LaneState {
   int scen[T], l[T], fb[T], tb[T], lo[T], cnt[T];
   int raP[T], rbP[T], raQ[T], rbQ[T];
@@ -237,7 +238,7 @@ struct LaneState {
   int hold[T];
   double xalpha[T];          // a deferred last step x += alpha p of the inner solve
   // one small buffer per reduction site (see lane_sum): [site][warp][lane]
-  double red2[NRED_SITES * (NTHREADS / 32) * T];
+  double red2[NRED_SITES * (NT / 32) * T];
   // running maxima of |dP| [0] and |dQ| [1] (abs_bits patterns)
   unsigned long long emax[2][T];
   int drained;
@@ -272,8 +273,8 @@ __device__ __forceinline__ Pair<double> lane_reduce(double* red, double v0, doub
 }
 
 // True when some active lane is not held (block-uniform).
-template <int T>
-__device__ __forceinline__ bool any_stepping(const LaneState<T>& L) {
+template <int T, int NT>
+__device__ __forceinline__ bool any_stepping(const LaneState<T, NT>& L) {
   __syncthreads();
   return __syncthreads_or(threadIdx.x < T && L.active[threadIdx.x] != 0 &&
                           L.hold[threadIdx.x] == 0);
@@ -326,11 +327,11 @@ __device__ __forceinline__ double from_bits(unsigned long long b) {
 // Every thread returns the totals of its own lanes.  A site's buffer is
 // read right after the barrier and rewritten only after a later barrier,
 // so consecutive reductions at different sites need no barrier between.
-template <int T, int SITE, typename X, int N>
-__device__ __forceinline__ Vec<X, N> lane_sum(LaneState<T>& L, Vec<X, N> v) {
-  static_assert(N == Geo<T>::LP, "a thread's lanes");
-  const Geo<T> g;
-  constexpr int TPR = Geo<T>::TPR, NW = NTHREADS / 32;
+template <int T, int SITE, typename X, int N, int NT>
+__device__ __forceinline__ Vec<X, N> lane_sum(LaneState<T, NT>& L, Vec<X, N> v) {
+  static_assert(N == Geo<T, NT>::LP, "a thread's lanes");
+  const Geo<T, NT> g;
+  constexpr int TPR = Geo<T, NT>::TPR, NW = NT / 32;
 #pragma unroll
   for (int off = 16; off >= TPR; off >>= 1)
 #pragma unroll
@@ -395,12 +396,12 @@ __device__ __forceinline__ void lane_sum3(LaneState<T>& L, Vec<X, N>& a, Vec<X, 
 }
 
 // The same for running maxima held as abs_bits patterns.
-template <int T, int SITE, int N>
+template <int T, int SITE, int N, int NT>
 __device__ __forceinline__ Vec<unsigned long long, N> lane_max_bits(
-    LaneState<T>& L, Vec<unsigned long long, N> v) {
-  static_assert(N == Geo<T>::LP, "a thread's lanes");
-  const Geo<T> g;
-  constexpr int TPR = Geo<T>::TPR, NW = NTHREADS / 32;
+    LaneState<T, NT>& L, Vec<unsigned long long, N> v) {
+  static_assert(N == Geo<T, NT>::LP, "a thread's lanes");
+  const Geo<T, NT> g;
+  constexpr int TPR = Geo<T, NT>::TPR, NW = NT / 32;
 #pragma unroll
   for (int off = 16; off >= TPR; off >>= 1)
 #pragma unroll

@@ -83,6 +83,14 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   int T = c.opt.tile ? c.opt.tile : (c.tile ? c.tile : 2);
   if (ext) T = std::min(T, 8);
   const bool f32 = c.opt.precision != GPCG_BATCHED_FP64;
+  // the launch gpcg_n1_screen takes for as many scenarios, so that both round
+  // the inner solve alike
+  const bool red = reduced_form(c.opt.precond, c.MPf, c.MQf);
+  WideLaunch wl{NTHREADS, 0, T};
+  if (red && !ext && !c.opt.tile && !c.opt.ctas_per_sm) {
+    wl = wide_launch(n_out, c.num_sms, c.MPf.n, !f32);
+    if (wl.nt != NTHREADS) T = 2;
+  }
   const size_t vt = f32 ? 4 : 8;
   const size_t head = 256;
   const size_t scen = up256(S * 4) * 3 + up256(S * 8);
@@ -90,7 +98,6 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   const size_t st_bytes = up256((size_t)c.n * T * 8);
   // five vectors (one in the reduced form of the inner solve without
   // extension rows); the state theta and e + jf (two arrays' worth)
-  const bool red = reduced_form(c.opt.precond, c.MPf, c.MQf);
   const int nv = red && !ext ? 1 : 5;
   const size_t per_slot = nv * vec_bytes + 3 * st_bytes;
   // what fits is decided on five vectors in either form
@@ -109,8 +116,9 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   if (per_sm <= 0) per_sm = occ;
   per_sm = std::max(per_sm, 1);
   const size_t fit = (cap - head - scen) / per_slot;
+  const bool wide = wl.nt != NTHREADS;
   const int slots = (int)std::max<size_t>(1, std::min<size_t>(
-      fit, (size_t)std::min(n_tiles, c.num_sms * per_sm)));
+      fit, (size_t)(wide ? wl.grid : std::min(n_tiles, c.num_sms * per_sm))));
 
   // validate the outage list through a fixed host buffer
   {
@@ -158,6 +166,7 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   P.out_bus_map = c.bus_of_user;
   P.S = (int)S;
   P.n_tiles = n_tiles;
+  P.fill = wide ? wl.fill : T;
   P.tile_counter = counter;
   const size_t vb = (size_t)slots * vec_bytes, sb = (size_t)slots * st_bytes;
   if (nv == 1) {
@@ -172,8 +181,11 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   (void)sb;
   P.wth = sbase; P.we = sbase + slots * ss; P.wf = sbase + 2 * slots * ss;
   P.sstride = ss;
-  ce = f32 ? launch_fdpf<float>(st, T, slots, P, c.MPf, c.MQf)
-           : launch_fdpf<double>(st, T, slots, P, c.MPd, c.MQd);
+  const size_t vec = (size_t)(std::max(c.MPf.n, c.MQf.n) + 1) * T * vt;
+  const size_t shared = wide_shared(wl.nt, vec);
+  if (shared) P.wr = nullptr;
+  ce = f32 ? launch_fdpf<float>(st, T, slots, P, c.MPf, c.MQf, 0, wl.nt, shared)
+           : launch_fdpf<double>(st, T, slots, P, c.MPd, c.MQd, 0, wl.nt, shared);
   if (ce != cudaSuccess) return err(GPCG_ERR_CUDA, "solve: %s", cudaGetErrorString(ce));
   set_last_error("");
   return GPCG_OK;

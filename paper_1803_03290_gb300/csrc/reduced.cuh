@@ -25,176 +25,277 @@
 
 namespace gpcg {
 
+// The dense products of the tail by CTAs of more than 256 threads: the threads
+// beyond the first 256 take a share of every row's terms (each TAIL_GROUPS-th
+// one), and the first group adds the shares up.
+template <int T, int NT>
+struct TailSplit {
+  static constexpr int RPS = Geo<T, NT>::RPS;
+  static constexpr int GROUPS = RPS > 256 ? RPS / 256 : 1;
+};
+
+// One row of a substitution as its table holds it.
+template <typename VT>
+struct SubRow {
+  int4 rc;
+  int4 c;
+  VT v[SUB_K], id;
+};
+template <typename VT>
+__device__ __forceinline__ SubRow<VT> sub_row(const SubTab<VT>& tab, int e) {
+  SubRow<VT> r;
+  r.rc = __ldg(tab.rc + e);
+  r.c = __ldg(tab.col + e);
+  ld_vals<SUB_K>(tab.val + (size_t)e * SUB_K, r.v);
+  r.id = __ldg(tab.id + e);
+  return r;
+}
+// a - (the row's entries times the solved values), times 1 / L_ii; the first NL
+// lanes of the thread.
+template <int T, int NL, typename VT, int LP>
+__device__ __forceinline__ void sub_apply(const SubRow<VT>& w, const SubTab<VT>& tab,
+                                          const VT* __restrict__ f, int lane, Vec<VT, LP>& a) {
+  const int c[SUB_K] = {w.c.x, w.c.y, w.c.z, w.c.w};
+#pragma unroll
+  for (int k = 0; k < SUB_K; ++k)
+    if (k < w.rc.y) {
+      const Vec<VT, LP> z = ldv<LP>(f + (size_t)c[k] * T + lane);
+#pragma unroll
+      for (int j = 0; j < NL; ++j) a.v[j] -= w.v[k] * z.v[j];
+    }
+  for (int h = w.rc.z, left = w.rc.y - SUB_K; left > 0; ++h, left -= SUB_K) {
+    const int4 cc = __ldg(tab.ccol + h);
+    const int d[SUB_K] = {cc.x, cc.y, cc.z, cc.w};
+    VT v[SUB_K];
+    ld_vals<SUB_K>(tab.cval + (size_t)h * SUB_K, v);
+#pragma unroll
+    for (int k = 0; k < SUB_K; ++k)
+      if (k < left) {
+        const Vec<VT, LP> z = ldv<LP>(f + (size_t)d[k] * T + lane);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) a.v[j] -= v[k] * z.v[j];
+      }
+  }
+#pragma unroll
+  for (int j = 0; j < NL; ++j) a.v[j] *= w.id;
+}
+// Whether a row is loaded a level ahead of its use: in the wide CTAs, whose
+// levels are a row or less per thread and wait on nothing else.
+template <int NT>
+constexpr bool SUB_AHEAD = NT > NTHREADS;
+
 // Forward substitution f = L^-1 r in place over the levels before the tail,
 // and the tail's right-hand side reduced and multiplied by the tail's dense
 // inverse (y into zt).  Adds the lanes' partial |r|^2 to rr and |f|^2 to ff.
-template <int T, typename VT>
+// NL: the thread's lanes that hold a scenario (FP64 solves of a tile with one).
+template <int T, int NT, int NL, typename VT>
 __device__ __forceinline__ void red_forward(const DevMatT<VT>& M, VT* __restrict__ f,
-                                            VT* __restrict__ zt, Vec<VT, Geo<T>::LP>& rr,
-                                            Vec<VT, Geo<T>::LP>& ff) {
-  constexpr int LP = Geo<T>::LP;
-  const Geo<T> g;
-  constexpr int RPS = Geo<T>::RPS, NPT = (TAIL_ROWS + RPS - 1) / RPS;
+                                            VT* __restrict__ zt, Vec<VT, Geo<T, NT>::LP>& rr,
+                                            Vec<VT, Geo<T, NT>::LP>& ff) {
+  constexpr int LP = Geo<T, NT>::LP;
+  const Geo<T, NT> g;
+  constexpr int RPS = Geo<T, NT>::RPS, NPT = (TAIL_ROWS + RPS - 1) / RPS;
   const int nl = M.tail_lev, t0 = M.tail_row0, nt = M.n - t0;
   int r0 = 0, r1 = nl > 0 ? __ldg(M.lev_ptr + 1) : 0;
+  SubRow<VT> nx;
+  int at = -1;
+  if (SUB_AHEAD<NT> && g.rs < r1) nx = sub_row(M.fwd, at = g.rs);
   for (int lev = 0; lev < nl; ++lev) {
     const int r2 = lev + 1 < nl ? __ldg(M.lev_ptr + lev + 2) : r1;
-    for (int i = r0 + g.rs; i < r1; i += RPS) {
-      const size_t o = (size_t)i * T + g.lane;
-      const VT id = __ldg(M.inv_diag + i);
+    for (int e = r0 + g.rs; e < r1; e += RPS) {
+      SubRow<VT> w;
+      if (SUB_AHEAD<NT> && at == e) w = nx;
+      else w = sub_row(M.fwd, e);
+      if (SUB_AHEAD<NT>) {
+        const int ne = e + RPS < r1 ? e + RPS : r1 + g.rs < r2 ? r1 + g.rs : -1;
+        if (ne >= 0) nx = sub_row(M.fwd, at = ne);
+      }
+      const size_t o = (size_t)w.rc.x * T + g.lane;
       Vec<VT, LP> a = ldv<LP>(f + o);
 #pragma unroll
-      for (int j = 0; j < LP; ++j) rr.v[j] += a.v[j] * a.v[j];
-      if (lev > 0) {  // the rows of level 0 have nothing to gather
-        int c[KL];
-        VT v[KL];
-        Vec<VT, LP> zc[KL];
-        ld_cols<KL>(M.L.col + (size_t)i * KL, c);
-        ld_vals<KL>(M.L.val + (size_t)i * KL, v);
-        const int o0 = __ldg(M.L.optr + i), o1 = __ldg(M.L.optr + i + 1);
+      for (int j = 0; j < NL; ++j) rr.v[j] += a.v[j] * a.v[j];
+      sub_apply<T, NL>(w, M.fwd, f, g.lane, a);
 #pragma unroll
-        for (int k = 0; k < KL; ++k) zc[k] = ldv<LP>(f + (size_t)c[k] * T + g.lane);
-#pragma unroll
-        for (int k = 0; k < KL; ++k)
-#pragma unroll
-          for (int j = 0; j < LP; ++j) a.v[j] -= v[k] * zc[k].v[j];
-        for (int e = o0; e < o1; ++e) {
-          const VT vv = __ldg(M.L.oval + e);
-          const Vec<VT, LP> zz = ldv<LP>(f + (size_t)__ldg(M.L.ocol + e) * T + g.lane);
-#pragma unroll
-          for (int j = 0; j < LP; ++j) a.v[j] -= vv * zz.v[j];
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < LP; ++j) {
-        a.v[j] *= id;
-        ff.v[j] += a.v[j] * a.v[j];
-      }
+      for (int j = 0; j < NL; ++j) ff.v[j] += a.v[j] * a.v[j];
       stv<LP>(f + o, a);
     }
+    // a thread without a row in this level: its row of the next one
+    if (SUB_AHEAD<NT> && at < r1 && r1 + g.rs < r2) nx = sub_row(M.fwd, at = r1 + g.rs);
     __syncthreads();
     r0 = r1;
     r1 = r2;
   }
   if (nt <= 0) return;
-  // the tail rows' right-hand side, minus the rows solved before
-  for (int k = g.rs; k < nt; k += RPS) {
-    const int i = t0 + k;
-    int c[KL];
-    VT v[KL];
-    ld_cols<KL>(M.L.col + (size_t)i * KL, c);
-    ld_vals<KL>(M.L.val + (size_t)i * KL, v);
-    Vec<VT, LP> a = ldv<LP>(f + (size_t)i * T + g.lane);
+  // the tail rows' right-hand side, minus the rows solved before: TH threads per
+  // row (the rows have up to dozens of such entries, each a chain of two loads)
+  constexpr int TPR = Geo<T, NT>::TPR, TH = TPR >= 32 ? 1 : 32 / TPR < 8 ? 32 / TPR : 8;
+  const int h = g.rs % TH;
+  for (int k0 = 0; k0 < nt; k0 += RPS / TH) {  // every thread takes part in the sums
+    const int k = k0 + g.rs / TH;
+    Vec<VT, LP> a = vzero<VT, LP>();
+    if (k < nt) {
+      const int e1 = __ldg(M.th_ptr + k + 1);
+      for (int e = __ldg(M.th_ptr + k) + h; e < e1; e += TH) {
+        const VT vv = __ldg(M.th_val + e);
+        const Vec<VT, LP> zz = ldv<LP>(f + (size_t)__ldg(M.th_col + e) * T + g.lane);
 #pragma unroll
-    for (int j = 0; j < LP; ++j) rr.v[j] += a.v[j] * a.v[j];
-#pragma unroll
-    for (int s = 0; s < KL; ++s) {
-      if (c[s] >= t0) continue;
-      const Vec<VT, LP> zz = ldv<LP>(f + (size_t)c[s] * T + g.lane);
-#pragma unroll
-      for (int j = 0; j < LP; ++j) a.v[j] -= v[s] * zz.v[j];
+        for (int j = 0; j < NL; ++j) a.v[j] += vv * zz.v[j];
+      }
     }
-    const int o0 = __ldg(M.L.optr + i), o1 = __ldg(M.L.optr + i + 1);
-    for (int e = o0; e < o1; ++e) {
-      const int cc = __ldg(M.L.ocol + e);
-      if (cc >= t0) continue;
-      const VT vv = __ldg(M.L.oval + e);
-      const Vec<VT, LP> zz = ldv<LP>(f + (size_t)cc * T + g.lane);
 #pragma unroll
-      for (int j = 0; j < LP; ++j) a.v[j] -= vv * zz.v[j];
+    for (int off = TH / 2; off > 0; off >>= 1)
+#pragma unroll
+      for (int j = 0; j < NL; ++j) a.v[j] += __shfl_xor_sync(0xffffffffu, a.v[j], off * TPR);
+    if (k < nt && h == 0) {
+      Vec<VT, LP> r = ldv<LP>(f + (size_t)(t0 + k) * T + g.lane);
+#pragma unroll
+      for (int j = 0; j < NL; ++j) {
+        rr.v[j] += r.v[j] * r.v[j];
+        r.v[j] -= a.v[j];
+      }
+      stv<LP>(zt + (size_t)k * T + g.lane, r);
     }
-    stv<LP>(zt + (size_t)k * T + g.lane, a);
   }
   __syncthreads();
   // y_t = X rhs: X_kj = xc[j nt + k], zero above the diagonal; a warp's rows
   // k are consecutive, so it stops at the diagonal of its last row
-  Vec<VT, LP> y[NPT];
-#pragma unroll
-  for (int m = 0; m < NPT; ++m) {
-    const int k = g.rs + m * RPS;
-    const int jend = min(nt, __shfl_sync(0xffffffffu, k, 31) + 1);  // every lane takes part
-    y[m] = vzero<VT, LP>();
+  constexpr int NG = TailSplit<T, NT>::GROUPS;
+  if constexpr (NG > 1) {
+    __shared__ __align__(16) VT part[NG - 1][TAIL_ROWS * T];
+    const int k = g.rs & 255, q = g.rs >> 8;
+    const int jend = min(nt, __shfl_sync(0xffffffffu, k, 31) + 1);
+    Vec<VT, LP> y = vzero<VT, LP>();
     if (k < nt) {
       const VT* col = M.xc + k;
-#pragma unroll 4
-      for (int j = 0; j < jend; ++j) {
+#pragma unroll 16
+      for (int j = q; j < jend; j += NG) {
         const VT xv = __ldg(col + (size_t)j * nt);
         const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)j * T + g.lane);
 #pragma unroll
-        for (int l = 0; l < LP; ++l) y[m].v[l] += xv * sv.v[l];
+        for (int l = 0; l < NL; ++l) y.v[l] += xv * sv.v[l];
+      }
+      if (q) stv<LP>(part[q - 1] + (size_t)k * T + g.lane, y);
+    }
+    __syncthreads();
+    if (q == 0 && k < nt) {
+#pragma unroll
+      for (int h = 0; h < NG - 1; ++h) {
+        const Vec<VT, LP> u = ldv<LP>(part[h] + (size_t)k * T + g.lane);
+#pragma unroll
+        for (int l = 0; l < NL; ++l) y.v[l] += u.v[l];
       }
 #pragma unroll
-      for (int l = 0; l < LP; ++l) ff.v[l] += y[m].v[l] * y[m].v[l];
+      for (int l = 0; l < NL; ++l) ff.v[l] += y.v[l] * y.v[l];
+      stv<LP>(zt + (size_t)k * T + g.lane, y);
     }
-  }
-  __syncthreads();
+  } else {
+    Vec<VT, LP> y[NPT];
 #pragma unroll
-  for (int m = 0; m < NPT; ++m) {
-    const int k = g.rs + m * RPS;
-    if (k < nt) stv<LP>(zt + (size_t)k * T + g.lane, y[m]);
+    for (int m = 0; m < NPT; ++m) {
+      const int k = g.rs + m * RPS;
+      const int jend = min(nt, __shfl_sync(0xffffffffu, k, 31) + 1);  // every lane takes part
+      y[m] = vzero<VT, LP>();
+      if (k < nt) {
+        const VT* col = M.xc + k;
+#pragma unroll 4
+        for (int j = 0; j < jend; ++j) {
+          const VT xv = __ldg(col + (size_t)j * nt);
+          const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)j * T + g.lane);
+#pragma unroll
+          for (int l = 0; l < NL; ++l) y[m].v[l] += xv * sv.v[l];
+        }
+#pragma unroll
+        for (int l = 0; l < NL; ++l) ff.v[l] += y[m].v[l] * y[m].v[l];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < NPT; ++m) {
+      const int k = g.rs + m * RPS;
+      if (k < nt) stv<LP>(zt + (size_t)k * T + g.lane, y[m]);
+    }
   }
 }
 
 // Backward substitution x = L^-T f in place, the tail first (its y in zt).
-template <int T, typename VT>
+template <int T, int NT, int NL, typename VT>
 __device__ __forceinline__ void red_backward(const DevMatT<VT>& M, VT* __restrict__ f,
                                              const VT* __restrict__ zt) {
-  constexpr int LP = Geo<T>::LP;
-  const Geo<T> g;
-  constexpr int RPS = Geo<T>::RPS, NPT = (TAIL_ROWS + RPS - 1) / RPS;
+  constexpr int LP = Geo<T, NT>::LP;
+  const Geo<T, NT> g;
+  constexpr int RPS = Geo<T, NT>::RPS, NPT = (TAIL_ROWS + RPS - 1) / RPS;
   const int t0 = M.tail_row0, nt = M.n - t0;
   if (nt > 0) {
     // z_t = X^T y_t: X_ik = xr[i nt + k], zero for i < k; a warp starts at
     // the diagonal of its first row
-#pragma unroll
-    for (int m = 0; m < NPT; ++m) {
-      const int k = g.rs + m * RPS;
+    constexpr int NG = TailSplit<T, NT>::GROUPS;
+    if constexpr (NG > 1) {
+      __shared__ __align__(16) VT part[NG - 1][TAIL_ROWS * T];
+      const int k = g.rs & 255, q = g.rs >> 8;
       const int ibeg = __shfl_sync(0xffffffffu, k, 0);
-      if (k >= nt) continue;
-      const VT* col = M.xr + k;
       Vec<VT, LP> a = vzero<VT, LP>();
-#pragma unroll 4
-      for (int i = ibeg; i < nt; ++i) {
-        const VT xv = __ldg(col + (size_t)i * nt);
-        const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)i * T + g.lane);
+      if (k < nt) {
+        const VT* col = M.xr + k;
+#pragma unroll 16
+        for (int i = ibeg + q; i < nt; i += NG) {
+          const VT xv = __ldg(col + (size_t)i * nt);
+          const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)i * T + g.lane);
 #pragma unroll
-        for (int l = 0; l < LP; ++l) a.v[l] += xv * sv.v[l];
+          for (int l = 0; l < NL; ++l) a.v[l] += xv * sv.v[l];
+        }
+        if (q) stv<LP>(part[q - 1] + (size_t)k * T + g.lane, a);
       }
-      stv<LP>(f + (size_t)(t0 + k) * T + g.lane, a);
+      __syncthreads();
+      if (q == 0 && k < nt) {
+#pragma unroll
+        for (int h = 0; h < NG - 1; ++h) {
+          const Vec<VT, LP> u = ldv<LP>(part[h] + (size_t)k * T + g.lane);
+#pragma unroll
+          for (int l = 0; l < NL; ++l) a.v[l] += u.v[l];
+        }
+        stv<LP>(f + (size_t)(t0 + k) * T + g.lane, a);
+      }
+    } else {
+#pragma unroll
+      for (int m = 0; m < NPT; ++m) {
+        const int k = g.rs + m * RPS;
+        const int ibeg = __shfl_sync(0xffffffffu, k, 0);
+        if (k >= nt) continue;
+        const VT* col = M.xr + k;
+        Vec<VT, LP> a = vzero<VT, LP>();
+#pragma unroll 4
+        for (int i = ibeg; i < nt; ++i) {
+          const VT xv = __ldg(col + (size_t)i * nt);
+          const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)i * T + g.lane);
+#pragma unroll
+          for (int l = 0; l < NL; ++l) a.v[l] += xv * sv.v[l];
+        }
+        stv<LP>(f + (size_t)(t0 + k) * T + g.lane, a);
+      }
     }
     __syncthreads();
   }
   const int nb = M.ntblev;
   int r0 = nb > 0 ? __ldg(M.tblev_ptr) : 0, r1 = nb > 0 ? __ldg(M.tblev_ptr + 1) : 0;
+  SubRow<VT> nx;
+  int at = -1;
+  if (SUB_AHEAD<NT> && r0 + g.rs < r1) nx = sub_row(M.bwd, at = r0 + g.rs);
   for (int lev = 0; lev < nb; ++lev) {
     const int r2 = lev + 1 < nb ? __ldg(M.tblev_ptr + lev + 2) : r1;
-    for (int k = r0 + g.rs; k < r1; k += RPS) {
-      const int i = __ldg(M.tblev_rows + k);
-      const size_t o = (size_t)i * T + g.lane;
-      int c[KU];
-      VT v[KU];
-      Vec<VT, LP> zc[KU];
-      ld_cols<KU>(M.U.col + (size_t)i * KU, c);
-      ld_vals<KU>(M.U.val + (size_t)i * KU, v);
-      const int o0 = __ldg(M.U.optr + i), o1 = __ldg(M.U.optr + i + 1);
-      const VT id = __ldg(M.inv_diag + i);
-      Vec<VT, LP> a = ldv<LP>(f + o);
-#pragma unroll
-      for (int s = 0; s < KU; ++s) zc[s] = ldv<LP>(f + (size_t)c[s] * T + g.lane);
-#pragma unroll
-      for (int s = 0; s < KU; ++s)
-#pragma unroll
-        for (int j = 0; j < LP; ++j) a.v[j] -= v[s] * zc[s].v[j];
-      for (int e = o0; e < o1; ++e) {
-        const VT vv = __ldg(M.U.oval + e);
-        const Vec<VT, LP> zz = ldv<LP>(f + (size_t)__ldg(M.U.ocol + e) * T + g.lane);
-#pragma unroll
-        for (int j = 0; j < LP; ++j) a.v[j] -= vv * zz.v[j];
+    for (int e = r0 + g.rs; e < r1; e += RPS) {
+      SubRow<VT> w;
+      if (SUB_AHEAD<NT> && at == e) w = nx;
+      else w = sub_row(M.bwd, e);
+      if (SUB_AHEAD<NT>) {
+        const int ne = e + RPS < r1 ? e + RPS : r1 + g.rs < r2 ? r1 + g.rs : -1;
+        if (ne >= 0) nx = sub_row(M.bwd, at = ne);
       }
-#pragma unroll
-      for (int j = 0; j < LP; ++j) a.v[j] *= id;
+      const size_t o = (size_t)w.rc.x * T + g.lane;
+      Vec<VT, LP> a = ldv<LP>(f + o);
+      sub_apply<T, NL>(w, M.bwd, f, g.lane, a);
       stv<LP>(f + o, a);
     }
+    if (SUB_AHEAD<NT> && at < r1 && r1 + g.rs < r2) nx = sub_row(M.bwd, at = r1 + g.rs);
     __syncthreads();
     r0 = r1;
     r1 = r2;
@@ -240,25 +341,35 @@ __device__ inline int reduced_cg(const RedScalars& q, double tol2, int max_inner
   return its;
 }
 
-template <int T>
+template <int T, int NT = NTHREADS>
 struct RedLanes {
   double vr[T], xa[T];
-  double part[2][NTHREADS / 32][T];  // the warps' partial r.r and |f|^2
+  double part[2][NT / 32][T];  // the warps' partial r.r and |f|^2
 };
 
 // PCG on B_s x = f for the lanes that are active and not held, f in place:
 // on return lane s's solution is S.xa[s] times the vector (xa = 0: no step).
 // Adds each lane's iteration count to iters.
-template <int T, typename VT>
+template <int T, int NT, typename VT>
 __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT>& M,
-                                           LaneState<T>& L, RedLanes<T>& S, VT* f,
+                                           LaneState<T, NT>& L, RedLanes<T, NT>& S, VT* f,
                                            const int* ra, const int* rb, int* iters,
                                            const int* hold) {
-  constexpr int LP = Geo<T>::LP;
-  constexpr int NW = NTHREADS / 32, TPR = Geo<T>::TPR;
+  constexpr int LP = Geo<T, NT>::LP;
+  constexpr int NW = NT / 32, TPR = Geo<T, NT>::TPR;
   __shared__ __align__(16) VT zt[TAIL_ROWS * T];
-  const Geo<T> g;
+  const Geo<T, NT> g;
   const int tid = threadIdx.x, warp = tid >> 5, wl = tid & 31;
+  // diagnostics (P.phase_cycles set): thread 0's SM cycles between the barriers
+  // (recurrence, forward, backward), in the slots after the per-scenario times
+  const bool tim = P.phase_cycles != nullptr && tid == 0;
+  long long tm = tim ? clock64() : 0;
+  auto lap = [&](int k) {
+    if (!tim) return;
+    const long long t = clock64();
+    atomicAdd(P.phase_cycles + 8 + 2 * (size_t)P.S + k, (unsigned long long)(t - tm));
+    tm = t;
+  };
   if (tid < T) {  // v_m.r0, before f is overwritten; the zero row of the padding
     double vr = 0.0;
     if (L.active[tid] && L.l[tid] >= 0) {
@@ -271,7 +382,13 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
   }
   __syncthreads();
   Vec<VT, LP> rr = vzero<VT, LP>(), ff = vzero<VT, LP>();
-  red_forward<T, VT>(M, f, zt, rr, ff);
+  // FP64 solves of a tile with a scenario in its first lane only: half the work
+  // (in the wide CTAs, which take one scenario a tile)
+  constexpr bool MAY_ONE = T == 2 && sizeof(VT) == 8 && NT > NTHREADS;
+  const bool one = MAY_ONE && L.scen[T > 1 ? 1 : 0] < 0;
+  if constexpr (MAY_ONE)
+    if (one) red_forward<T, NT, 1, VT>(M, f, zt, rr, ff);
+  if (!one) red_forward<T, NT, LP, VT>(M, f, zt, rr, ff);
 #pragma unroll
   for (int off = 16; off >= TPR; off >>= 1)
 #pragma unroll
@@ -286,6 +403,7 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
       S.part[1][warp][g.lane + j] = (double)ff.v[j];
     }
   __syncthreads();
+  lap(1);
   // a warp per lane: the sparse dot products, the recurrence, and L^-1 v_m
   // added to the lane's vector
   const int t0 = M.tail_row0;
@@ -293,10 +411,11 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
     double xa = 0.0;
     if (L.active[s] && !(hold && hold[s])) {
       RedScalars q{};
-      double R = 0.0, Z = 0.0;
-      for (int k = 0; k < NW; ++k) {
-        R += S.part[0][k][s];
-        Z += S.part[1][k][s];
+      double R = wl < NW ? S.part[0][wl][s] : 0.0, Z = wl < NW ? S.part[1][wl][s] : 0.0;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        R += __shfl_xor_sync(0xffffffffu, R, off);
+        Z += __shfl_xor_sync(0xffffffffu, Z, off);
       }
       q.R = R;
       q.Z = Z;
@@ -341,8 +460,12 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
     if (wl == 0) S.xa[s] = xa;
   }
   __syncthreads();
-  red_backward<T, VT>(M, f, zt);
+  lap(0);
+  if constexpr (MAY_ONE)
+    if (one) red_backward<T, NT, 1, VT>(M, f, zt);
+  if (!one) red_backward<T, NT, LP, VT>(M, f, zt);
   if (M.ntblev == 0) __syncthreads();
+  lap(2);
 }
 
 }  // namespace gpcg
