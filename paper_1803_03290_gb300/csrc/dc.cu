@@ -200,6 +200,7 @@ __global__ void __launch_bounds__(NTHREADS) dc_base_kernel(DevMatT<double> M, De
   constexpr int T = 2;
   const Geo<T> g;
   __shared__ __align__(16) double zt[TAIL_ROWS * T];
+  __shared__ __align__(16) double part[TAIL_PART<T, NTHREADS>];
   for (int k = g.rs; k <= M.n; k += Geo<T>::RPS) {
     Pair<double> v{0.0, 0.0};
     if (k < M.n) {
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(NTHREADS) dc_base_kernel(DevMatT<double> M, De
   }
   __syncthreads();
   Vec<double, 2> rr = vzero<double, 2>(), ff = vzero<double, 2>();
-  red_forward<T, NTHREADS, 2, double>(M, f, zt, rr, ff);
+  red_forward<T, NTHREADS, 2, double>(M, f, zt, part, rr, ff);
   __syncthreads();
   for (int k = M.tail_row0 + g.rs; k < M.n; k += Geo<T>::RPS)
     st2(f + (size_t)k * T, ld2(zt + (size_t)(k - M.tail_row0) * T));
@@ -222,6 +223,7 @@ __global__ void __launch_bounds__(NTHREADS, FDPF_MIN_BLOCKS)
   constexpr int T = 2;
   __shared__ LaneState<T> L;
   __shared__ __align__(16) double zt[TAIL_ROWS * T];
+  __shared__ __align__(16) double part[TAIL_PART<T, NTHREADS>];
   const Geo<T> g;
   const int tid = threadIdx.x, warp = tid >> 5, wl = tid & 31;
   const DevGrid& G = P.G;
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(NTHREADS, FDPF_MIN_BLOCKS)
       }
     }
     __syncthreads();
-    red_backward<T, NTHREADS, 2, double>(M, f, zt);
+    red_backward<T, NTHREADS, 2, double>(M, f, zt, part);
     if (M.ntblev == 0) __syncthreads();
     // theta in the caller's bus order (slack and islanded buses 0)
     if (D.theta)

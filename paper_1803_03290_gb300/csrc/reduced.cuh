@@ -25,14 +25,52 @@
 
 namespace gpcg {
 
-// The dense products of the tail by CTAs of more than 256 threads: the threads
-// beyond the first 256 take a share of every row's terms (each TAIL_GROUPS-th
-// one), and the first group adds the shares up.
+// The dense products of the tail: the threads are split into as many groups as
+// the tail's rows (rounded up to warps) fit the CTA's row slots, a group takes
+// every groups-th term of each row, and the first one adds the shares up.  TR: X^T
+// (row-major xr, terms from the diagonal of the warp's first row) or X (column-
+// major xc, terms up to the diagonal of the warp's last row); either way
+// consecutive threads read consecutive values.
+template <int T, int NT, int NL, bool TR, typename VT>
+__device__ __forceinline__ bool tail_product(const VT* __restrict__ X, int nt,
+                                             const VT* __restrict__ s, VT* __restrict__ part,
+                                             int& k, Vec<VT, Geo<T, NT>::LP>& a) {
+  constexpr int LP = Geo<T, NT>::LP, RPS = Geo<T, NT>::RPS, UN = NT == 1024 ? 16 : 8;
+  const Geo<T, NT> g;
+  a = vzero<VT, LP>();
+  if constexpr (RPS >= 32 && Geo<T, NT>::TPR == 1) {
+    const int pad = (nt + 31) & ~31, ng = RPS / pad;  // ng >= 1: nt <= 248 < RPS
+    const int q = g.rs / pad;
+    k = g.rs - q * pad;
+    if (q < ng) {  // whole warps
+      const int first = TR ? (k & ~31) + q : q;
+      const int last = TR ? nt : min(nt, (k | 31) + 1);
+      if (k < nt) {
+        const VT* col = X + k;
+#pragma unroll UN
+        for (int j = first; j < last; j += ng) {
+          const VT xv = __ldg(col + (size_t)j * nt);
+          const Vec<VT, LP> sv = ldv<LP>(s + (size_t)j * T + g.lane);
+#pragma unroll
+          for (int l = 0; l < NL; ++l) a.v[l] += xv * sv.v[l];
+        }
+        if (q) stv<LP>(part + ((size_t)(q - 1) * pad + k) * T + g.lane, a);
+      }
+    }
+    __syncthreads();
+    if (q || k >= nt) return false;
+    for (int h = 0; h < ng - 1; ++h) {
+      const Vec<VT, LP> u = ldv<LP>(part + ((size_t)h * pad + k) * T + g.lane);
+#pragma unroll
+      for (int l = 0; l < NL; ++l) a.v[l] += u.v[l];
+    }
+    return true;
+  }
+  return false;
+}
+// Shared memory of the groups' shares.
 template <int T, int NT>
-struct TailSplit {
-  static constexpr int RPS = Geo<T, NT>::RPS;
-  static constexpr int GROUPS = RPS > 256 ? RPS / 256 : 1;
-};
+constexpr int TAIL_PART = Geo<T, NT>::TPR == 1 ? Geo<T, NT>::RPS * T : 1;
 
 // One row of a substitution as its table holds it.
 template <typename VT>
@@ -90,7 +128,8 @@ constexpr bool SUB_AHEAD = NT > NTHREADS;
 // NL: the thread's lanes that hold a scenario (FP64 solves of a tile with one).
 template <int T, int NT, int NL, typename VT>
 __device__ __forceinline__ void red_forward(const DevMatT<VT>& M, VT* __restrict__ f,
-                                            VT* __restrict__ zt, Vec<VT, Geo<T, NT>::LP>& rr,
+                                            VT* __restrict__ zt, VT* __restrict__ part,
+                                            Vec<VT, Geo<T, NT>::LP>& rr,
                                             Vec<VT, Geo<T, NT>::LP>& ff) {
   constexpr int LP = Geo<T, NT>::LP;
   const Geo<T, NT> g;
@@ -157,33 +196,11 @@ __device__ __forceinline__ void red_forward(const DevMatT<VT>& M, VT* __restrict
     }
   }
   __syncthreads();
-  // y_t = X rhs: X_kj = xc[j nt + k], zero above the diagonal; a warp's rows
-  // k are consecutive, so it stops at the diagonal of its last row
-  constexpr int NG = TailSplit<T, NT>::GROUPS;
-  if constexpr (NG > 1) {
-    __shared__ __align__(16) VT part[NG - 1][TAIL_ROWS * T];
-    const int k = g.rs & 255, q = g.rs >> 8;
-    const int jend = min(nt, __shfl_sync(0xffffffffu, k, 31) + 1);
-    Vec<VT, LP> y = vzero<VT, LP>();
-    if (k < nt) {
-      const VT* col = M.xc + k;
-#pragma unroll 16
-      for (int j = q; j < jend; j += NG) {
-        const VT xv = __ldg(col + (size_t)j * nt);
-        const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)j * T + g.lane);
-#pragma unroll
-        for (int l = 0; l < NL; ++l) y.v[l] += xv * sv.v[l];
-      }
-      if (q) stv<LP>(part[q - 1] + (size_t)k * T + g.lane, y);
-    }
-    __syncthreads();
-    if (q == 0 && k < nt) {
-#pragma unroll
-      for (int h = 0; h < NG - 1; ++h) {
-        const Vec<VT, LP> u = ldv<LP>(part[h] + (size_t)k * T + g.lane);
-#pragma unroll
-        for (int l = 0; l < NL; ++l) y.v[l] += u.v[l];
-      }
+  // y_t = X rhs: X_kj = xc[j nt + k], zero above the diagonal
+  if constexpr (TPR == 1) {
+    int k;
+    Vec<VT, LP> y;
+    if (tail_product<T, NT, NL, false>(M.xc, nt, zt, part, k, y)) {
 #pragma unroll
       for (int l = 0; l < NL; ++l) ff.v[l] += y.v[l] * y.v[l];
       stv<LP>(zt + (size_t)k * T + g.lane, y);
@@ -220,41 +237,19 @@ __device__ __forceinline__ void red_forward(const DevMatT<VT>& M, VT* __restrict
 // Backward substitution x = L^-T f in place, the tail first (its y in zt).
 template <int T, int NT, int NL, typename VT>
 __device__ __forceinline__ void red_backward(const DevMatT<VT>& M, VT* __restrict__ f,
-                                             const VT* __restrict__ zt) {
+                                             const VT* __restrict__ zt,
+                                             VT* __restrict__ part) {
   constexpr int LP = Geo<T, NT>::LP;
   const Geo<T, NT> g;
   constexpr int RPS = Geo<T, NT>::RPS, NPT = (TAIL_ROWS + RPS - 1) / RPS;
   const int t0 = M.tail_row0, nt = M.n - t0;
   if (nt > 0) {
-    // z_t = X^T y_t: X_ik = xr[i nt + k], zero for i < k; a warp starts at
-    // the diagonal of its first row
-    constexpr int NG = TailSplit<T, NT>::GROUPS;
-    if constexpr (NG > 1) {
-      __shared__ __align__(16) VT part[NG - 1][TAIL_ROWS * T];
-      const int k = g.rs & 255, q = g.rs >> 8;
-      const int ibeg = __shfl_sync(0xffffffffu, k, 0);
-      Vec<VT, LP> a = vzero<VT, LP>();
-      if (k < nt) {
-        const VT* col = M.xr + k;
-#pragma unroll 16
-        for (int i = ibeg + q; i < nt; i += NG) {
-          const VT xv = __ldg(col + (size_t)i * nt);
-          const Vec<VT, LP> sv = ldv<LP>(zt + (size_t)i * T + g.lane);
-#pragma unroll
-          for (int l = 0; l < NL; ++l) a.v[l] += xv * sv.v[l];
-        }
-        if (q) stv<LP>(part[q - 1] + (size_t)k * T + g.lane, a);
-      }
-      __syncthreads();
-      if (q == 0 && k < nt) {
-#pragma unroll
-        for (int h = 0; h < NG - 1; ++h) {
-          const Vec<VT, LP> u = ldv<LP>(part[h] + (size_t)k * T + g.lane);
-#pragma unroll
-          for (int l = 0; l < NL; ++l) a.v[l] += u.v[l];
-        }
+    // z_t = X^T y_t: X_ik = xr[i nt + k], zero for i < k
+    if constexpr (Geo<T, NT>::TPR == 1) {
+      int k;
+      Vec<VT, LP> a;
+      if (tail_product<T, NT, NL, true>(M.xr, nt, zt, part, k, a))
         stv<LP>(f + (size_t)(t0 + k) * T + g.lane, a);
-      }
     } else {
 #pragma unroll
       for (int m = 0; m < NPT; ++m) {
@@ -358,6 +353,7 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
   constexpr int LP = Geo<T, NT>::LP;
   constexpr int NW = NT / 32, TPR = Geo<T, NT>::TPR;
   __shared__ __align__(16) VT zt[TAIL_ROWS * T];
+  __shared__ __align__(16) VT part[TAIL_PART<T, NT>];
   const Geo<T, NT> g;
   const int tid = threadIdx.x, warp = tid >> 5, wl = tid & 31;
   // diagnostics (P.phase_cycles set): thread 0's SM cycles between the barriers
@@ -387,8 +383,8 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
   constexpr bool MAY_ONE = T == 2 && sizeof(VT) == 8 && NT > NTHREADS;
   const bool one = MAY_ONE && L.scen[T > 1 ? 1 : 0] < 0;
   if constexpr (MAY_ONE)
-    if (one) red_forward<T, NT, 1, VT>(M, f, zt, rr, ff);
-  if (!one) red_forward<T, NT, LP, VT>(M, f, zt, rr, ff);
+    if (one) red_forward<T, NT, 1, VT>(M, f, zt, part, rr, ff);
+  if (!one) red_forward<T, NT, LP, VT>(M, f, zt, part, rr, ff);
 #pragma unroll
   for (int off = 16; off >= TPR; off >>= 1)
 #pragma unroll
@@ -462,8 +458,8 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
   __syncthreads();
   lap(0);
   if constexpr (MAY_ONE)
-    if (one) red_backward<T, NT, 1, VT>(M, f, zt);
-  if (!one) red_backward<T, NT, LP, VT>(M, f, zt);
+    if (one) red_backward<T, NT, 1, VT>(M, f, zt, part);
+  if (!one) red_backward<T, NT, LP, VT>(M, f, zt, part);
   if (M.ntblev == 0) __syncthreads();
   lap(2);
 }
