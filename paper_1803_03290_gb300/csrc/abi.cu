@@ -51,6 +51,9 @@ void launch_branch_cols(cudaStream_t, int, const int32_t*, const int32_t*, const
                         const double*, const int32_t*, const int32_t*, const int32_t*,
                         const int32_t*, int32_t*, double*, double*, double*);
 void launch_flow_values(cudaStream_t, int, const double*, const double*, const double*, double2*);
+void launch_bus_cols(cudaStream_t, int, const int32_t*, const int32_t*, const double*,
+                     const Ell<double>&, int, const double*, const int32_t*, const int32_t*,
+                     double*, double*);
 void launch_gather_pair(cudaStream_t, int, const int4*, const double2*, double2*);
 void launch_ext_rows(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
                      const int32_t*, const double*, const double*, const int32_t*, int32_t*,
@@ -167,6 +170,7 @@ struct MatDev {
   // the branches' columns in the complete factor (null without one)
   int32_t *parent = nullptr, *br_ptr = nullptr, *br_row = nullptr;
   double *br_fv = nullptr, *br_fm = nullptr, *br_sc = nullptr;
+  BusCols bus;  // B'': the buses that can gain a row
   BranchCols cols() const { return BranchCols{br_ptr, br_row, br_fv, br_fm, br_sc}; }
   template <typename VT>
   DevMatT<VT> view(bool f16 = false) const;
@@ -192,6 +196,7 @@ DevMatT<double> MatDev::view<double>(bool) const {
   M.c = c;
   M.xptr = xptr; M.xrow = xrow; M.xval = xval; M.xdiag = xdiag; M.xnb = xnb; M.xbr = xbr;
   M.br = cols();
+  M.bus = bus;
   M.fwd = fwd.view<double>(); M.bwd = bwd.view<double>();
   M.th_ptr = th_ptr; M.th_col = th_col; M.th_val = th_val;
   return M;
@@ -221,6 +226,7 @@ DevMatT<float> MatDev::view<float>(bool f16) const {
   M.c = c;
   M.xptr = xptr; M.xrow = xrow; M.xval = xval32; M.xdiag = xdiag32; M.xnb = xnb; M.xbr = xbr;
   M.br = cols();
+  M.bus = bus;
   M.fwd = fwd.view<float>(); M.bwd = bwd.view<float>();
   M.th_ptr = th_ptr; M.th_col = th_col; M.th_val = th_val32;
   return M;
@@ -731,6 +737,33 @@ static gpcg_status build_matrices(gpcg_ctx* c) {
     M.xbr = c->G.adj_br;
     launch_ext_rows(0, c->n, c->G.adj_ptr, c->G.adj_idx, c->G.adj_br, c->G.f, c->G.cf, c->wQ,
                     M.row_of_bus, M.xrow, M.xval, M.xval32, M.xdiag, M.xdiag32);
+    M.bus = BusCols{};
+    if (M.br_ptr) {  // their columns in the complete factor
+      const MatrixPlan& P = M.plan;
+      std::vector<int32_t> ptr(c->n + 1, 0), row, seen(P.n, -1);
+      for (int b = 0; b < c->n; ++b) {
+        if (c->bus_type[b] == GPCG_PV) {
+          const size_t r0 = row.size();
+          for (int e = c->bg.adj.ptr[b]; e < c->bg.adj.ptr[b + 1]; ++e)
+            for (int i = P.row_of_bus[c->bg.adj.idx[e]]; i >= 0 && seen[i] != b;) {
+              seen[i] = b;
+              row.push_back(i);
+              i = P.U.ptr[i] + 1 < P.U.ptr[i + 1] ? P.U.idx[P.U.ptr[i] + 1] : -1;
+            }
+          std::sort(row.begin() + r0, row.end());
+        }
+        ptr[b + 1] = (int32_t)row.size();
+      }
+      int32_t *d_ptr, *d_row;
+      double *d_f, *d_ff;
+      CUDA_TRY(upload(own, &d_ptr, ptr.data(), ptr.size()));
+      CUDA_TRY(upload(own, &d_row, row.data(), row.size()));
+      CUDA_TRY(dalloc(own, &d_f, row.size()));
+      CUDA_TRY(dalloc(own, &d_ff, (size_t)c->n));
+      launch_bus_cols(0, c->n, c->G.adj_ptr, M.xrow, M.xval, M.U.view<double>(), P.n, M.inv_diag,
+                      d_ptr, d_row, d_f, d_ff);
+      M.bus = BusCols{d_ptr, d_row, d_f, d_ff};
+    }
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaDeviceSynchronize());
   }
@@ -1238,7 +1271,7 @@ struct Layout {
 };
 
 // zs: z in shared memory; one: a single vector per slot (the reduced form of
-// the inner solve without extension rows), at wr
+// the inner solve), at wr
 static Layout make_layout(const gpcg_ctx* c, int T, int slots, size_t vt_size, bool zs = false,
                           bool one = false) {
   Layout L;
@@ -1261,7 +1294,7 @@ static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, i
                             bool f16 = false, bool zs = false, int nt = NTHREADS) {
   const DevMatT<VT> MP = c->MP.view<VT>(f16), MQ = c->MQ.view<VT>(f16);
   const bool red = !zs && reduced_form(P.precond, MP, MQ);
-  const bool one = red && !P.sc.gen_bus && !P.G.qmax;
+  const bool one = red;
   Layout Lo = make_layout(c, T, slots, sizeof(VT), zs, one);
   gpcg_status s = ensure_work(c, Lo.bytes);
   if (s != GPCG_OK) return s;
@@ -1284,7 +1317,8 @@ static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, i
   P.tile_counter = c->d_counter;
   if (!P.fill) P.fill = T;
   const size_t rows = (size_t)std::max(c->MP.plan.n, c->MQ.plan.n) + 1;
-  const size_t wide = one ? wide_shared(nt, rows * T * sizeof(VT)) : 0;
+  const bool plain_rows = !P.sc.gen_bus && !P.G.qmax;  // no extension rows
+  const size_t wide = one && plain_rows ? wide_shared(nt, rows * T * sizeof(VT)) : 0;
   if (wide) P.wr = nullptr;
   CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st));
   CUDA_TRY(launch_fdpf<VT>(st, T, slots, P, MP, MQ, zs ? Lo.vec_bytes : 0, nt, wide));
@@ -1763,7 +1797,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
   } else if (mem == GPCG_MEM_DEVICE && !c->phase_on) {
     // device mode: islanding + solve as one CUDA graph, captured on the
     // context's own stream for this argument set and replayed on `st`
-    Layout Lo = make_layout(c, T, slots, f32 ? 4 : 8, zs, red && !ext && !zs);
+    Layout Lo = make_layout(c, T, slots, f32 ? 4 : 8, zs, red && !zs);
     s_ = ensure_work(c, Lo.bytes);
     if (s_ != GPCG_OK) { cleanup(); return s_; }
     std::vector<uintptr_t> key = {S, (uintptr_t)T, (uintptr_t)slots,

@@ -490,7 +490,7 @@ __global__ void branch_cols_kernel(int m, const int32_t* __restrict__ f,
     fv[e] = i == ra ? c : i == rb ? -1.0 : 0.0;
     fm[e] = i == ra ? ca : i == rb ? cb : 0.0;
   }
-  double vy = 0.0, my = 0.0;
+  double vy = 0.0, my = 0.0, vv = 0.0;
   for (int e = p0; e < p1; ++e) {
     const int j = row[e];
     const double a = fv[e] * inv_diag[j], b = fm[e] * inv_diag[j];
@@ -498,6 +498,7 @@ __global__ void branch_cols_kernel(int m, const int32_t* __restrict__ f,
     fm[e] = b;
     vy = fma(a, b, vy);
     my = fma(b, b, my);
+    vv = fma(a, a, vv);
     auto spread = [&](int k, double v) {
       int x = e + 1, y = p1 - 1;  // row k's place: every k is an ancestor of j
       while (x < y) {
@@ -520,6 +521,57 @@ __global__ void branch_cols_kernel(int m, const int32_t* __restrict__ f,
   o[SC_CA] = ca;
   o[SC_CB] = cb;
   o[SC_W] = w[l];
+  o[SC_VV] = vv;
+}
+
+// L^-1 c_b of the buses with rows in bptr (BusCols), one thread per bus; the
+// couplings from the bus's adjacency (xptr, xrow, xval).
+__global__ void bus_cols_kernel(int nb, const int32_t* __restrict__ xptr,
+                                const int32_t* __restrict__ xrow,
+                                const double* __restrict__ xval, const int32_t* __restrict__ ucol,
+                                const double* __restrict__ uval,
+                                const int32_t* __restrict__ uoptr,
+                                const int32_t* __restrict__ uocol,
+                                const double* __restrict__ uoval, int n,
+                                const double* __restrict__ inv_diag,
+                                const int32_t* __restrict__ ptr, const int32_t* __restrict__ row,
+                                double* f, double* ff) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= nb) return;
+  const int p0 = ptr[b], p1 = ptr[b + 1];
+  double s2 = 0.0;
+  if (p0 < p1) {
+    auto place = [&](int from, int k) {
+      int x = from, y = p1 - 1;
+      while (x < y) {
+        const int mid = (x + y) >> 1;
+        if (row[mid] < k) x = mid + 1; else y = mid;
+      }
+      return x;
+    };
+    for (int e = p0; e < p1; ++e) f[e] = 0.0;
+    for (int e = xptr[b]; e < xptr[b + 1]; ++e)
+      if (xrow[e] >= 0) f[place(p0, xrow[e])] += xval[e];
+    for (int e = p0; e < p1; ++e) {
+      const int j = row[e];
+      const double a = f[e] * inv_diag[j];
+      f[e] = a;
+      s2 = fma(a, a, s2);
+      for (int s = 0; s < KU; ++s) {
+        const int k = ucol[(size_t)j * KU + s];
+        if (k < n) f[place(e + 1, k)] -= uval[(size_t)j * KU + s] * a;
+      }
+      for (int s = uoptr[j]; s < uoptr[j + 1]; ++s) f[place(e + 1, uocol[s])] -= uoval[s] * a;
+    }
+  }
+  ff[b] = s2;
+}
+void launch_bus_cols(cudaStream_t st, int nb, const int32_t* xptr, const int32_t* xrow,
+                     const double* xval, const Ell<double>& U, int n, const double* inv_diag,
+                     const int32_t* ptr, const int32_t* row, double* f, double* ff) {
+  if (nb > 0)
+    bus_cols_kernel<<<nblk(nb, 128), 128, 0, st>>>(nb, xptr, xrow, xval, U.col, U.val, U.optr,
+                                                   U.ocol, U.oval, n, inv_diag, ptr, row, f, ff);
 }
 
 void launch_branch_count(cudaStream_t st, int m, const int32_t* f, const int32_t* t,

@@ -68,13 +68,23 @@ struct Ell {
 // where L^-1 v can be nonzero are the ancestors of its ends in the
 // elimination tree: positions [ptr[l], ptr[l + 1]) of row (ascending), with
 // fv = L^-1 v and fm = L^-1 v_m there.  sc holds SC_N scalars per branch.
-enum { SC_VY = 0, SC_MY, SC_VM2, SC_CA, SC_CB, SC_W, SC_N = 6 };
+enum { SC_VY = 0, SC_MY, SC_VM2, SC_CA, SC_CB, SC_W, SC_VV, SC_N };
 struct BranchCols {
   const int32_t *ptr = nullptr, *row = nullptr;
   const double *fv = nullptr, *fm = nullptr;
   // v.M^-1 v_m, v_m.M^-1 v_m, v_m.v_m, the entries of v_m at the from and the
-  // to end's rows (0: no row, or the island's end), and the branch's weight
+  // to end's rows (0: no row, or the island's end), the branch's weight, and
+  // v.M^-1 v
   const double* sc = nullptr;
+};
+
+// The same for the couplings of the buses that can gain a row of B'' (PV buses:
+// a tripped generator's, or one held at a reactive limit): for bus b the column
+// c_b of its row's off-diagonal entries, f = L^-1 c_b on the rows [ptr[b],
+// ptr[b + 1]), and |f|^2 in ff[b].
+struct BusCols {
+  const int32_t *ptr = nullptr, *row = nullptr;
+  const double *f = nullptr, *ff = nullptr;
 };
 
 // The rows of a substitution in the order it visits them -- level by level,
@@ -134,6 +144,7 @@ struct DevMatT {
   const int32_t* xbr = nullptr;  // the branch of each adjacency entry
   const VT *xval = nullptr, *xdiag = nullptr;
   BranchCols br;  // null pointers: the factor is not the complete one
+  BusCols bus;    // B'' only
   // forward: all levels (lev_ptr); backward: the rows before the tail (tblev_ptr)
   SubTab<VT> fwd, bwd;
   // the tail rows' factor entries on the rows before the tail (CSR by tail row)

@@ -375,7 +375,8 @@ __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<
                                              LaneState<T, NT>& L, const VT* __restrict__ x,
                                              const VT* __restrict__ p, double* th, double* EF,
                                              const SwitchState<T>* SW = nullptr,
-                                             const double* scale = nullptr) {
+                                             const double* scale = nullptr,
+                                             const RedExt<T>* X = nullptr) {
   constexpr int LP = Geo<T, NT>::LP;
   const Geo<T, NT> g;
   const int l0 = g.lane, l1 = g.lane + 1;
@@ -386,7 +387,8 @@ __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<
     act0 = act0 && xa0 != (VT)0;
     act1 = act1 && xa1 != (VT)0;
   }
-  if (!act0 && !act1) return;
+  // (the extension rows' threads stay)
+  if (!act0 && !act1 && !(GEN && !IS_P)) return;
   const int lo0 = L.lo[l0], cnt0 = L.cnt[l0], lo1 = L.lo[l1], cnt1 = L.cnt[l1];
   const int4* __restrict__ md = IS_P ? P.tabP.md : P.tabQ.md;
   const bool keep_th = IS_P && P.out_theta;
@@ -440,9 +442,14 @@ __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<
       if (!L.active[ln]) continue;
       const int b = SW->xb[ln][s];
       const size_t oe = (size_t)(M.n + 1 + s) * T + ln;
-      VT dx = x[oe];
-      const VT xa = (VT)L.xalpha[ln];
-      if (xa != (VT)0) dx = fma(xa, p[oe], dx);
+      VT dx;
+      if (X) {
+        dx = (VT)X->xe[ln][s];
+      } else {
+        dx = x[oe];
+        const VT xa = (VT)L.xalpha[ln];
+        if (xa != (VT)0) dx = fma(xa, p[oe], dx);
+      }
       double2* ef = reinterpret_cast<double2*>(EF + ef_at<T>(b, ln));
       const double2 u = ef[0];
       const double r = v_ratio<VT>(dx, u.x, u.y);
@@ -676,8 +683,7 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T, N
 // CTAs fit an SM, and the register budget is set for two.
 //
 // RED: the inner solves in their reduced form (reduced.cuh), for the complete
-// base-case factor: one vector per slot, P.wr.  With extension rows (GEN) the
-// Q solves stay with the PCG over five vectors.
+// base-case factor: one vector per slot, P.wr.
 //
 // NT threads a CTA: NTHREADS when the tiles fill the GPU at five CTAs per SM;
 // wide_threads (fdpf.h) says when fewer, wider CTAs take them.
@@ -690,6 +696,11 @@ __global__ void __launch_bounds__(NT, ZS ? 2 : NT == NTHREADS ? FDPF_MIN_BLOCKS 
   if constexpr (RED) {
     __shared__ RedLanes<T, NT> rl;
     RL = &rl;
+  }
+  RedExt<T>* RX_ = nullptr;
+  if constexpr (RED && GEN) {
+    __shared__ RedExt<T> rx;
+    RX_ = &rx;
   }
   // the parameter blocks in shared memory: the out-of-line passes take them
   // by reference, so their fields are read from shared memory rather than
@@ -917,10 +928,11 @@ __global__ void __launch_bounds__(NT, ZS ? 2 : NT == NTHREADS ? FDPF_MIN_BLOCKS 
     if (tid < T) L.hold[tid] = from_bits(L.emax[1][tid]) <= P.tol;
     GPCG_PHASE(4);
     if (any_stepping(L)) {
-      if constexpr (RED && !GEN) {
-        red_solve<T, NT, VT>(P, MQ, L, *RL, r, L.raQ, L.rbQ, L.inQ, L.hold);
+      if constexpr (RED) {
+        red_solve<T, NT, VT, GEN>(P, MQ, L, *RL, r, L.raQ, L.rbQ, L.inQ, L.hold, SW, RX_, L.wQ,
+                                  MQ.c ? L.cl : nullptr);
         GPCG_PHASE(5);
-        update_pass<T, NT, VT, false, GEN>(P, MQ, L, r, nullptr, th, EF, SW, RL->xa);
+        update_pass<T, NT, VT, false, GEN>(P, MQ, L, r, nullptr, th, EF, SW, RL->xa, RX_);
       } else if constexpr (NT == NTHREADS) {
       pcg_solve<T, VT, true, GEN>(P, MQ, L, x, r, p, q, z, L.raQ, L.rbQ, L.wQ, L.inQ,
                                   MQ.c ? L.cl : nullptr, SW, L.hold);

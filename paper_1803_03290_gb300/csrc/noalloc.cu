@@ -96,9 +96,8 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   const size_t scen = up256(S * 4) * 3 + up256(S * 8);
   const size_t vec_bytes = up256((size_t)(c.rows + 1) * T * vt);
   const size_t st_bytes = up256((size_t)c.n * T * 8);
-  // five vectors (one in the reduced form of the inner solve without
-  // extension rows); the state theta and e + jf (two arrays' worth)
-  const int nv = red && !ext ? 1 : 5;
+  // five vectors (one in the reduced form of the inner solve); the state theta and e + jf (two arrays' worth)
+  const int nv = red ? 1 : 5;
   const size_t per_slot = nv * vec_bytes + 3 * st_bytes;
   // what fits is decided on five vectors in either form
   const size_t most = 5 * vec_bytes + 3 * st_bytes;

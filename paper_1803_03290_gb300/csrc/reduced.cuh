@@ -336,6 +336,234 @@ __device__ inline int reduced_cg(const RedScalars& q, double tol2, int max_inner
   return its;
 }
 
+// ------------------------------------------------- with extension rows
+// A lane with nx extension rows (B'' rows of switched buses) solves
+//   [ B_s  C ; C^T  D ],  C's columns the couplings c_s, preconditioned by
+//   [ M ; diag D ].
+// The matrix rows' part of every vector then lies in the span of 2 + nx known
+// ones, r0, v_m and the c_s (their M^-1 images for iterates), and the extension
+// rows are coordinates of their own, so the PCG of pcg_solve runs on at most 10
+// + 8 coordinates with
+//   G_ij = rho_i.M^-1 rho_j = f_i.f_j,  N_ij = rho_i.rho_j,  u_i = v.M^-1 rho_i.
+// The f_s = L^-1 c_s are sparse (BusCols; about 20 rows per bus, the PV buses cut
+// B'' into small pieces).  If the outaged branch joins a switched bus to row o,
+// its coupling is not part of c_s: c_s = c_b + k v, as v has only the entry at o.
+constexpr int RX = 2 + KX;  // coordinates on the matrix rows
+template <int T>
+struct RedExt {
+  double G[T][RX][RX], N[T][RX][RX], u[T][RX];
+  double D[T][KX][KX];
+  double k[T][KX];   // c_s = c_b + k v
+  double xe[T][KX];  // right-hand side, then solution on the extension rows
+};
+
+// Couplings of extension row s of lane ln without the outaged branch: visit(row,
+// value) per matrix row, and the branch's own value at row o (bo), if any.
+template <typename VT, typename F>
+__device__ __forceinline__ void ext_couplings(const DevMatT<VT>& M, int b, int lb, F visit) {
+  const int e1 = __ldg(M.xptr + b + 1);
+  for (int e = __ldg(M.xptr + b); e < e1; ++e) {
+    const int rw = __ldg(M.xrow + e);
+    if (rw >= 0 && __ldg(M.xbr + e) != lb) visit(rw, (double)__ldg(M.xval + e));
+  }
+}
+
+// What has to be taken from r0 before the forward pass overwrites it: N_0j, the
+// right-hand side on the extension rows, D and the c_s dot products; thread
+// `ln`, one per lane.
+template <int T, int NT, typename VT>
+__device__ __noinline__ void ext_setup(const DevMatT<VT>& M, const LaneState<T, NT>& L,
+                                       const SwitchState<T>& SW, RedExt<T>& X, const VT* f,
+                                       int ln, int ra, int rb, double w, double c) {
+  const int nx = SW.nx[ln], l = L.l[ln];
+  double ca = 0.0, cb = 0.0;
+  if (l >= 0) {
+    const double* sc = M.br.sc + (size_t)l * SC_N;
+    ca = sc[SC_CA];
+    cb = sc[SC_CB];
+  }
+  for (int s = 0; s < nx; ++s) {
+    const int b = SW.xb[ln][s];
+    X.xe[ln][s] = (double)f[(size_t)(M.n + 1 + s) * T + ln];
+    // v = c e_ra - e_rb has the other end's entry only when b is an end
+    X.k[ln][s] = b == L.fb[ln] ? (rb >= 0 ? -w * c : 0.0) : b == L.tb[ln] ? (ra >= 0 ? w : 0.0) : 0.0;
+    double r0 = 0.0, vm = 0.0;
+    ext_couplings(M, b, l, [&](int rw, double v) {
+      r0 = fma(v, (double)f[(size_t)rw * T + ln], r0);
+      if (rw == ra) vm = fma(v, ca, vm);
+      if (rw == rb) vm = fma(v, cb, vm);
+    });
+    X.N[ln][0][2 + s] = X.N[ln][2 + s][0] = r0;
+    X.N[ln][1][2 + s] = X.N[ln][2 + s][1] = vm;
+    for (int t = 0; t <= s; ++t) {
+      double cc = 0.0, d = 0.0;
+      const int bt = SW.xb[ln][t];
+      ext_couplings(M, b, l, [&](int rw, double v) {
+        ext_couplings(M, bt, l, [&](int rt, double vt) {
+          if (rt == rw) cc = fma(v, vt, cc);
+        });
+      });
+      if (t == s) {
+        // the diagonal without the outaged branch's term
+        d = (double)M.xdiag[b];
+        if (b == L.fb[ln]) d -= w * c * c;
+        else if (b == L.tb[ln]) d -= w;
+      } else {
+        const int e1 = __ldg(M.xptr + b + 1);
+        for (int e = __ldg(M.xptr + b); e < e1; ++e)
+          if (__ldg(M.xnb + e) == bt && __ldg(M.xbr + e) != l) d += (double)__ldg(M.xval + e);
+      }
+      X.N[ln][2 + s][2 + t] = X.N[ln][2 + t][2 + s] = cc;
+      X.D[ln][s][t] = X.D[ln][t][s] = d;
+    }
+  }
+}
+
+// Position of row i in the sorted rows [e0, e1), or -1.
+__device__ __forceinline__ int find_row(const int32_t* __restrict__ row, int e0, int e1, int i) {
+  while (e0 < e1) {
+    const int mid = (e0 + e1) >> 1, r = __ldg(row + mid);
+    if (r == i) return mid;
+    if (r < i) e0 = mid + 1; else e1 = mid;
+  }
+  return -1;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
+// The lane's coordinates and the PCG on them, by one warp (all 32 threads): thread
+// i < 2 + nx holds coordinate i, thread 16 + s the extension row s.  q: the scalars
+// of r0 and v as reduced_cg takes them.  Returns the iterations; on return x is
+// the thread's coordinate of the solution.
+template <int T, int NT, typename VT, typename AT>
+__device__ __noinline__ int ext_solve(const DevMatT<VT>& M, const LaneState<T, NT>& L,
+                                      const SwitchState<T>& SW, RedExt<T>& X,
+                                      const RedScalars& q, int ln, AT at, double tol2,
+                                      int max_inner, double& x) {
+  const int wl = threadIdx.x & 31, nx = SW.nx[ln], K = 2 + nx, l = L.l[ln];
+  auto& G = X.G[ln];
+  auto& N = X.N[ln];
+  double vv = 0.0;
+  int e0 = 0, e1 = 0;
+  if (l >= 0) {
+    vv = __ldg(M.br.sc + (size_t)l * SC_N + SC_VV);
+    e0 = __ldg(M.br.ptr + l);
+    e1 = __ldg(M.br.ptr + l + 1);
+  }
+  if (wl == 0) {
+    G[0][0] = q.Z; G[0][1] = G[1][0] = q.m0; G[1][1] = q.my;
+    N[0][0] = q.R; N[0][1] = N[1][0] = q.vr; N[1][1] = q.vm2;
+    X.u[ln][0] = q.u;
+    X.u[ln][1] = q.vy;
+  }
+  for (int s = 0; s < nx; ++s) {
+    const int b = SW.xb[ln][s], s0 = __ldg(M.bus.ptr + b), s1 = __ldg(M.bus.ptr + b + 1);
+    const double ks = X.k[ln][s];
+    double h = 0.0, a = 0.0, m = 0.0;  // f_b with f0, L^-1 v, L^-1 v_m
+    for (int e = s0 + wl; e < s1; e += 32) {
+      const int i = __ldg(M.bus.row + e);
+      const double fb = __ldg(M.bus.f + e);
+      h = fma(fb, (double)*at(i), h);
+      if (l >= 0) {
+        const int p = find_row(M.br.row, e0, e1, i);
+        if (p >= 0) {
+          a = fma(fb, __ldg(M.br.fv + p), a);
+          m = fma(fb, __ldg(M.br.fm + p), m);
+        }
+      }
+    }
+    h = warp_sum(h);
+    a = warp_sum(a);
+    m = warp_sum(m);
+    if (wl == 0) {
+      G[0][2 + s] = G[2 + s][0] = fma(ks, q.u, h);
+      G[1][2 + s] = G[2 + s][1] = fma(ks, q.vy, m);
+      X.u[ln][2 + s] = fma(ks, vv, a);
+      G[2 + s][2 + s] = __ldg(M.bus.ff + b) + ks * (2.0 * a + ks * vv);
+    }
+    for (int t = 0; t < s; ++t) {
+      const int bt = SW.xb[ln][t], t0 = __ldg(M.bus.ptr + bt), t1 = __ldg(M.bus.ptr + bt + 1);
+      double d = 0.0;
+      for (int e = s0 + wl; e < s1; e += 32) {
+        const int p = find_row(M.bus.row, t0, t1, __ldg(M.bus.row + e));
+        if (p >= 0) d = fma(__ldg(M.bus.f + e), __ldg(M.bus.f + p), d);
+      }
+      d = warp_sum(d);
+      __syncwarp();
+      if (wl == 0) {
+        // f_s.f_t with f_s = f_b + ks fv: u holds v.M^-1 c_t with its own kt
+        const double kt = X.k[ln][t], at_ = X.u[ln][2 + t] - kt * vv;
+        G[2 + s][2 + t] = G[2 + t][2 + s] = d + ks * at_ + kt * a + ks * kt * vv;
+      }
+    }
+    __syncwarp();
+  }
+  __syncwarp();
+  const bool mn = wl < K, ex = wl >= 16 && wl < 16 + nx;
+  const int s = wl - 16;
+  const double gd = ex ? X.D[ln][s][s] : 0.0;
+  auto row_dot = [&](const double (&A)[RX][RX], double v) {  // (A v)_wl
+    double r = 0.0;
+    for (int j = 0; j < K; ++j) {
+      const double vj = __shfl_sync(0xffffffffu, v, j);
+      if (mn) r = fma(A[wl][j], vj, r);
+    }
+    return r;
+  };
+  double r = mn ? (wl == 0 ? 1.0 : 0.0) : ex ? X.xe[ln][s] : 0.0;
+  x = 0.0;
+  auto pre = [&](double v) { return ex ? (gd > 0.0 ? v / gd : 0.0) : v; };
+  const double n0 = row_dot(N, r);  // (every thread takes part in the shuffles)
+  const double bb = warp_sum(mn ? r * n0 : r * r);
+  double z = pre(r);
+  double gz = row_dot(G, z);
+  double rz = warp_sum(mn ? r * gz : r * z);
+  if (!(bb > 0.0) || !(rz > 0.0)) return 0;
+  double p = z, best = bb;
+  int its = 0, stall = 0;
+  while (its < max_inner) {
+    // q = B_ext p: main coordinates, and the extension rows
+    const double gp = row_dot(G, p);
+    double up = 0.0, qe = 0.0;
+    for (int j = 0; j < K; ++j) {
+      const double pj = __shfl_sync(0xffffffffu, p, j);
+      up = fma(X.u[ln][j], pj, up);
+      if (ex) qe = fma(G[2 + s][j], pj, qe);
+    }
+    for (int t = 0; t < nx; ++t) {
+      const double pt = __shfl_sync(0xffffffffu, p, 16 + t);
+      if (ex) qe = fma(X.D[ln][s][t], pt, qe);
+    }
+    const double pe = __shfl_sync(0xffffffffu, p, wl >= 2 && wl < K ? 14 + wl : 31);
+    double qv = mn ? p : ex ? qe : 0.0;
+    if (wl == 1) qv -= q.w * up;
+    if (mn && wl >= 2) qv += pe;
+    const double pq = warp_sum(mn ? qv * gp : ex ? p * qv : 0.0);
+    if (!(pq > 0.0) || !isfinite(pq)) break;
+    const double al = rz / pq;
+    x = fma(al, p, x);
+    r = fma(-al, qv, r);
+    ++its;
+    const double nr = row_dot(N, r);
+    const double rr = warp_sum(mn ? r * nr : ex ? r * r : 0.0);
+    if (!(rr > tol2 * bb) || !isfinite(rr)) break;
+    if (rr < 0.999 * best) { best = rr; stall = 0; }
+    else if (++stall >= STALL_ITERS) break;
+    if (rr > 1e4 * best) break;
+    z = pre(r);
+    gz = row_dot(G, z);
+    const double rzn = warp_sum(mn ? r * gz : ex ? r * z : 0.0);
+    if (!(rzn > 0.0)) break;
+    const double be = rzn / rz;
+    rz = rzn;
+    p = fma(be, p, z);
+  }
+  return its;
+}
+
 template <int T, int NT = NTHREADS>
 struct RedLanes {
   double vr[T], xa[T];
@@ -345,11 +573,16 @@ struct RedLanes {
 // PCG on B_s x = f for the lanes that are active and not held, f in place:
 // on return lane s's solution is S.xa[s] times the vector (xa = 0: no step).
 // Adds each lane's iteration count to iters.
-template <int T, int NT, typename VT>
+//
+// EXT: lanes may have extension rows (SW, X; w, c: the lanes' branch weights and
+// from-end factors); their solution is left in X.xe.
+template <int T, int NT, typename VT, bool EXT = false>
 __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT>& M,
                                            LaneState<T, NT>& L, RedLanes<T, NT>& S, VT* f,
                                            const int* ra, const int* rb, int* iters,
-                                           const int* hold) {
+                                           const int* hold, const SwitchState<T>* SW = nullptr,
+                                           RedExt<T>* X = nullptr, const double* w = nullptr,
+                                           const double* c = nullptr) {
   constexpr int LP = Geo<T, NT>::LP;
   constexpr int NW = NT / 32, TPR = Geo<T, NT>::TPR;
   __shared__ __align__(16) VT zt[TAIL_ROWS * T];
@@ -375,6 +608,9 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
     }
     S.vr[tid] = vr;
     f[(size_t)M.n * T + tid] = (VT)0;
+    if constexpr (EXT)
+      if (L.active[tid] && SW->nx[tid] > 0)
+        ext_setup<T, NT>(M, L, *SW, *X, f, tid, ra[tid], rb[tid], w[tid], c ? c[tid] : 1.0);
   }
   __syncthreads();
   Vec<VT, LP> rr = vzero<VT, LP>(), ff = vzero<VT, LP>();
@@ -441,6 +677,41 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
         q.u = u;
         q.m0 = m0;
       }
+      auto place = [&](int i) {
+        return i < t0 ? f + (size_t)i * T + s : zt + (size_t)(i - t0) * T + s;
+      };
+      bool done = false;
+      if constexpr (EXT) {
+        const int nx = SW->nx[s];
+        if (nx > 0) {
+          done = true;
+          double x;
+          const int its = ext_solve<T, NT>(M, L, *SW, *X, q, s, place,
+                                           P.inner_rtol * P.inner_rtol, P.max_inner, x);
+          xa = __shfl_sync(0xffffffffu, x, 0);
+          const double xv = __shfl_sync(0xffffffffu, x, 1);
+          if (wl >= 16 && wl < 16 + nx) X->xe[s][wl - 16] = x;
+          if (xa != 0.0) {
+            double kv = 0.0;  // the c_s' share of v
+            for (int k = 0; k < nx; ++k) {
+              const double xs = __shfl_sync(0xffffffffu, x, 2 + k) / xa;
+              kv = fma(xs, X->k[s][k], kv);
+              const int b = SW->xb[s][k], b1 = __ldg(M.bus.ptr + b + 1);
+              for (int e = __ldg(M.bus.ptr + b) + wl; e < b1; e += 32) {
+                VT* y = place(__ldg(M.bus.row + e));
+                *y = (VT)fma(xs, __ldg(M.bus.f + e), (double)*y);
+              }
+              __syncwarp();
+            }
+            for (int e = e0 + wl; e < e1; e += 32) {
+              VT* y = place(__ldg(M.br.row + e));
+              *y = (VT)fma(xv / xa, __ldg(M.br.fm + e), fma(kv, __ldg(M.br.fv + e), (double)*y));
+            }
+          }
+          if (wl == 0) iters[s] += its;
+        }
+      }
+      if (!done) {
       double xb;
       const int its = reduced_cg(q, P.inner_rtol * P.inner_rtol, P.max_inner, xa, xb);
       if (xa != 0.0 && xb != 0.0) {
@@ -452,7 +723,10 @@ __device__ GPCG_PASS_INLINE void red_solve(const FdpfParams& P, const DevMatT<VT
         }
       }
       if (wl == 0) iters[s] += its;
+      }
     }
+    if constexpr (EXT)
+      if (xa == 0.0 && wl < KX) X->xe[s][wl] = 0.0;  // no step
     if (wl == 0) S.xa[s] = xa;
   }
   __syncthreads();
