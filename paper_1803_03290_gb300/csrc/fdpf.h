@@ -96,13 +96,16 @@ inline size_t wide_shared(int nt, size_t vec_bytes) {
 // dense tail's terms are split over the threads).  Kernel times for tolerance
 // 1e-10, CTAs of 256 / 512 / 1,024 threads: 97 outages of a 2,000-bus grid 2.04 /
 // 1.58 / 1.48 ms (one scenario a tile; two: - / 1.76 / 1.65), 300 outages 2.02 / 1.75
-// / 1.65 ms, 600 outages 3.72 / 2.89 / 3.06 ms; 180 outages of 120 buses 1.57 / 1.82 /
+// / 1.65 ms, 600 outages 3.72 / 2.89 / 3.06 ms, 1,000 outages 4.04 / 3.46 / 4.98 ms,
+// 2,700 outages 6.9 / 8.1 / 12.1 ms; 10,000 buses, 1,000 outages 16.1 / 13.7 / 16.3 ms,
+// 1,500 outages 18.2 / 20.1 / 23.2 ms; 180 outages of 120 buses 1.57 / 1.82 /
 // 2.07 ms; base case of 10,000 buses 16.2 / 12.5 / 11.3 ms.
 inline WideLaunch wide_launch(int S, int num_sms, int rows, bool fp64) {
   const int most = rows >= 1024 ? 1024 : rows >= 512 || fp64 ? 512 : NTHREADS;
   const WideLaunch w = S <= num_sms       ? WideLaunch{std::min(1024, most), S, 1}
                        : S <= 2 * num_sms ? WideLaunch{std::min(1024, most), (S + 1) / 2, 2}
-                       : S <= 4 * num_sms ? WideLaunch{std::min(512, most), (S + 1) / 2, 2}
+                       : S <= 8 * num_sms
+                           ? WideLaunch{std::min(512, most), std::min((S + 1) / 2, 2 * num_sms), 2}
                                           : WideLaunch{NTHREADS, 0, 2};
   return w.nt == NTHREADS ? WideLaunch{NTHREADS, 0, 2} : w;
 }

@@ -588,13 +588,19 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T, N
     }
   }
   Vec<unsigned long long, LP> ml = vzero<unsigned long long, LP>();  // abs_bits patterns
+  // screening without flows: the lanes' maxima so far as lower bounds in FP32,
+  // shared by the CTA (see below)
+  const bool screen = !P.out_flow;
+  if (threadIdx.x < T) L.seen[threadIdx.x] = 0u;
+  __syncthreads();
   Vec<int, LP> nov = vzero<int, LP>();  // branches loaded above their rating
   const int nw = (G.m + 31) >> 5;       // words of a scenario's overload mask
-  if (P.out_ovmask && dn) {
-    for (int w = g.rs; w < nw; w += Geo<T, NT>::RPS)
+  if (P.out_ovmask) {  // (uniform: the threads of a warp may hold different lanes)
+    if (dn)
+      for (int w = g.rs; w < nw; w += Geo<T, NT>::RPS)
 #pragma unroll
-      for (int j = 0; j < LP; ++j)
-        if ((dn >> j) & 1) P.out_ovmask[(size_t)L.scen[g.lane + j] * nw + w] = 0u;
+        for (int j = 0; j < LP; ++j)
+          if ((dn >> j) & 1) P.out_ovmask[(size_t)L.scen[g.lane + j] * nw + w] = 0u;
     __syncthreads();  // the rows are cleared before any bit is set
   }
   if (dn) {
@@ -616,7 +622,43 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T, N
           if (!((dn >> j) & 1)) continue;
           const int lo = L.lo[ln], cnt = L.cnt[ln];
           double Pab = 0.0;
-          if (k != L.l[ln] && !in_island(pa, lo, cnt) && !in_island(pb, lo, cnt)) {
+          bool on = k != L.l[ln] && !in_island(pa, lo, cnt) && !in_island(pb, lo, cnt);
+          if (screen && on) {
+            // The loading is only compared -- with 1 and with the largest so
+            // far.  Its FP32 value with a bound on its error settles both for
+            // all but a few branches, which are then evaluated in FP64; the
+            // results are those of FP64 for every branch.  Each of the products
+            // below has at most 8 roundings of 2^-24 of its magnitude, and so
+            // has their sum: err = 2^-20 (|c^2 g| + |g|, |c g|, |c b|) times the
+            // voltages' magnitudes covers it twice.
+            const float ea = to_f32(va[h].x), fa = to_f32(va[h].y);
+            const float eb = to_f32(vb[h].x), fb = to_f32(vb[h].y);
+            const float ga = to_f32(y0.x), gc = to_f32(y0.y), bc = to_f32(y1.x), gb = to_f32(y1.y);
+            const float irf = to_f32(ir);
+            const float a2 = fmaf(ea, ea, fa * fa), b2 = fmaf(eb, eb, fb * fb);
+            const float cr = gc * fmaf(ea, eb, fa * fb), sr = bc * fmaf(fa, eb, -ea * fb);
+            const float pab = fabsf(fmaf(ga, a2, -(cr + sr))), pba = fabsf(fmaf(gb, b2, sr - cr));
+            const float mag = a2 + b2;
+            const float err = 9.5367432e-7f *
+                              (fmaf(fabsf(ga), a2, fabsf(gb) * b2) +
+                               mag * (fabsf(gc) + fabsf(bc))) * irf;
+            const float ldf = fmaxf(pab, pba) * irf, lower = ldf - err, upper = ldf + err;
+            const bool sure = upper < 1.0f || lower > 1.0f;
+            // (a NaN compares false and goes the FP64 way)
+            const float seen = __uint_as_float(
+                *reinterpret_cast<const volatile unsigned*>(&L.seen[ln]));
+            if (sure && (!P.out_maxload || upper < seen)) {
+              on = false;
+              if (lower > 1.0f) {
+                nov.v[j] += 1;
+                if (P.out_ovmask)
+                  atomicOr(P.out_ovmask + (size_t)L.scen[ln] * nw + (k >> 5), 1u << (k & 31));
+              }
+            } else if (P.out_maxload && lower > seen) {
+              atomicMax(&L.seen[ln], __float_as_uint(lower));
+            }
+          }
+          if (on) {
             // P_ab = c^2 g |V_a|^2 - c (g Re(V_a conj V_b) + b Im(V_a conj V_b)),
             // P_ba = g |V_b|^2 - c (g Re(V_a conj V_b) - b Im(V_a conj V_b)),
             // c = 1 / turns ratio at a (the pi-model sees V_a c)

@@ -242,6 +242,7 @@ struct LaneState {
   // running maxima of |dP| [0] and |dQ| [1] (abs_bits patterns)
   unsigned long long emax[2][T];
   int drained;
+  unsigned seen[T];  // retire_pass: lower bounds of the maximum loading (FP32 bits)
 };
 
 // Sum (or max) over the row slots of each lane's partial values, for
