@@ -31,6 +31,9 @@ void launch_laplacian_values(cudaStream_t, int, const int32_t*, const int32_t*, 
                              const double*, const int32_t*, const int32_t*, double*, int32_t*);
 void launch_ic_level(cudaStream_t, int, int, const int32_t*, const int32_t*, const double*,
                      const int32_t*, const int32_t*, double*, int32_t*);
+void launch_ic_narrow(cudaStream_t, const int32_t*, int, int, const int32_t*, const int32_t*,
+                      const double*, const int32_t*, const int32_t*, double*, int32_t*);
+int ic_narrow_rows();
 void launch_scatter(cudaStream_t, int, const int32_t*, const double*, double*);
 void launch_to_float(cudaStream_t, int, const double*, float*);
 void launch_gather_diag(cudaStream_t, int, const int32_t*, const double*, double*);
@@ -560,9 +563,20 @@ static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w) {
   CUDA_TRY(cudaMemset(c->d_err, 0, sizeof(int32_t)));
   launch_laplacian_values(st, P.n, M.bus_of_row, M.row_of_bus, c->G.adj_ptr, c->G.adj_idx,
                           c->G.adj_br, w, c->G.f, M.c, M.a_ptr, M.a_idx, M.a_val, c->d_err);
-  for (size_t k = 0; k + 1 < P.lev_ptr.size(); ++k)
-    launch_ic_level(st, P.lev_ptr[k], P.lev_ptr[k + 1], M.a_ptr, M.a_idx, M.a_val, M.l_ptr,
-                    M.l_idx, M.l_val, c->d_err);
+  // wide levels one launch each, runs of narrow ones one launch together
+  for (int k = 0, nl = (int)P.lev_ptr.size() - 1; k < nl;) {
+    int e = k;
+    while (e < nl && P.lev_ptr[e + 1] - P.lev_ptr[e] <= ic_narrow_rows()) ++e;
+    if (e > k) {
+      launch_ic_narrow(st, M.lev_ptr, k, e, M.a_ptr, M.a_idx, M.a_val, M.l_ptr, M.l_idx, M.l_val,
+                       c->d_err);
+      k = e;
+    } else {
+      launch_ic_level(st, P.lev_ptr[k], P.lev_ptr[k + 1], M.a_ptr, M.a_idx, M.a_val, M.l_ptr,
+                      M.l_idx, M.l_val, c->d_err);
+      ++k;
+    }
+  }
   launch_gather_diag(st, P.n, M.a_diag, M.a_val, M.diag);
   launch_to_float(st, P.n, M.diag, M.diag32);
   launch_inv_diag(st, P.n, M.l_diag, M.l_val, M.inv_diag, M.inv_diag32);

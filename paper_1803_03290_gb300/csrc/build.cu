@@ -183,6 +183,52 @@ __global__ void ic_level_kernel(int row0, int row1, const int32_t* __restrict__ 
   }
 }
 
+// The narrow levels [lev0, lev1) in one launch of one CTA, a warp per row: a
+// launch per level (67 on a 2,000-bus grid) and a thread walking both rows of
+// every product one entry at a time took most of a re-factorisation.  The row's
+// entries are computed in order; the sum over the columns rows i and j share has
+// its terms spread over the warp (each looks the column of row j up in row i).
+constexpr int IC_NARROW = 512;  // rows of a level, at most
+__global__ void __launch_bounds__(1024)
+    ic_narrow_kernel(const int32_t* __restrict__ lev_ptr, int lev0, int lev1,
+                     const int32_t* __restrict__ a_ptr, const int32_t* __restrict__ a_idx,
+                     const double* __restrict__ a_val, const int32_t* __restrict__ l_ptr,
+                     const int32_t* __restrict__ l_idx, double* l_val, int32_t* err) {
+  const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
+  for (int lev = lev0; lev < lev1; ++lev) {
+    const int r1 = lev_ptr[lev + 1];
+    for (int i = lev_ptr[lev] + warp; i < r1; i += 32) {
+      const int ls = l_ptr[i], le = l_ptr[i + 1];
+      for (int k = ls; k < le; ++k) {
+        const int j = l_idx[k], q0 = l_ptr[j], q1 = l_ptr[j + 1] - 1;
+        double s = 0.0;
+        for (int q = q0 + wl; q < q1; q += 32) {
+          const int c = l_idx[q];
+          int lo = ls, hi = k;  // row i's entries before k
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (l_idx[mid] < c) lo = mid + 1; else hi = mid;
+          }
+          if (lo < k && l_idx[lo] == c) s = fma(l_val[lo], l_val[q], s);
+        }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (wl == 0) {
+          s = csr_lookup(a_idx, a_val, a_ptr[i], a_ptr[i + 1], j) - s;
+          if (j < i) {
+            l_val[k] = s / l_val[q1];
+          } else {
+            if (!(s > 0.0)) { atomicExch(err, 2); s = 1.0; }
+            l_val[k] = sqrt(s);
+          }
+        }
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+  }
+}
+
 __global__ void scatter_kernel(int nnz, const int32_t* __restrict__ map,
                                const double* __restrict__ src, double* dst) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -238,6 +284,14 @@ void launch_ic_level(cudaStream_t st, int row0, int row1, const int32_t* a_ptr,
     ic_level_kernel<<<nblk(n, 128), 128, 0, st>>>(row0, row1, a_ptr, a_idx, a_val, l_ptr,
                                                   l_idx, l_val, err);
 }
+void launch_ic_narrow(cudaStream_t st, const int32_t* lev_ptr, int lev0, int lev1,
+                      const int32_t* a_ptr, const int32_t* a_idx, const double* a_val,
+                      const int32_t* l_ptr, const int32_t* l_idx, double* l_val, int32_t* err) {
+  if (lev1 > lev0)
+    ic_narrow_kernel<<<1, 1024, 0, st>>>(lev_ptr, lev0, lev1, a_ptr, a_idx, a_val, l_ptr, l_idx,
+                                         l_val, err);
+}
+int ic_narrow_rows() { return IC_NARROW; }
 void launch_scatter(cudaStream_t st, int nnz, const int32_t* map, const double* src,
                     double* dst) {
   if (nnz) scatter_kernel<<<nblk(nnz, 256), 256, 0, st>>>(nnz, map, src, dst);
@@ -332,39 +386,46 @@ void launch_inv_diag(cudaStream_t st, int n, const int32_t* pos, const double* l
 }
 // X = inverse of the factor's tail block L_tt (rows and columns
 // [t0, t0 + nt) of L, lower triangular): column c of X by forward
-// substitution of L_tt x = e_c, one thread per column, in FP64.  Written
-// column-major (xc[c nt + i] = X_ic) and row-major (xr[i nt + c] = X_ic),
-// zeros above the diagonal, in FP64 (xr optional) and FP32.
+// substitution of L_tt x = e_c in FP64, a warp per column with the row's
+// terms spread over its threads (a thread per column in one CTA took 1 ms for
+// 232 rows: each term waited for its own loads).  Written column-major
+// (xc[c nt + i] = X_ic) and row-major (xr[i nt + c] = X_ic), zeros above the
+// diagonal, in FP64 (xr optional) and FP32.
 // With lsc (the scaled factor Ls = L D^-1) the block inverted is the one
 // the FP16 storage represents: L_ij = fp16(Ls_ij) L_jj.
-__global__ void tail_inverse_kernel(int t0, int nt, const int32_t* __restrict__ l_ptr,
-                                    const int32_t* __restrict__ l_idx,
-                                    const double* __restrict__ l_val,
-                                    const double* __restrict__ lsc, double* xc, double* xr,
-                                    float* xc32, float* xr32) {
-  for (int c = threadIdx.x; c < nt; c += blockDim.x) {
-    // xc holds the column in FP64 while it is built (its earlier entries
-    // are the unknowns solved before)
-    for (int i = 0; i < nt; ++i) {
-      double v = 0.0;
-      if (i >= c) {
-        const int R = t0 + i, e0 = l_ptr[R], e1 = l_ptr[R + 1] - 1;  // diagonal last
-        double sum = (i == c) ? 1.0 : 0.0;
-        for (int e = e0; e < e1; ++e) {
-          const int jg = l_idx[e], j = jg - t0;
-          if (j < c) continue;
-          const double lij =
-              lsc ? (double)__half2float(__double2half(lsc[e])) * l_val[l_ptr[jg + 1] - 1]
-                  : l_val[e];
-          sum -= lij * xc[(size_t)c * nt + j];
-        }
-        v = sum / l_val[e1];
-      }
-      xc[(size_t)c * nt + i] = v;
-      if (xr) xr[(size_t)i * nt + c] = v;
-      xc32[(size_t)c * nt + i] = (float)v;
-      xr32[(size_t)i * nt + c] = (float)v;
+constexpr int TI_WARPS = 4;
+__global__ void __launch_bounds__(32 * TI_WARPS)
+    tail_inverse_kernel(int t0, int nt, const int32_t* __restrict__ l_ptr,
+                        const int32_t* __restrict__ l_idx, const double* __restrict__ l_val,
+                        const double* __restrict__ lsc, double* xc, double* xr, float* xc32,
+                        float* xr32) {
+  __shared__ double col[TI_WARPS][TAIL_ROWS];
+  const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
+  const int c = blockIdx.x * TI_WARPS + warp;
+  if (c >= nt) return;
+  double* x = col[warp];
+  for (int i = wl; i < c; i += 32) x[i] = 0.0;
+  for (int i = c; i < nt; ++i) {
+    const int R = t0 + i, e0 = l_ptr[R], e1 = l_ptr[R + 1] - 1;  // diagonal last
+    double s = 0.0;
+    for (int e = e0 + wl; e < e1; e += 32) {
+      const int jg = l_idx[e], j = jg - t0;
+      if (j < c) continue;
+      const double lij =
+          lsc ? (double)__half2float(__double2half(lsc[e])) * l_val[l_ptr[jg + 1] - 1] : l_val[e];
+      s = fma(lij, x[j], s);
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (wl == 0) x[i] = ((i == c ? 1.0 : 0.0) - s) / l_val[e1];
+    __syncwarp();
+  }
+  for (int i = wl; i < nt; i += 32) {
+    const double v = x[i];
+    xc[(size_t)c * nt + i] = v;
+    if (xr) xr[(size_t)i * nt + c] = v;
+    xc32[(size_t)c * nt + i] = (float)v;
+    xr32[(size_t)i * nt + c] = (float)v;
   }
 }
 
@@ -372,7 +433,8 @@ void launch_tail_inverse(cudaStream_t st, int t0, int nt, const int32_t* l_ptr,
                          const int32_t* l_idx, const double* l_val, const double* lsc, double* xc,
                          double* xr, float* xc32, float* xr32) {
   if (nt > 0)
-    tail_inverse_kernel<<<1, 128, 0, st>>>(t0, nt, l_ptr, l_idx, l_val, lsc, xc, xr, xc32, xr32);
+    tail_inverse_kernel<<<(nt + TI_WARPS - 1) / TI_WARPS, 32 * TI_WARPS, 0, st>>>(
+        t0, nt, l_ptr, l_idx, l_val, lsc, xc, xr, xc32, xr32);
 }
 
 void launch_adj_values(cudaStream_t st, int n, const int32_t* br, const double* cf,
