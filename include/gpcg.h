@@ -265,7 +265,9 @@ GPCG_API gpcg_status gpcg_base_solve(gpcg_ctx *ctx, double *theta, double *vm,
  *   flow[n_out][n_branch]                     active power at the from end
  *   island_label[n_out][n_bus]                min bus index of each bus's
  *                                             component after the outage
- *   iters[n_out][3]                           {outer, inner P, inner Q}
+ *   iters[n_out][3]                           {outer, inner P, inner Q}; with
+ *                                             FP32 inner solves the counts
+ *                                             depend on their rounding
  *   status[n_out]                             GPCG_SCEN_*
  *   max_loading[n_out]                        max over branches of
  *                                             max(|P_ij|,|P_ji|)/rating
@@ -360,7 +362,8 @@ GPCG_API gpcg_status gpcg_n1_adjoint(gpcg_ctx *ctx, const int32_t *outages, int3
  *   overload[s]    = those branches as a bit mask (as in gpcg_n1_screen).
  * Inputs: P[n_bus] bus injections (NULL: the grid's P_sched), host or device
  * memory as mem says.  Outputs, each optional: theta[n_out][n_bus],
- * flow[n_out][n_branch], iters[n_out] (PCG iterations), status[n_out]
+ * flow[n_out][n_branch], iters[n_out] (PCG iterations; FP64 calls
+ * without it take a direct form of the solve), status[n_out]
  * (GPCG_SCEN_OK, or GPCG_SCEN_ISLAND_NO_GEN when an island's injection has
  * no main-island generator to go to and the slack takes it), max_loading,
  * n_overload[n_out], overload[n_out][GPCG_MASK_WORDS(n_branch)].

@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(NTHREADS, FDPF_MIN_BLOCKS)
 // bridge's flow zero.
 // Bound by the loads and stores of one pass over the rows and one over the
 // branches: 13,500 outages of a 10,000-bus grid with every output 29.8 ms by
-// the PCG (1.85 iterations of three passes over five vectors).
+// the PCG (1.85 iterations of three passes over five vectors), 4.6 ms here.
 
 // f0 (lane 0) and fg (lane 1) of a call, by one CTA; rows as [row][2].
 __global__ void __launch_bounds__(NTHREADS) dc_base_kernel(DevMatT<double> M, DevGrid G,
