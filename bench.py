@@ -85,18 +85,25 @@ class ClockSampler:
                 "samples": len(self.rows)}
 
 
-def algorithmic_bytes(info, iters, w, n_bus, n_branch):
+def algorithmic_bytes(info, iters, w, n_bus, n_branch, reduced=False):
     """Bytes the method must move per screen (per-unit figures: 15 w n per
     inner PCG iteration, 32 n per outer half-iteration's FP64 mismatch,
     16 n + 8 m for the flows, plus the shared matrix and factor bytes per
-    iteration amortised over the scenarios)."""
+    iteration amortised over the scenarios).  `reduced`: the complete factor in
+    the vectors' precision, whose PCG runs on scalars -- one forward and one
+    backward substitution (4 w n and the factor twice) per half-iteration's
+    solve, whatever its iteration count."""
     outer = iters[:, 0].astype(np.float64)
     inP = iters[:, 1].astype(np.float64)
     inQ = iters[:, 2].astype(np.float64)
     S = iters.shape[0]
-    vec = 15.0 * w * (inP.sum() * info["n_p"] + inQ.sum() * info["n_q"])
     mis = 32.0 * n_bus * (2.0 * outer + 1.0).sum()
     flows = S * (16.0 * n_bus + 8.0 * n_branch)
+    if reduced:
+        vec = 4.0 * w * outer.sum() * (info["n_p"] + info["n_q"])
+        mats = outer.sum() * 2 * (info["nnz_lp"] + info["nnz_lq"]) * (w + 4) / max(S, 1)
+        return vec + mis + flows + mats
+    vec = 15.0 * w * (inP.sum() * info["n_p"] + inQ.sum() * info["n_q"])
     mats = (inP.sum() * (info["nnz_p"] + 2 * info["nnz_lp"]) +
             inQ.sum() * (info["nnz_q"] + 2 * info["nnz_lq"])) * (w + 4) / max(S, 1)
     return vec + mis + flows + mats
@@ -353,7 +360,8 @@ def run_gpcg(args):
         c.set_options(precision=prec)
 
     w = 8 if prec == gp.BATCHED_FP64 else 4
-    algo = algorithmic_bytes(info, iters, w, n, m)
+    reduced = args.precond == "exact" and args.precision != "fp16f"
+    algo = algorithmic_bytes(info, iters, w, n, m, reduced)
     fd_ms = statistics.mean(k[1] for k in kern_ms)
     peak, peak_kind = load_peaks()
     achieved = algo / (fd_ms / 1e3) / 1e9
@@ -500,7 +508,8 @@ def run_gen(args):
     w = 8 if prec == gp.BATCHED_FP64 else 4
     # the extension row adds one row to every B'' pass
     info_x = dict(info, n_q=info["n_q"] + 1)
-    algo = algorithmic_bytes(info_x, iters, w, n, m)
+    reduced = args.precond == "exact" and args.precision != "fp16f"
+    algo = algorithmic_bytes(info_x, iters, w, n, m, reduced)
     fd_ms = statistics.mean(k[1] for k in kern_ms)
     peak, peak_kind = load_peaks()
     achieved = algo / (fd_ms / 1e3) / 1e9
