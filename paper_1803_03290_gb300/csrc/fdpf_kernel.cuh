@@ -732,8 +732,13 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T, N
 //
 // NT threads a CTA: NTHREADS when the tiles fill the GPU at five CTAs per SM;
 // wide_launch (fdpf.h) says when fewer, wider CTAs take them.
+//
+// The PCG's kernels get the registers of four CTAs per SM (64): at five (48) its
+// passes spill.  IC(0), 2,700 outages of a 2,000-bus grid: 121.5 ms against 144.8;
+// the FP16-stored factor, 13,500 outages of 10,000 buses: 93.5 ms against 95.2.
 template <int T, typename VT, bool GEN, bool ZS = false, bool RED = false, int NT = NTHREADS>
-__global__ void __launch_bounds__(NT, ZS ? 2 : NT == NTHREADS ? FDPF_MIN_BLOCKS : 1024 / NT)
+__global__ void __launch_bounds__(
+    NT, ZS ? 2 : NT != NTHREADS ? 1024 / NT : RED ? FDPF_MIN_BLOCKS : PCG_MIN_BLOCKS)
     fdpf_tiles_kernel(FdpfParams P_, DevMatT<VT> MP_, DevMatT<VT> MQ_) {
   static_assert(!(ZS && RED), "z is a vector of the PCG");
   __shared__ LaneState<T, NT> L;

@@ -32,6 +32,7 @@ constexpr int UNR = FDPF_UNROLL;  // rows per thread in flight in the SpMV
 #ifndef FDPF_MIN_BLOCKS
 #define FDPF_MIN_BLOCKS 5  // resident CTAs per SM the register budget is cut for
 #endif
+constexpr int PCG_MIN_BLOCKS = FDPF_MIN_BLOCKS < 4 ? FDPF_MIN_BLOCKS : 4;  // of the general PCG
 
 // Inner iterations without progress after which a solve stops: the outer
 // FP64 loop then refines the answer (iterative refinement).
