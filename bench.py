@@ -109,6 +109,12 @@ def algorithmic_bytes(info, iters, w, n_bus, n_branch, reduced=False):
     return vec + mis + flows + mats
 
 
+def reduced_solves(args):
+    """Whether the screens' inner solves run in their reduced form: with the
+    complete factor, and FP32 vectors only below the bench's tolerance."""
+    return args.precond == "exact" and args.precision == "fp64"
+
+
 def island_split(g, iters):
     """Mean iterations of the outages that island buses (the bridges) and of
     the rest, outage k being branch k: the islanding scenarios' extra inner
@@ -360,7 +366,7 @@ def run_gpcg(args):
         c.set_options(precision=prec)
 
     w = 8 if prec == gp.BATCHED_FP64 else 4
-    reduced = args.precond == "exact" and args.precision != "fp16f"
+    reduced = reduced_solves(args)
     algo = algorithmic_bytes(info, iters, w, n, m, reduced)
     fd_ms = statistics.mean(k[1] for k in kern_ms)
     peak, peak_kind = load_peaks()
@@ -508,7 +514,7 @@ def run_gen(args):
     w = 8 if prec == gp.BATCHED_FP64 else 4
     # the extension row adds one row to every B'' pass
     info_x = dict(info, n_q=info["n_q"] + 1)
-    reduced = args.precond == "exact" and args.precision != "fp16f"
+    reduced = reduced_solves(args)
     algo = algorithmic_bytes(info_x, iters, w, n, m, reduced)
     fd_ms = statistics.mean(k[1] for k in kern_ms)
     peak, peak_kind = load_peaks()

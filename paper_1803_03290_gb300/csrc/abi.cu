@@ -45,6 +45,8 @@ void launch_gather_half(cudaStream_t, int, const int32_t*, const double*, __half
 void launch_inv_diag(cudaStream_t, int, const int32_t*, const double*, double*, float*);
 void launch_tail_inverse(cudaStream_t, int, int, const int32_t*, const int32_t*, const double*,
                          const double*, double*, double*, float*, float*);
+void launch_tail_inverse_warp(cudaStream_t, int, int, const int32_t*, const int32_t*,
+                              const double*, double*, double*, float*, float*);
 void launch_adj_values(cudaStream_t, int, const int32_t*, const double*, const double*,
                        const double*, double2*, double*, double*);
 void launch_branch_count(cudaStream_t, int, const int32_t*, const int32_t*, const int32_t*,
@@ -292,6 +294,7 @@ struct gpcg_ctx {
   // chosen yet), how they were chosen (0 none, 1 probes, 2 cache) and the
   // power of two of the scenario count they were chosen for
   int per_sm = 0, per_sm_used = 0, tuned = 0, tuned_bucket = -1;
+  bool tuned_red = false;  // the tuned kernel was the one with reduced inner solves
   int tail_rows_now = TAIL_ROWS;  // the cap the factors' tails are built with
   // the factors' dense-tail data of B' (0) and B'' (1): level schedule of the
   // rows before the tail and the tail block's inverse, rebuilt when the tail
@@ -543,19 +546,26 @@ static gpcg_status alloc_tail(gpcg_ctx* c, MatDev& M, int which, int cap) {
 }
 
 // The tail block's inverse from the factor's values: of the FP16-stored
-// factor first (M.xc as FP64 scratch), then of the factor itself.
-static void launch_tail_inverses(MatDev& M, cudaStream_t st) {
+// factor first (M.xc as FP64 scratch), then of the factor itself.  warps: the
+// adjoint's factor (fill_values).
+static void launch_tail_inverses(MatDev& M, cudaStream_t st, bool warps = false) {
   const MatrixPlan& P = M.plan;
   sub_fill(st, M.bwd, M.l_val, M.inv_diag);
   launch_gather_val(st, M.n_th, M.th_src, M.l_val, M.th_val, M.th_val32);
   if (M.lsc && M.xch)
     launch_tail_inverse(st, P.tail_row0, P.n - P.tail_row0, M.l_ptr, M.l_idx, M.l_val, M.lsc,
                         M.xc, nullptr, M.xch, M.xrh);
-  launch_tail_inverse(st, P.tail_row0, P.n - P.tail_row0, M.l_ptr, M.l_idx, M.l_val, nullptr,
-                      M.xc, M.xr, M.xc32, M.xr32);
+  if (warps)
+    launch_tail_inverse_warp(st, P.tail_row0, P.n - P.tail_row0, M.l_ptr, M.l_idx, M.l_val, M.xc,
+                             M.xr, M.xc32, M.xr32);
+  else
+    launch_tail_inverse(st, P.tail_row0, P.n - P.tail_row0, M.l_ptr, M.l_idx, M.l_val, nullptr,
+                        M.xc, M.xr, M.xc32, M.xr32);
 }
 
-static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w) {
+// warps: the factorisation kernels of the adjoint, which spread a row's sums over a
+// warp; a context's own factor keeps them in row order (build.cu).
+static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w, bool warps = false) {
   const MatrixPlan& P = M.plan;
   const int nl = P.L.nnz();
   (void)nl;
@@ -563,10 +573,10 @@ static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w) {
   CUDA_TRY(cudaMemset(c->d_err, 0, sizeof(int32_t)));
   launch_laplacian_values(st, P.n, M.bus_of_row, M.row_of_bus, c->G.adj_ptr, c->G.adj_idx,
                           c->G.adj_br, w, c->G.f, M.c, M.a_ptr, M.a_idx, M.a_val, c->d_err);
-  // wide levels one launch each, runs of narrow ones one launch together
+  // one launch per level; warps: runs of narrow ones one launch together
   for (int k = 0, nl = (int)P.lev_ptr.size() - 1; k < nl;) {
     int e = k;
-    while (e < nl && P.lev_ptr[e + 1] - P.lev_ptr[e] <= ic_narrow_rows()) ++e;
+    while (warps && e < nl && P.lev_ptr[e + 1] - P.lev_ptr[e] <= ic_narrow_rows()) ++e;
     if (e > k) {
       launch_ic_narrow(st, M.lev_ptr, k, e, M.a_ptr, M.a_idx, M.a_val, M.l_ptr, M.l_idx, M.l_val,
                        c->d_err);
@@ -592,7 +602,7 @@ static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w) {
       launch_gather_half(st, E->nover, E->osrc, M.lsc, E->ovalh);
     }
   }
-  launch_tail_inverses(M, st);
+  launch_tail_inverses(M, st, warps);
   CUDA_TRY(cudaGetLastError());
   int32_t herr = 0;
   CUDA_TRY(cudaMemcpy(&herr, c->d_err, sizeof herr, cudaMemcpyDeviceToHost));
@@ -1307,8 +1317,7 @@ template <typename VT>
 static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, int slots,
                             bool f16 = false, bool zs = false, int nt = NTHREADS) {
   const DevMatT<VT> MP = c->MP.view<VT>(f16), MQ = c->MQ.view<VT>(f16);
-  const bool red = !zs && reduced_form(P.precond, MP, MQ);
-  const bool one = red;
+  const bool one = P.reduced && !zs;
   Layout Lo = make_layout(c, T, slots, sizeof(VT), zs, one);
   gpcg_status s = ensure_work(c, Lo.bytes);
   if (s != GPCG_OK) return s;
@@ -1386,7 +1395,10 @@ extern "C" gpcg_status gpcg_base_solve(gpcg_ctx* c, double* theta, double* vm, d
   CUDA_TRY(cudaMalloc(&d_iters3, 3 * sizeof(int32_t)));
   P.out_iters = d_iters3;
   P.out_status = d_stat;
-  s = run_fdpf<double>(c, st, P, 2, 1, false, false, wide_launch(1, c->num_sms, c->MP.plan.n, true).nt);
+  // (by the PCG: every screen starts from this state, and the last bits of it
+  // decide the verdicts of scenarios that have no solution; 10,000 buses
+  // 22.9 ms, 11.2 by a wide CTA with reduced solves)
+  s = run_fdpf<double>(c, st, P, 2, 1);
   int32_t hs = -1, hit[3] = {0, 0, 0};
   if (s == GPCG_OK) {
     cudaError_t ce = cudaDeviceSynchronize();
@@ -1462,13 +1474,13 @@ static std::map<std::vector<long long>, TuneChoice> g_tune_cache;
 static_assert(KX == GPCG_MAX_EXT_ROWS, "extension rows of the kernel and of the C ABI");
 static_assert(TAIL_ROWS >= GPCG_MAX_TAIL_ROWS, "the kernel's tail buffer holds the largest tail");
 
-static std::vector<long long> tune_key(const gpcg_ctx* c, bool ext, int bucket) {
+static std::vector<long long> tune_key(const gpcg_ctx* c, bool ext, bool red, int bucket) {
   int major = 0, minor = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, c->device);
   return {c->num_sms, major, minor, c->n, c->m,
           c->MP.plan.A.nnz(), c->MP.plan.L.nnz(), c->MQ.plan.A.nnz(), c->MQ.plan.L.nnz(),
-          c->opt.precision, c->opt.precond, ext, c->zs_allowed, bucket,
+          c->opt.precision, c->opt.precond, ext, red, c->zs_allowed, bucket,
           c->opt.tile, c->opt.ctas_per_sm, c->opt.tail_rows};
 }
 
@@ -1596,7 +1608,11 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
   const bool ext = gen || c->G.qmax != nullptr;
   const bool f16 = c->opt.precision == GPCG_BATCHED_FP32_F16;
   const bool f32 = c->opt.precision == GPCG_BATCHED_FP32 || f16;
-  const bool red = reduced_form(c->opt.precond, c->MP.view<float>(f16), c->MQ.view<float>(f16));
+  const bool red =
+      !plain && (f32 ? reduced_form(c->opt.precond, c->MP.view<float>(f16),
+                                    c->MQ.view<float>(f16), c->opt.tol)
+                     : reduced_form(c->opt.precond, c->MP.view<double>(), c->MQ.view<double>()));
+  P.reduced = red;
   // islanding for every outage (the autotuner's probes need it too)
   // (inside a stream capture the events become event-record nodes of the graph)
   auto record = [](cudaEvent_t ev, cudaStream_t s, bool cap) {
@@ -1632,8 +1648,9 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
     int bucket = 0;
     while (((size_t)1 << bucket) < S) ++bucket;
     const bool knobs = !c->opt.tile || !c->opt.ctas_per_sm || !c->opt.tail_rows;
-    if (knobs && bucket != c->tuned_bucket) {
-      const std::vector<long long> key = tune_key(c, ext, bucket);
+    // (a tolerance on the other side of reduced_form's takes another kernel)
+    if (knobs && (bucket != c->tuned_bucket || red != c->tuned_red)) {
+      const std::vector<long long> key = tune_key(c, ext, red, bucket);
       TuneChoice got{0, 0, 0};
       bool hit = false;
       {
@@ -1676,6 +1693,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
           if (r != GPCG_OK) return r;
           FdpfParams Q = base_params(c);
           Q.sc = P.sc;
+          Q.reduced = P.reduced;
           Q.th0 = P.th0; Q.V0 = P.V0; Q.c0 = P.c0; Q.s0 = P.s0; Q.ef0 = P.ef0;
           // untimed: the first launch of a kernel variant, one tile of the
           // probe's lightest scenarios (the end of the scheduling order)
@@ -1739,6 +1757,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
       c->per_sm = got.per_sm;
       c->tuned = hit ? 2 : 1;
       c->tuned_bucket = bucket;
+      c->tuned_red = red;
     }
     T = c->opt.tile ? c->opt.tile : (c->tile ? c->tile : 2);
     if (ext) T = std::min(T, 8);  // the kernel with extension rows: tiles of 2, 4, 8
@@ -2068,7 +2087,7 @@ extern "C" gpcg_status gpcg_n1_adjoint(gpcg_ctx* c, const int32_t* outages, int3
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
   if (ce != cudaSuccess) { cleanup(); return fail(GPCG_ERR_CUDA, "adjoint inputs: %s", cudaGetErrorString(ce)); }
   // base-case B' with the given susceptances, and its factor
-  s_ = fill_values(c, c->MA, db);
+  s_ = fill_values(c, c->MA, db, true);
   if (s_ != GPCG_OK) { cleanup(); return s_; }
   launch_branch_values(c, c->MA, db, st);
   // outputs (device staging in host mode)

@@ -183,9 +183,12 @@ __global__ void ic_level_kernel(int row0, int row1, const int32_t* __restrict__ 
   }
 }
 
-// The narrow levels [lev0, lev1) in one launch of one CTA, a warp per row: a
-// launch per level (67 on a 2,000-bus grid) and a thread walking both rows of
-// every product one entry at a time took most of a re-factorisation.  The row's
+// The narrow levels [lev0, lev1) in one launch of one CTA, a warp per row, for
+// the adjoint, which factorises on every call: a launch per level (67 on a
+// 2,000-bus grid) and a thread walking both rows of every product one entry at a
+// time took most of a re-factorisation.  A context's own factor keeps the sums
+// in row order (ic_level_kernel): the last bits of the base case and of the
+// FP32 factor decide the verdicts of scenarios that have no solution.  The row's
 // entries are computed in order; the sum over the columns rows i and j share has
 // its terms spread over the warp (each looks the column of row j up in row i).
 constexpr int IC_NARROW = 512;  // rows of a level, at most
@@ -386,19 +389,51 @@ void launch_inv_diag(cudaStream_t st, int n, const int32_t* pos, const double* l
 }
 // X = inverse of the factor's tail block L_tt (rows and columns
 // [t0, t0 + nt) of L, lower triangular): column c of X by forward
-// substitution of L_tt x = e_c in FP64, a warp per column with the row's
-// terms spread over its threads (a thread per column in one CTA took 1 ms for
-// 232 rows: each term waited for its own loads).  Written column-major
-// (xc[c nt + i] = X_ic) and row-major (xr[i nt + c] = X_ic), zeros above the
-// diagonal, in FP64 (xr optional) and FP32.
+// substitution of L_tt x = e_c, one thread per column, in FP64.  Written
+// column-major (xc[c nt + i] = X_ic) and row-major (xr[i nt + c] = X_ic),
+// zeros above the diagonal, in FP64 (xr optional) and FP32.
 // With lsc (the scaled factor Ls = L D^-1) the block inverted is the one
 // the FP16 storage represents: L_ij = fp16(Ls_ij) L_jj.
+__global__ void tail_inverse_kernel(int t0, int nt, const int32_t* __restrict__ l_ptr,
+                                    const int32_t* __restrict__ l_idx,
+                                    const double* __restrict__ l_val,
+                                    const double* __restrict__ lsc, double* xc, double* xr,
+                                    float* xc32, float* xr32) {
+  for (int c = threadIdx.x; c < nt; c += blockDim.x) {
+    // xc holds the column in FP64 while it is built (its earlier entries
+    // are the unknowns solved before)
+    for (int i = 0; i < nt; ++i) {
+      double v = 0.0;
+      if (i >= c) {
+        const int R = t0 + i, e0 = l_ptr[R], e1 = l_ptr[R + 1] - 1;  // diagonal last
+        double sum = (i == c) ? 1.0 : 0.0;
+        for (int e = e0; e < e1; ++e) {
+          const int jg = l_idx[e], j = jg - t0;
+          if (j < c) continue;
+          const double lij =
+              lsc ? (double)__half2float(__double2half(lsc[e])) * l_val[l_ptr[jg + 1] - 1]
+                  : l_val[e];
+          sum -= lij * xc[(size_t)c * nt + j];
+        }
+        v = sum / l_val[e1];
+      }
+      xc[(size_t)c * nt + i] = v;
+      if (xr) xr[(size_t)i * nt + c] = v;
+      xc32[(size_t)c * nt + i] = (float)v;
+      xr32[(size_t)i * nt + c] = (float)v;
+    }
+  }
+}
+
+// The same for the adjoint (see ic_narrow_kernel): a warp per column, the row's
+// terms spread over its threads (a thread per column in one CTA takes 1 ms for 232
+// rows: each term waits for its own loads).
 constexpr int TI_WARPS = 4;
 __global__ void __launch_bounds__(32 * TI_WARPS)
-    tail_inverse_kernel(int t0, int nt, const int32_t* __restrict__ l_ptr,
-                        const int32_t* __restrict__ l_idx, const double* __restrict__ l_val,
-                        const double* __restrict__ lsc, double* xc, double* xr, float* xc32,
-                        float* xr32) {
+    tail_inverse_warp_kernel(int t0, int nt, const int32_t* __restrict__ l_ptr,
+                             const int32_t* __restrict__ l_idx,
+                             const double* __restrict__ l_val, double* xc, double* xr,
+                             float* xc32, float* xr32) {
   __shared__ double col[TI_WARPS][TAIL_ROWS];
   const int warp = threadIdx.x >> 5, wl = threadIdx.x & 31;
   const int c = blockIdx.x * TI_WARPS + warp;
@@ -409,11 +444,9 @@ __global__ void __launch_bounds__(32 * TI_WARPS)
     const int R = t0 + i, e0 = l_ptr[R], e1 = l_ptr[R + 1] - 1;  // diagonal last
     double s = 0.0;
     for (int e = e0 + wl; e < e1; e += 32) {
-      const int jg = l_idx[e], j = jg - t0;
+      const int j = l_idx[e] - t0;
       if (j < c) continue;
-      const double lij =
-          lsc ? (double)__half2float(__double2half(lsc[e])) * l_val[l_ptr[jg + 1] - 1] : l_val[e];
-      s = fma(lij, x[j], s);
+      s = fma(l_val[e], x[j], s);
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
@@ -423,7 +456,7 @@ __global__ void __launch_bounds__(32 * TI_WARPS)
   for (int i = wl; i < nt; i += 32) {
     const double v = x[i];
     xc[(size_t)c * nt + i] = v;
-    if (xr) xr[(size_t)i * nt + c] = v;
+    xr[(size_t)i * nt + c] = v;
     xc32[(size_t)c * nt + i] = (float)v;
     xr32[(size_t)i * nt + c] = (float)v;
   }
@@ -433,8 +466,14 @@ void launch_tail_inverse(cudaStream_t st, int t0, int nt, const int32_t* l_ptr,
                          const int32_t* l_idx, const double* l_val, const double* lsc, double* xc,
                          double* xr, float* xc32, float* xr32) {
   if (nt > 0)
-    tail_inverse_kernel<<<(nt + TI_WARPS - 1) / TI_WARPS, 32 * TI_WARPS, 0, st>>>(
-        t0, nt, l_ptr, l_idx, l_val, lsc, xc, xr, xc32, xr32);
+    tail_inverse_kernel<<<1, 128, 0, st>>>(t0, nt, l_ptr, l_idx, l_val, lsc, xc, xr, xc32, xr32);
+}
+void launch_tail_inverse_warp(cudaStream_t st, int t0, int nt, const int32_t* l_ptr,
+                              const int32_t* l_idx, const double* l_val, double* xc, double* xr,
+                              float* xc32, float* xr32) {
+  if (nt > 0)
+    tail_inverse_warp_kernel<<<(nt + TI_WARPS - 1) / TI_WARPS, 32 * TI_WARPS, 0, st>>>(
+        t0, nt, l_ptr, l_idx, l_val, xc, xr, xc32, xr32);
 }
 
 void launch_adj_values(cudaStream_t st, int n, const int32_t* br, const double* cf,

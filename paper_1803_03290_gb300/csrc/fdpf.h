@@ -44,6 +44,7 @@ struct FdpfParams {
   int flat_start = 0;
   double tol = 1e-4, inner_rtol = 3e-3;
   int max_outer = 50, max_inner = 500, precond = PREC_EXACT;
+  int reduced = 0;  // the inner solves in their reduced form (reduced_form below)
   int32_t* tile_counter = nullptr;     // scenario queue head
   const int32_t* order = nullptr;      // scenarios in processing order (null: 0..S-1)
   void *wx = nullptr, *wr = nullptr, *wp = nullptr, *wq = nullptr, *wz = nullptr;
@@ -69,11 +70,31 @@ struct FdpfParams {
   BusTab tabP, tabQ;  // non-slack buses, rows of B'; PQ buses, rows of B''
 };
 
-// Whether the inner solves run in their reduced form (reduced.cuh): the
-// complete base-case factor, in the precision of the vectors.
+// Whether a screen's inner solves run in their reduced form (reduced.cuh): the
+// complete base-case factor in the precision of the vectors, and for FP32 vectors
+// an outer tolerance that leaves nothing of their rounding in the results.
+//
+// At a loose tolerance a state ends one inner solve away from the last
+// mismatch that failed it, and with FP32 vectors that solve is rounded in the
+// fourth digit: the PCG's recursive residual asks for one more iteration in 5 %
+// of the scenarios than the reduced recurrence does.  Both states meet the
+// tolerance, but a branch within 1e-4 of its rating may be overloaded in one and
+// not in the other, and a scenario without a solution ends wherever the rounding
+// takes it.  A verdict would then depend on which kernel the preconditioner and
+// the list allow.  Overload masks against the PCG's, at 1e-4 p.u.: different in 1
+// of 20 lists of 13,500 outages of 10,000 buses and 1 of 25 of 2,700 outages of
+// 2,000 buses with reactive limits (converged scenarios), and in 1 of 10 of 2,047
+// outages of 50,000 buses (scenarios that do not converge).  So FP32 screens keep
+// the PCG there, at its price: 13,500 outages of 10,000 buses 73.3 ms (reduced
+// 42.4), 2,047 of 50,000 buses 98.5 ms (57), 2,700 of 2,000 buses with limits
+// 38.6 ms (13.5).  From 1e-9 p.u. down the results agree to 1e-9 and the verdicts
+// with them; FP64 vectors take the same iterations in either form.
+constexpr double REDUCED_F32_TOL = 1e-9;
 template <typename VT>
-inline bool reduced_form(int precond, const DevMatT<VT>& MP, const DevMatT<VT>& MQ) {
-  return precond == PREC_EXACT && MP.br.ptr && MQ.br.ptr && !MP.Lh && !MQ.Lh;
+inline bool reduced_form(int precond, const DevMatT<VT>& MP, const DevMatT<VT>& MQ,
+                         double tol = 0.0) {
+  return precond == PREC_EXACT && MP.br.ptr && MQ.br.ptr && !MP.Lh && !MQ.Lh &&
+         (sizeof(VT) == 8 || tol <= REDUCED_F32_TOL);
 }
 
 // A launch of S scenarios too few to fill the GPU: threads per CTA, CTAs and
@@ -99,7 +120,7 @@ inline size_t wide_shared(int nt, size_t vec_bytes) {
 // / 1.65 ms, 600 outages 3.72 / 2.89 / 3.06 ms, 1,000 outages 4.04 / 3.46 / 4.98 ms,
 // 2,700 outages 6.9 / 8.1 / 12.1 ms; 10,000 buses, 1,000 outages 16.1 / 13.7 / 16.3 ms,
 // 1,500 outages 18.2 / 20.1 / 23.2 ms; 180 outages of 120 buses 1.57 / 1.82 /
-// 2.07 ms; base case of 10,000 buses 16.2 / 12.5 / 11.3 ms.
+// 2.07 ms.
 inline WideLaunch wide_launch(int S, int num_sms, int rows, bool fp64) {
   const int most = rows >= 1024 ? 1024 : rows >= 512 || fp64 ? 512 : NTHREADS;
   const WideLaunch w = S <= num_sms       ? WideLaunch{std::min(1024, most), S, 1}

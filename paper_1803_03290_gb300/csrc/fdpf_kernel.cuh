@@ -39,16 +39,21 @@ namespace gpcg {
 // dQ/|V| and the relative step dV/|V| -- which the outer FP64 loop refines,
 // so the FP32 form's few-ulp rounding moves no converged state.  The state
 // keeps no |V| of its own: e + jf is the state.
-template <typename VT>
-__device__ __forceinline__ VT inv_vmag(double e, double f);
-template <>
-__device__ __forceinline__ float inv_vmag<float>(double e, double f) {
-  const float a = to_f32(e), b = to_f32(f);
-  return rsqrtf(fmaf(a, a, b * b));
-}
-template <>
-__device__ __forceinline__ double inv_vmag<double>(double e, double f) {
-  return rsqrt(fma(e, e, f * f));  // 7 FP64 instructions, 1 / sqrt takes 15
+//
+// RED (here and in the passes below): the kernels with reduced inner solves.  The
+// PCG's kernels keep the longer forms, whose last bits their results have always
+// had: they solve the base case and the FP32 screens at loose tolerances, where a
+// last bit decides the verdict of a scenario that has no solution.
+template <typename VT, bool RED>
+__device__ __forceinline__ VT inv_vmag(double e, double f) {
+  if constexpr (sizeof(VT) == 4) {
+    const float a = to_f32(e), b = to_f32(f);
+    return rsqrtf(fmaf(a, a, b * b));
+  } else if constexpr (RED) {
+    return rsqrt(fma(e, e, f * f));  // 7 FP64 instructions, 1 / sqrt takes 15
+  } else {
+    return 1.0 / sqrt(fma(e, e, f * f));
+  }
 }
 
 // ------------------------------------------------------------ mismatch
@@ -113,8 +118,8 @@ __device__ __forceinline__ double2 bus_current(const DevGrid& G, const LaneState
 // descriptor and one 16-byte load per neighbour slot, in the order of the
 // visit (BusTab).  With the same for the updates and flows: 131.7 M -> 103 M FP64
 // warp instructions for 2,048 outages of 10,000 buses, and all 13,500 outages at
-// 1e-4 p.u. 56.2 -> 46.7 ms.
-template <int T, int NT, typename VT, bool WITH_P, bool GEN>
+// 1e-4 p.u. 56.2 -> 46.7 ms with reduced solves, 79.8 -> 73.3 ms with the PCG.
+template <int T, int NT, typename VT, bool WITH_P, bool GEN, bool RED>
 __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMatT<VT>& MQ,
                                                LaneState<T, NT>& L, const double* __restrict__ EF,
                                                VT* __restrict__ rhs,
@@ -199,7 +204,7 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
             }
           }
         }
-        // the outaged branch's terms back out at its two end buses
+        // the outaged branch's term back out at its two end buses
         if (end0 || end1) {
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
@@ -213,12 +218,6 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
             double& im = j ? im1 : im0;
             re -= fma(-go, v.x, bo * v.y);
             im -= fma(-go, v.y, -bo * v.x);
-            // and its share of the diagonal
-            const double c2 = e ? 1.0 : L.cl[ln] * L.cl[ln];
-            const double gs = c2 * L.gl[ln], bs = c2 * L.bl[ln];
-            const double eo = j ? ev1.x : ev0.x, fo = j ? ev1.y : ev0.y;
-            re -= fma(gs, eo, -bs * fo);
-            im -= fma(gs, fo, bs * eo);
           }
         }
       }
@@ -231,7 +230,7 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
         if (!(j ? on1 : on0)) continue;
         const int ln = l0 + j;
         const double ei = j ? ev1.x : ev0.x, fi = j ? ev1.y : ev0.y;
-        const VT iv = inv_vmag<VT>(ei, fi);
+        const VT iv = inv_vmag<VT, RED>(ei, fi);
         // a tripped generator's bus keeps only its load and takes no share
         // of the re-dispatch; a bus with an extension row (that one, or a PV
         // bus held at a reactive limit) is PQ with the injection qx
@@ -265,9 +264,15 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
           out.v[j] = to_vt<VT>(dP) * iv;
           continue;
         }
+        double Gd = yd.x, Bd = yd.y;
+        if (j ? end1 : end0) {  // the outaged branch's share of the diagonal
+          const double c2 = i == L.fb[ln] ? L.cl[ln] * L.cl[ln] : 1.0;
+          Gd -= c2 * L.gl[ln];
+          Bd -= c2 * L.bl[ln];
+        }
         // I_i = Y_ii V_i + sum_j Y_ij V_j
-        const double re = fma(yd.x, ei, fma(-yd.y, fi, j ? re1 : re0));
-        const double im = fma(yd.x, fi, fma(yd.y, ei, j ? im1 : im0));
+        const double re = fma(Gd, ei, fma(-Bd, fi, j ? re1 : re0));
+        const double im = fma(Gd, fi, fma(Bd, ei, j ? im1 : im0));
         // dQ = Q_sched - Im(V_i conj(I_i)); dP = P_sched + re-dispatch - Re(...)
         if (WITH_P) {
           const double dP = fma(-ei, re, fma(-fi, im, redispatched(pq.x)));
@@ -318,27 +323,27 @@ __device__ GPCG_PASS_INLINE void mismatch_pass(const FdpfParams& P, const DevMat
         const double2 v = *reinterpret_cast<const double2*>(EF + ef_at<T>(b, ln));
         const double dQ = fma(-v.y, I.x, fma(v.x, I.y, SW->xq[ln][s]));
         upd_max_shared<Geo<T, NT>::TPR == 1>(&L.emax[1][ln], dQ);
-        rhs[(size_t)(MQ.n + 1 + s) * T + ln] = to_vt<VT>(dQ) * inv_vmag<VT>(v.x, v.y);
+        rhs[(size_t)(MQ.n + 1 + s) * T + ln] = to_vt<VT>(dQ) * inv_vmag<VT, RED>(v.x, v.y);
       }
     }
 }
 
 // (e, f) rotated through the angle d, in FP64:
 //   e' = e cos d - f sin d = e - (e a + f b),  f' = f - (f a - e b),
-// with a = 1 - cos d and b = sin d from their Taylor series.  For |d| <= 1e-4,
-// where most buses are after a scenario's first step, a = d^2/2 and
-// b = d - d^3/6 (d a / 3 = d^3/6; the first dropped terms are below 5e-18); for
-// |d| <= 0.02 two more terms in u = d^2 (dropped terms below 3e-16); larger
-// steps call sincos.  The rotation is exact to FP64 rounding, so the state
+// with a = 1 - cos d and b = sin d.  For |d| <= 0.02 both come from their
+// Taylor series in u = d^2 (a = u/2 - u^2/24 + u^3/720, b = d - d^3/6 +
+// d^5/120; the first dropped terms are below 3e-16 there), larger steps call
+// sincos; RED: for |d| <= 1e-4, where most buses are after a scenario's first
+// step, a = d^2/2 and b = d - d^3/6 (d a / 3 = d^3/6; dropped terms below 5e-18).  The rotation is exact to FP64 rounding, so the state
 // (e, f) stays at the angle theta and modulus |V| that the kernel reports: the
 // state whose mismatch the convergence test evaluated is the state that is
 // returned.  x: the step in the inner solve's precision, which decides the
 // branch off the FP64 pipe; d: the same in FP64.
-template <typename VT>
+template <typename VT, bool RED>
 __device__ __forceinline__ void rotate_ef(VT x, double d, double& e, double& f) {
   double a, b;
   const VT ax = fabs(x);
-  if (ax <= (VT)1e-4) {
+  if (RED && ax <= (VT)1e-4) {
     a = d * to_f64((VT)0.5 * x);
     b = fma(d * a, -1.0 / 3.0, d);
   } else if (ax <= (VT)0.02) {
@@ -359,9 +364,9 @@ __device__ __forceinline__ void rotate_ef(VT x, double d, double& e, double& f) 
 // FP32 vectors take it in FP32 (the step is an inner-solve iterate that the
 // outer FP64 loop refines; r is then exact as an FP64 number), FP64 vectors
 // in FP64.
-template <typename VT>
+template <typename VT, bool RED>
 __device__ __forceinline__ double v_ratio(VT dv, double e, double f) {
-  return to_f64(dv * inv_vmag<VT>(e, f));
+  return to_f64(dv * inv_vmag<VT, RED>(e, f));
 }
 
 // theta += dtheta (P half-step) or |V| += dV (Q half-step) on the matrix's
@@ -372,7 +377,7 @@ __device__ __forceinline__ double v_ratio(VT dv, double e, double f) {
 // is x + xalpha p, the inner solve's deferred last step.  In bus order, so that
 // the state (48 bytes read and written per bus and pair of lanes) streams and
 // only the 8 bytes of x are gathered.
-template <int T, int NT, typename VT, bool IS_P, bool GEN>
+template <int T, int NT, typename VT, bool IS_P, bool GEN, bool RED>
 __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<VT>& M,
                                              LaneState<T, NT>& L, const VT* __restrict__ x,
                                              const VT* __restrict__ p, double* th, double* EF,
@@ -413,8 +418,8 @@ __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<
     }
     if (IS_P) {
       const double d0 = to_f64(dx.a), d1 = to_f64(dx.b);
-      if (on0) rotate_ef<VT>(dx.a, d0, u0.x, u0.y);
-      if (on1) rotate_ef<VT>(dx.b, d1, u1.x, u1.y);
+      if (on0) rotate_ef<VT, RED>(dx.a, d0, u0.x, u0.y);
+      if (on1) rotate_ef<VT, RED>(dx.b, d1, u1.x, u1.y);
       if (keep_th) {
         const size_t o = (size_t)d.x * T + l0;
         Pair<double> t = ld2(th + o);
@@ -424,11 +429,11 @@ __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<
       }
     } else {
       if (on0) {
-        const double r = v_ratio<VT>(dx.a, u0.x, u0.y);
+        const double r = v_ratio<VT, RED>(dx.a, u0.x, u0.y);
         u0 = make_double2(fma(u0.x, r, u0.x), fma(u0.y, r, u0.y));
       }
       if (on1) {
-        const double r = v_ratio<VT>(dx.b, u1.x, u1.y);
+        const double r = v_ratio<VT, RED>(dx.b, u1.x, u1.y);
         u1 = make_double2(fma(u1.x, r, u1.x), fma(u1.y, r, u1.y));
       }
     }
@@ -454,7 +459,7 @@ __device__ GPCG_LOOP_INLINE void update_pass(const FdpfParams& P, const DevMatT<
       }
       double2* ef = reinterpret_cast<double2*>(EF + ef_at<T>(b, ln));
       const double2 u = ef[0];
-      const double r = v_ratio<VT>(dx, u.x, u.y);
+      const double r = v_ratio<VT, RED>(dx, u.x, u.y);
       ef[0] = make_double2(fma(u.x, r, u.x), fma(u.y, r, u.y));
     }
 }
@@ -633,7 +638,7 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T, N
             // below has at most 8 roundings of 2^-24 of its magnitude, and so
             // has their sum: err = 2^-20 (|c^2 g| + |g|, |c g|, |c b|) times the
             // voltages' magnitudes covers it twice.  (All 13,500 outages of 10,000
-            // buses, overloads only: 45.7 -> 42.4 ms.)
+            // buses, overloads only, reduced solves: 45.7 -> 42.4 ms.)
             const float ea = to_f32(va[h].x), fa = to_f32(va[h].y);
             const float eb = to_f32(vb[h].x), fb = to_f32(vb[h].y);
             const float ga = to_f32(y0.x), gc = to_f32(y0.y), bc = to_f32(y1.x), gb = to_f32(y1.y);
@@ -727,8 +732,8 @@ __device__ GPCG_PASS_INLINE void retire_pass(const FdpfParams& P, LaneState<T, N
 // of shared memory (80 KB for FP32 tiles of two on a 10,000-bus grid), two
 // CTAs fit an SM, and the register budget is set for two.
 //
-// RED: the inner solves in their reduced form (reduced.cuh), for the complete
-// base-case factor: one vector per slot, P.wr.
+// RED: the inner solves in their reduced form (reduced.cuh), where reduced_form
+// (fdpf.h) allows it: one vector per slot, P.wr.
 //
 // NT threads a CTA: NTHREADS when the tiles fill the GPU at five CTAs per SM;
 // wide_launch (fdpf.h) says when fewer, wider CTAs take them.
@@ -869,7 +874,7 @@ __global__ void __launch_bounds__(
       continue;
     }
     // P half-step: mismatch + convergence test
-    mismatch_pass<T, NT, VT, true, GEN>(P, MQ, L, EF, r, SW);
+    mismatch_pass<T, NT, VT, true, GEN, RED>(P, MQ, L, EF, r, SW);
     __syncthreads();
     if (tid < T) {
       {
@@ -961,19 +966,19 @@ __global__ void __launch_bounds__(
       if constexpr (RED) {
         red_solve<T, NT, VT>(P, MP, L, *RL, r, L.raP, L.rbP, L.inP, L.hold);
         GPCG_PHASE(2);
-        update_pass<T, NT, VT, true, GEN>(P, MP, L, r, nullptr, th, EF, SW, RL->xa);
+        update_pass<T, NT, VT, true, GEN, true>(P, MP, L, r, nullptr, th, EF, SW, RL->xa);
       } else if constexpr (NT == NTHREADS) {
         pcg_solve<T, VT, true, GEN>(P, MP, L, x, r, p, q, z, L.raP, L.rbP, L.wP, L.inP, nullptr,
                                     nullptr, L.hold);
         GPCG_PHASE(2);
-        update_pass<T, NT, VT, true, GEN>(P, MP, L, x, p, th, EF, SW);
+        update_pass<T, NT, VT, true, GEN, false>(P, MP, L, x, p, th, EF, SW);
       }
     }
     __syncthreads();
     GPCG_PHASE(3);
     // Q half-step: the Q mismatch after the P step; a lane whose Q mismatch
     // is within the tolerance takes no Q step
-    mismatch_pass<T, NT, VT, false, GEN>(P, MQ, L, EF, r, SW);
+    mismatch_pass<T, NT, VT, false, GEN, RED>(P, MQ, L, EF, r, SW);
     __syncthreads();
     if (tid < T) L.hold[tid] = from_bits(L.emax[1][tid]) <= P.tol;
     GPCG_PHASE(4);
@@ -982,12 +987,12 @@ __global__ void __launch_bounds__(
         red_solve<T, NT, VT, GEN>(P, MQ, L, *RL, r, L.raQ, L.rbQ, L.inQ, L.hold, SW, RX_, L.wQ,
                                   MQ.c ? L.cl : nullptr);
         GPCG_PHASE(5);
-        update_pass<T, NT, VT, false, GEN>(P, MQ, L, r, nullptr, th, EF, SW, RL->xa, RX_);
+        update_pass<T, NT, VT, false, GEN, true>(P, MQ, L, r, nullptr, th, EF, SW, RL->xa, RX_);
       } else if constexpr (NT == NTHREADS) {
       pcg_solve<T, VT, true, GEN>(P, MQ, L, x, r, p, q, z, L.raQ, L.rbQ, L.wQ, L.inQ,
                                   MQ.c ? L.cl : nullptr, SW, L.hold);
       GPCG_PHASE(5);
-      update_pass<T, NT, VT, false, GEN>(P, MQ, L, x, p, th, EF, SW);
+      update_pass<T, NT, VT, false, GEN, false>(P, MQ, L, x, p, th, EF, SW);
       }
     }
     if (g.rs == 0)
@@ -1066,12 +1071,12 @@ cudaError_t launch_fdpf_g(cudaStream_t st, int T, int grid, const FdpfParams& P,
     }
   }
   if constexpr (!GEN) {
-    if (nt != NTHREADS && T == 2 && reduced_form(P.precond, MP, MQ))
+    if (nt != NTHREADS && T == 2 && P.reduced)
       return nt == 512 ? launch_wide<VT, 512>(st, grid, P, MP, MQ, wide_bytes)
                        : launch_wide<VT, 1024>(st, grid, P, MP, MQ, wide_bytes);
   }
-  return reduced_form(P.precond, MP, MQ) ? launch_tiles<GEN, VT, true>(st, T, grid, P, MP, MQ)
-                                         : launch_tiles<GEN, VT, false>(st, T, grid, P, MP, MQ);
+  return P.reduced ? launch_tiles<GEN, VT, true>(st, T, grid, P, MP, MQ)
+                   : launch_tiles<GEN, VT, false>(st, T, grid, P, MP, MQ);
 }
 
 template <bool GEN, typename VT, bool RED>

@@ -85,7 +85,8 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   const bool f32 = c.opt.precision != GPCG_BATCHED_FP64;
   // the launch gpcg_n1_screen takes for as many scenarios, so that both round
   // the inner solve alike
-  const bool red = reduced_form(c.opt.precond, c.MPf, c.MQf);
+  const bool red = f32 ? reduced_form(c.opt.precond, c.MPf, c.MQf, c.opt.tol)
+                       : reduced_form(c.opt.precond, c.MPd, c.MQd);
   WideLaunch wl{NTHREADS, 0, T};
   if (red && !ext && !c.opt.tile && !c.opt.ctas_per_sm) {
     wl = wide_launch(n_out, c.num_sms, c.MPf.n, !f32);
@@ -157,6 +158,7 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   P.max_outer = c.opt.max_outer;
   P.max_inner = c.opt.max_inner;
   P.precond = c.opt.precond;
+  P.reduced = red;
   P.sc = ScenInfo{const_cast<int32_t*>(outages), lo, cnt, coef, nogen};
   P.th0 = c.th0; P.V0 = c.V0; P.c0 = c.c0; P.s0 = c.s0; P.ef0 = c.ef0;
   P.out_theta = theta; P.out_vm = vm; P.out_flow = flow; P.out_maxload = max_loading;

@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(PT) plain_fdpf_kernel(FdpfParams P, DevMatT<do
         const double d = W.x[k];
         W.th[i] += d;
         double2 u = EF[i];
-        rotate_ef<double>(d, d, u.x, u.y);
+        rotate_ef<double, false>(d, d, u.x, u.y);
         EF[i] = u;
       }
       if (!grid_barrier(W)) return;

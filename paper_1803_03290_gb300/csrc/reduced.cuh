@@ -21,8 +21,9 @@
 // stopping rule.  10,000 buses, all 13,500 outages, 1e-4 p.u.: with FP64 vectors
 // every iteration count is that of the five-vector PCG, with FP32 vectors they
 // are those counts too (3.81 P iterations a scenario; the five-vector PCG's FP32
-// residuals asked for 3.88).  Screen 79.9 -> 56.2 ms with FP32 vectors, 163 ->
-// 102 ms with FP64 ones.
+// residuals asked for 3.88).  Screen 163 -> 102 ms with FP64 vectors; 3,001 outages
+// at 1e-10 p.u. with FP32 ones 62.9 -> 41.0 ms.  reduced_form (fdpf.h) says which
+// screens take it.
 #pragma once
 #include "fdpf_ops.cuh"
 
