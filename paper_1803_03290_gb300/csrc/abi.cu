@@ -1341,7 +1341,7 @@ static gpcg_status run_fdpf(gpcg_ctx* c, cudaStream_t st, FdpfParams P, int T, i
   if (!P.fill) P.fill = T;
   const size_t rows = (size_t)std::max(c->MP.plan.n, c->MQ.plan.n) + 1;
   const bool plain_rows = !P.sc.gen_bus && !P.G.qmax;  // no extension rows
-  const size_t wide = one && plain_rows ? wide_shared(nt, rows * T * sizeof(VT)) : 0;
+  const size_t wide = one && plain_rows ? wide_shared<VT>(nt, rows * T * sizeof(VT)) : 0;
   if (wide) P.wr = nullptr;
   CUDA_TRY(cudaMemsetAsync(c->d_counter, 0, sizeof(int32_t), st));
   CUDA_TRY(launch_fdpf<VT>(st, T, slots, P, MP, MQ, zs ? Lo.vec_bytes : 0, nt, wide));

@@ -131,6 +131,12 @@ cudaError_t launch_fdpf(cudaStream_t st, int T, int grid, const FdpfParams& P,
 }
 
 template <typename VT>
+size_t wide_shared(int nt, size_t vec_bytes) {
+  const size_t room = nt == 1024 ? wide_room<VT, 1024>() : nt == 512 ? wide_room<VT, 512>() : 0;
+  return vec_bytes <= room ? vec_bytes : 0;
+}
+
+template <typename VT>
 int fdpf_max_blocks_per_sm(int T, bool gen, size_t zbytes, bool red) {
   if (gen) return zbytes ? 0 : fdpf_blocks_gen<VT>(T, red);
   return fdpf_blocks_g<false, VT>(T, zbytes, red);
@@ -155,6 +161,8 @@ template cudaError_t launch_fdpf<float>(cudaStream_t, int, int, const FdpfParams
                                         const DevMatT<float>&, const DevMatT<float>&, size_t, int, size_t);
 template cudaError_t launch_fdpf<double>(cudaStream_t, int, int, const FdpfParams&,
                                          const DevMatT<double>&, const DevMatT<double>&, size_t, int, size_t);
+template size_t wide_shared<float>(int, size_t);
+template size_t wide_shared<double>(int, size_t);
 template int fdpf_max_blocks_per_sm<float>(int, bool, size_t, bool);
 template int fdpf_max_blocks_per_sm<double>(int, bool, size_t, bool);
 template cudaError_t launch_apply<float>(cudaStream_t, int, const DevMatT<float>&, int, int,

@@ -106,13 +106,13 @@ inline bool reduced_form(int precond, const DevMatT<VT>& MP, const DevMatT<VT>& 
 struct WideLaunch {
   int nt, grid, fill;
 };
-// Dynamic shared memory a wide CTA may take for the vector of its solves (the
-// substitutions' gathers then wait on shared memory): what one CTA of 1,024
-// threads or two of 512 leave of an SM's 227 KB beside their own arrays.
-inline size_t wide_shared(int nt, size_t vec_bytes) {
-  const size_t room = nt == 1024 ? 200u << 10 : nt == 512 ? 88u << 10 : 0;
-  return vec_bytes <= room ? vec_bytes : 0;
-}
+// Dynamic shared memory a wide CTA takes for the vector of its solves (the
+// substitutions' gathers then wait on shared memory), 0 if the vector does not
+// fit: what one CTA of 1,024 threads or two of 512 leave of the SM's shared memory
+// beside the kernel's own arrays (27.8 KB for FP64 and 1,024 threads), as the
+// device and the kernel report it.
+template <typename VT>
+size_t wide_shared(int nt, size_t vec_bytes);
 // Grids of fewer rows than threads gain nothing (FP64 solves do from 512: the
 // dense tail's terms are split over the threads).  Kernel times for tolerance
 // 1e-10, CTAs of 256 / 512 / 1,024 threads: 97 outages of a 2,000-bus grid 2.04 /

@@ -1053,6 +1053,26 @@ cudaError_t launch_wide(cudaStream_t st, int grid, const FdpfParams& P, const De
   return cudaGetLastError();
 }
 
+// Dynamic shared memory a CTA of the wide kernel may take with 1024 / NT resident.
+template <typename VT, int NT>
+size_t wide_room() {
+  cudaFuncAttributes a;
+  int dev = 0, block = 0, sm = 0, reserved = 0;
+  if (cudaFuncGetAttributes(&a, fdpf_tiles_kernel<2, VT, false, false, true, NT>) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
+          cudaSuccess ||
+      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) !=
+          cudaSuccess) {
+    cudaGetLastError();  // the vector stays in global memory
+    return 0;
+  }
+  const long long room =
+      std::min<long long>(block, sm / (1024 / NT) - reserved) - (long long)a.sharedSizeBytes;
+  return room > 0 ? (size_t)room : 0;
+}
+
 template <bool GEN, typename VT>
 cudaError_t launch_fdpf_g(cudaStream_t st, int T, int grid, const FdpfParams& P,
                           const DevMatT<VT>& MP, const DevMatT<VT>& MQ, size_t zbytes = 0,

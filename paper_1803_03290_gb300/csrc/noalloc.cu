@@ -183,7 +183,8 @@ extern "C" gpcg_status gpcg_n1_screen_noalloc(gpcg_ctx* ctx, const int32_t* outa
   P.wth = sbase; P.we = sbase + slots * ss; P.wf = sbase + 2 * slots * ss;
   P.sstride = ss;
   const size_t vec = (size_t)(std::max(c.MPf.n, c.MQf.n) + 1) * T * vt;
-  const size_t shared = wide_shared(wl.nt, vec);
+  const size_t shared =
+      f32 ? wide_shared<float>(wl.nt, vec) : wide_shared<double>(wl.nt, vec);
   if (shared) P.wr = nullptr;
   ce = f32 ? launch_fdpf<float>(st, T, slots, P, c.MPf, c.MQf, 0, wl.nt, shared)
            : launch_fdpf<double>(st, T, slots, P, c.MPd, c.MQd, 0, wl.nt, shared);
