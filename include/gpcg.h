@@ -185,10 +185,14 @@ typedef struct {
  * stride from the call's scheduling order; the fastest is kept, a candidate
  * replacing the one before it only when 3 % faster: first the tile width
  * (2, 4, 8), then the tiles per SM, then the dense tail (248, 128, 64 rows
- * or none).  Choices are cached
+ * or none).  A list of at most eight scenarios per SM whose inner solves run in
+ * their reduced form (complete factor; FP64, or FP32 and tol <= 1e-9; no reactive
+ * limits) takes wider CTAs with a tile width and a number per SM of their own
+ * where neither is asked for: its probes are of that launch and choose the
+ * dense tail alone.  Choices are cached
  * for the process, keyed by the device (SM count, compute capability), the
  * grid's sizes (buses, branches, nonzeros of B', B'' and their factors),
- * precision, preconditioner, kernel kind and the power of two of the
+ * precision, preconditioner, kernel kind, CTA width and the power of two of the
  * scenario count; a context whose key is cached takes the cached choice
  * without probing.  Every choice gives the same results up to the rounding
  * of the inner solve. */

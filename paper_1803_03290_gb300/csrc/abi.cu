@@ -293,7 +293,8 @@ struct gpcg_ctx {
   // the autotuner's state: tiles per SM and dense-tail cap in use (0: not
   // chosen yet), how they were chosen (0 none, 1 probes, 2 cache) and the
   // power of two of the scenario count they were chosen for
-  int per_sm = 0, per_sm_used = 0, tuned = 0, tuned_bucket = -1;
+  int per_sm = 0, per_sm_used = 0, tile_used = 0, tuned = 0, tuned_bucket = -1;
+  int tuned_nt = 0;  // threads per CTA of the tuned launch
   bool tuned_red = false;  // the tuned kernel was the one with reduced inner solves
   int tail_rows_now = TAIL_ROWS;  // the cap the factors' tails are built with
   // the factors' dense-tail data of B' (0) and B'' (1): level schedule of the
@@ -927,6 +928,7 @@ extern "C" gpcg_status gpcg_create(const gpcg_grid* g, const gpcg_options* opt, 
   gpcg_ctx* c = new gpcg_ctx();
   c->opt = o;
   c->tile = o.tile;  // 0: chosen on the first batched screen
+  c->tile_used = o.tile;
   c->per_sm = o.ctas_per_sm;
   c->tail_rows_now = o.tail_rows > 0 ? o.tail_rows : (o.tail_rows < 0 ? 0 : TAIL_ROWS);
   c->n = n;
@@ -1209,7 +1211,7 @@ extern "C" gpcg_status gpcg_set_options(gpcg_ctx* c, const gpcg_options* opt) {
   drop_graph(c);
   c->opt = *opt;
   if (retune) {
-    c->tile = opt->tile;
+    c->tile = c->tile_used = opt->tile;
     c->per_sm = opt->ctas_per_sm;
     c->tuned = 0;
     c->tuned_bucket = -1;
@@ -1244,7 +1246,7 @@ extern "C" gpcg_status gpcg_get_info(const gpcg_ctx* c, gpcg_info* info) {
   info->blevels_p = (int)c->MP.plan.blev_ptr.size() - 1;
   info->blevels_q = (int)c->MQ.plan.blev_ptr.size() - 1;
   info->n_bridges = c->n_bridges;
-  info->tile = c->tile;
+  info->tile = c->tile_used;
   info->num_sms = c->num_sms;
   info->base_outer = c->base_outer;
   info->ctas_per_sm = c->per_sm_used;
@@ -1474,13 +1476,14 @@ static std::map<std::vector<long long>, TuneChoice> g_tune_cache;
 static_assert(KX == GPCG_MAX_EXT_ROWS, "extension rows of the kernel and of the C ABI");
 static_assert(TAIL_ROWS >= GPCG_MAX_TAIL_ROWS, "the kernel's tail buffer holds the largest tail");
 
-static std::vector<long long> tune_key(const gpcg_ctx* c, bool ext, bool red, int bucket) {
+static std::vector<long long> tune_key(const gpcg_ctx* c, bool ext, bool red,
+                                       const WideLaunch& wl, int bucket) {
   int major = 0, minor = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, c->device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, c->device);
   return {c->num_sms, major, minor, c->n, c->m,
           c->MP.plan.A.nnz(), c->MP.plan.L.nnz(), c->MQ.plan.A.nnz(), c->MQ.plan.L.nnz(),
-          c->opt.precision, c->opt.precond, ext, red, c->zs_allowed, bucket,
+          c->opt.precision, c->opt.precond, ext, red, wl.nt, wl.fill, c->zs_allowed, bucket,
           c->opt.tile, c->opt.ctas_per_sm, c->opt.tail_rows};
 }
 
@@ -1643,14 +1646,24 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
     return c->zs_allowed && !ext && (t == 2 || t == 4) && blocks(t, true) > 0;
   };
   if (!plain) {
+    // few scenarios, no knob asked for by the caller (a fixed tile width promises
+    // the same sums for any number of scenarios): wide CTAs
+    WideLaunch wl{NTHREADS, 0, 0};
+    if (red && !ext && !c->opt.tile && !c->opt.ctas_per_sm && !use_zs(2))
+      wl = wide_launch((int)S, c->num_sms, c->MP.plan.n, !f32);
+    const bool wide = wl.nt != NTHREADS;
     // tile width, tiles per SM and dense tail: fixed by the options, else
     // chosen by the autotuner for this power of two of the scenario count
+    // (wide CTAs have a tile width and a number per SM of their own)
     int bucket = 0;
     while (((size_t)1 << bucket) < S) ++bucket;
-    const bool knobs = !c->opt.tile || !c->opt.ctas_per_sm || !c->opt.tail_rows;
-    // (a tolerance on the other side of reduced_form's takes another kernel)
-    if (knobs && (bucket != c->tuned_bucket || red != c->tuned_red)) {
-      const std::vector<long long> key = tune_key(c, ext, red, bucket);
+    const bool knobs =
+        (!wide && (!c->opt.tile || !c->opt.ctas_per_sm)) || !c->opt.tail_rows;
+    // (a tolerance on the other side of reduced_form's, or a count on the other
+    // side of wide_launch's, takes another kernel)
+    if (knobs &&
+        (bucket != c->tuned_bucket || red != c->tuned_red || wl.nt != c->tuned_nt)) {
+      const std::vector<long long> key = tune_key(c, ext, red, wl, bucket);
       TuneChoice got{0, 0, 0};
       bool hit = false;
       {
@@ -1662,6 +1675,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
         auto max_ps = [&](int t) { return std::max(1, blocks(t, use_zs(t))); };
         std::vector<int> tiles = c->opt.tile ? std::vector<int>{c->opt.tile}
                                              : std::vector<int>{2, 4, 8};
+        if (wide) tiles = {2};
         if (ext)
           for (int& t : tiles) t = std::min(t, 8);
         // the probe every candidate screens: the call's outages, or when
@@ -1702,10 +1716,13 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
           Q.n_tiles = (nq + t - 1) / t;
           Q.order = c->d_porder + (np - nq);
           const bool z = use_zs(t);
-          const int sl = std::max(1, std::min(Q.n_tiles, c->num_sms * ps));
+          // (a list for wide CTAs is its own probe)
+          const int sl = std::max(
+              1, std::min(wide ? (timed ? wl.grid : 1) : Q.n_tiles, wide ? wl.grid : c->num_sms * ps));
+          Q.fill = wide ? wl.fill : 0;
           CUDA_TRY(cudaEventRecord(c->ev[3], st));
-          r = f32 ? run_fdpf<float>(c, st, Q, t, sl, f16, z)
-                  : run_fdpf<double>(c, st, Q, t, sl, false, z);
+          r = f32 ? run_fdpf<float>(c, st, Q, t, sl, f16, z, wl.nt)
+                  : run_fdpf<double>(c, st, Q, t, sl, false, z, wl.nt);
           if (r != GPCG_OK) return r;
           CUDA_TRY(cudaEventRecord(c->ev[2], st));
           CUDA_TRY(cudaEventSynchronize(c->ev[2]));
@@ -1732,7 +1749,7 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
           if (v > best * MARGIN) { best = v; bT = t; bP = ps; }
         }
         // (b) tiles per SM: the occupancy maximum and the two counts below it
-        if (!c->opt.ctas_per_sm)
+        if (!c->opt.ctas_per_sm && !wide)
           for (int ps = max_ps(bT) - 1; ps >= std::max(1, max_ps(bT) - 2); --ps) {
             double v = 0.0;
             gpcg_status r = rate(bT, ps, cap0, true, &v);
@@ -1753,34 +1770,32 @@ static gpcg_status n1_screen_impl(gpcg_ctx* c, const int32_t* outages, int32_t n
       }
       gpcg_status r = set_tail(c, got.tail);
       if (r != GPCG_OK) { cleanup(); return r; }
-      c->tile = got.tile;
-      c->per_sm = got.per_sm;
+      if (!wide) {
+        c->tile = got.tile;
+        c->per_sm = got.per_sm;
+      }
       c->tuned = hit ? 2 : 1;
       c->tuned_bucket = bucket;
       c->tuned_red = red;
+      c->tuned_nt = wl.nt;
     }
-    T = c->opt.tile ? c->opt.tile : (c->tile ? c->tile : 2);
+    T = c->opt.tile ? c->opt.tile : (c->tile && !wide ? c->tile : 2);
     if (ext) T = std::min(T, 8);  // the kernel with extension rows: tiles of 2, 4, 8
-    zs = use_zs(T);
-    // few scenarios, no knob asked for by the caller (a fixed tile width promises
-    // the same sums for any number of scenarios): wide CTAs
-    WideLaunch wl{NTHREADS, 0, T};
-    if (red && !ext && !zs && !c->opt.tile && !c->opt.ctas_per_sm) {
-      wl = wide_launch((int)S, c->num_sms, c->MP.plan.n, !f32);
-      if (wl.nt != NTHREADS) T = 2;
-    }
+    zs = !wide && use_zs(T);
     const int n_tiles = (int)((S + T - 1) / T);
     int per_sm = c->opt.ctas_per_sm ? c->opt.ctas_per_sm : c->per_sm;
     if (!c->opt.ctas_per_sm && per_sm > blocks(T, zs)) per_sm = blocks(T, zs);
     if (per_sm == 0 || (zs && per_sm > blocks(T, true))) per_sm = blocks(T, zs);
     per_sm = std::max(per_sm, 1);
-    c->per_sm_used = per_sm;
     slots = std::max(1, std::min(n_tiles, c->num_sms * per_sm));
-    if (wl.nt != NTHREADS) {
+    if (wide) {
+      per_sm = 1024 / wl.nt;
       nt = wl.nt;
       slots = wl.grid;
       P.fill = wl.fill;
     }
+    c->per_sm_used = per_sm;
+    c->tile_used = T;
     P.S = (int)S;
     P.n_tiles = n_tiles;
     P.order = c->d_order;
