@@ -614,17 +614,32 @@ static gpcg_status fill_values(gpcg_ctx* c, MatDev& M, const double* w, bool war
   return GPCG_OK;
 }
 
+// The columns of the reduced inner solves are worth having, not needed: where
+// their memory cannot be had, what was allocated since `from` is given back and the
+// solves take the PCG.  Other errors stay errors.
+static gpcg_status without_columns(MatDev& M, std::vector<void*>& own, size_t from,
+                                   cudaError_t ce) {
+  if (ce != cudaErrorMemoryAllocation) CUDA_TRY(ce);
+  cudaGetLastError();
+  for (; own.size() > from; own.pop_back()) cudaFree(own.back());
+  M.br_ptr = nullptr;
+  return GPCG_OK;
+}
+
 // The branches' columns of a complete factor whose values are built: rows
 // from the elimination tree (the parent of row i: the first entry after the
 // diagonal in its column), then values and scalars.  Synchronous.
 static gpcg_status build_branch_rows(gpcg_ctx* c, MatDev& M, std::vector<void*>& own) {
+  const size_t from = own.size();
+  cudaError_t ce;
   const MatrixPlan& P = M.plan;
   const int m = c->m;
   std::vector<int32_t> parent(std::max(P.n, 1), -1), ptr(m + 1, 0);
   for (int i = 0; i < P.n; ++i)
     if (P.U.ptr[i] + 1 < P.U.ptr[i + 1]) parent[i] = P.U.idx[P.U.ptr[i] + 1];
-  CUDA_TRY(upload(own, &M.parent, parent.data(), parent.size()));
-  CUDA_TRY(dalloc(own, &M.br_ptr, (size_t)m + 1));
+  if ((ce = upload(own, &M.parent, parent.data(), parent.size())) != cudaSuccess ||
+      (ce = dalloc(own, &M.br_ptr, (size_t)m + 1)) != cudaSuccess)
+    return without_columns(M, own, from, ce);
   launch_branch_count(0, m, c->G.f, c->G.t, M.row_of_bus, M.parent, M.br_ptr + 1);
   CUDA_TRY(cudaMemcpy(ptr.data() + 1, M.br_ptr + 1, (size_t)m * 4, cudaMemcpyDeviceToHost));
   size_t total = 0;
@@ -632,15 +647,14 @@ static gpcg_status build_branch_rows(gpcg_ctx* c, MatDev& M, std::vector<void*>&
     total += (size_t)ptr[l + 1];
     ptr[l + 1] = (int32_t)total;
   }
-  if (total > (size_t)INT32_MAX) {  // beyond the 32-bit positions: no columns
-    M.br_ptr = nullptr;
-    return GPCG_OK;
-  }
+  if (total > (size_t)INT32_MAX)  // beyond the 32-bit positions: no columns
+    return without_columns(M, own, from, cudaErrorMemoryAllocation);
   CUDA_TRY(cudaMemcpy(M.br_ptr, ptr.data(), ((size_t)m + 1) * 4, cudaMemcpyHostToDevice));
-  CUDA_TRY(dalloc(own, &M.br_row, total));
-  CUDA_TRY(dalloc(own, &M.br_fv, total));
-  CUDA_TRY(dalloc(own, &M.br_fm, total));
-  CUDA_TRY(dalloc(own, &M.br_sc, (size_t)m * SC_N));
+  if ((ce = dalloc(own, &M.br_row, total)) != cudaSuccess ||
+      (ce = dalloc(own, &M.br_fv, total)) != cudaSuccess ||
+      (ce = dalloc(own, &M.br_fm, total)) != cudaSuccess ||
+      (ce = dalloc(own, &M.br_sc, (size_t)m * SC_N)) != cudaSuccess)
+    return without_columns(M, own, from, ce);
   return GPCG_OK;
 }
 
@@ -781,13 +795,18 @@ static gpcg_status build_matrices(gpcg_ctx* c) {
       }
       int32_t *d_ptr, *d_row;
       double *d_f, *d_ff;
-      CUDA_TRY(upload(own, &d_ptr, ptr.data(), ptr.size()));
-      CUDA_TRY(upload(own, &d_row, row.data(), row.size()));
-      CUDA_TRY(dalloc(own, &d_f, row.size()));
-      CUDA_TRY(dalloc(own, &d_ff, (size_t)c->n));
-      launch_bus_cols(0, c->n, c->G.adj_ptr, M.xrow, M.xval, M.U.view<double>(), P.n, M.inv_diag,
-                      d_ptr, d_row, d_f, d_ff);
-      M.bus = BusCols{d_ptr, d_row, d_f, d_ff};
+      const size_t from = own.size();
+      cudaError_t ce;
+      if ((ce = upload(own, &d_ptr, ptr.data(), ptr.size())) != cudaSuccess ||
+          (ce = upload(own, &d_row, row.data(), row.size())) != cudaSuccess ||
+          (ce = dalloc(own, &d_f, row.size())) != cudaSuccess ||
+          (ce = dalloc(own, &d_ff, (size_t)c->n)) != cudaSuccess) {
+        if ((st = without_columns(M, own, from, ce)) != GPCG_OK) return st;
+      } else {
+        launch_bus_cols(0, c->n, c->G.adj_ptr, M.xrow, M.xval, M.U.view<double>(), P.n,
+                        M.inv_diag, d_ptr, d_row, d_f, d_ff);
+        M.bus = BusCols{d_ptr, d_row, d_f, d_ff};
+      }
     }
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaDeviceSynchronize());
@@ -2014,9 +2033,14 @@ static gpcg_status ensure_adj_matrix(gpcg_ctx* c) {
   if (M.br_ptr) {  // the branches' columns: rows shared, values its own
     int32_t total = 0;
     CUDA_TRY(cudaMemcpy(&total, M.br_ptr + c->m, sizeof total, cudaMemcpyDeviceToHost));
-    CUDA_TRY(dalloc(own, &M.br_fv, (size_t)total));
-    CUDA_TRY(dalloc(own, &M.br_fm, (size_t)total));
-    CUDA_TRY(dalloc(own, &M.br_sc, (size_t)c->m * SC_N));
+    const size_t from = own.size();
+    cudaError_t ce;
+    if ((ce = dalloc(own, &M.br_fv, (size_t)total)) != cudaSuccess ||
+        (ce = dalloc(own, &M.br_fm, (size_t)total)) != cudaSuccess ||
+        (ce = dalloc(own, &M.br_sc, (size_t)c->m * SC_N)) != cudaSuccess) {
+      const gpcg_status st = without_columns(M, own, from, ce);
+      if (st != GPCG_OK) return st;
+    }
   }
   CUDA_TRY(dalloc(own, &M.th_val, M.n_th));
   CUDA_TRY(dalloc(own, &M.th_val32, M.n_th));
