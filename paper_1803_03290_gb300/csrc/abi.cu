@@ -78,6 +78,9 @@ static gpcg_status fail(gpcg_status st, const char* fmt, ...) {
   vsnprintf(buf, sizeof buf, fmt, ap);
   va_end(ap);
   g_err = buf;
+  // the runtime keeps the error of a failed call for the next launch check, which
+  // would report it for a call that did nothing wrong
+  if (st == GPCG_ERR_CUDA || st == GPCG_ERR_OOM) cudaGetLastError();
   return st;
 }
 

@@ -33,6 +33,7 @@ gpcg_status err(gpcg_status st, const char* fmt, ...) {
   std::vsnprintf(buf, sizeof buf, fmt, ap);
   va_end(ap);
   set_last_error(buf);
+  if (st == GPCG_ERR_CUDA) cudaGetLastError();  // not for the next call to find
   return st;
 }
 
