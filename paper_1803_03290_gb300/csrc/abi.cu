@@ -340,6 +340,45 @@ static cudaError_t upload(std::vector<void*>& own, X** p, const X* src, size_t c
   return cudaMemcpy(*p, src, count * sizeof(X), cudaMemcpyHostToDevice);
 }
 
+// Arrays that are made together: one allocation and one copy to the device.  (A
+// context has about a hundred small tables; an allocation and a copy of their
+// own are 10 us for each, and as much again to free them.)
+class Pack {
+ public:
+  template <typename X>
+  void add(X** p, const X* src, size_t count) {
+    at_.push_back({(void**)p, place(up_), true});
+    const size_t off = at_.back().off;
+    up_ = off + std::max<size_t>(count, 1) * sizeof(X);
+    host_.resize(up_);
+    if (count) std::memcpy(host_.data() + off, src, count * sizeof(X));
+  }
+  template <typename X>
+  void add(X** p, size_t count) {  // filled on the device
+    at_.push_back({(void**)p, place(more_), false});
+    more_ = at_.back().off + std::max<size_t>(count, 1) * sizeof(X);
+  }
+  cudaError_t commit(std::vector<void*>& own) {
+    char* d = nullptr;
+    const size_t up = place(up_);
+    cudaError_t ce = dalloc(own, &d, up + more_);
+    if (ce != cudaSuccess) return ce;
+    for (const Item& i : at_) *i.p = d + (i.up ? i.off : up + i.off);
+    return up_ ? cudaMemcpy(d, host_.data(), up_, cudaMemcpyHostToDevice) : cudaSuccess;
+  }
+
+ private:
+  struct Item {
+    void** p;
+    size_t off;
+    bool up;
+  };
+  static size_t place(size_t b) { return (b + 255) / 256 * 256; }
+  std::vector<Item> at_;
+  std::vector<char> host_;
+  size_t up_ = 0, more_ = 0;
+};
+
 static void free_list(std::vector<void*>& v) {
   for (void* p : v) cudaFree(p);
   v.clear();
@@ -443,9 +482,8 @@ static void ell_fill(cudaStream_t st, EllDev& D, const double* csr_val) {
 // the levels' bounds in it): entries of row i are the positions [ptr_[i], ...)
 // of `A` without the diagonal, val_of maps them to positions of L's values.
 template <typename Entries>
-static cudaError_t sub_upload(std::vector<void*>& own, const std::vector<int32_t>& rows,
-                              const std::vector<int32_t>& ptr, int pad, const MatrixPlan& P,
-                              Entries entries, SubDev& D) {
+static void sub_pack(Pack& pack, const std::vector<int32_t>& rows, const std::vector<int32_t>& ptr,
+                     int pad, const MatrixPlan& P, Entries entries, SubDev& D) {
   const int n = (int)rows.size();
   std::vector<int32_t> order(rows);
   std::vector<std::pair<int, int>> ent;
@@ -475,19 +513,18 @@ static cudaError_t sub_upload(std::vector<void*>& own, const std::vector<int32_t
   }
   D.n = n;
   D.nc = (int)ccol.size();
-  cudaError_t ce;
-  if ((ce = upload(own, &D.rc, rc.data(), rc.size())) != cudaSuccess) return ce;
-  if ((ce = upload(own, &D.col, col.data(), col.size())) != cudaSuccess) return ce;
-  if ((ce = upload(own, &D.src, src.data(), src.size())) != cudaSuccess) return ce;
-  if ((ce = upload(own, &D.dsrc, dsrc.data(), dsrc.size())) != cudaSuccess) return ce;
-  if ((ce = upload(own, &D.ccol, ccol.data(), ccol.size())) != cudaSuccess) return ce;
-  if ((ce = upload(own, &D.csrc, csrc.data(), csrc.size())) != cudaSuccess) return ce;
-  if ((ce = dalloc(own, &D.cval, csrc.size())) != cudaSuccess) return ce;
-  if ((ce = dalloc(own, &D.cval32, csrc.size())) != cudaSuccess) return ce;
-  if ((ce = dalloc(own, &D.val, src.size())) != cudaSuccess) return ce;
-  if ((ce = dalloc(own, &D.val32, src.size())) != cudaSuccess) return ce;
-  if ((ce = dalloc(own, &D.id, dsrc.size())) != cudaSuccess) return ce;
-  return dalloc(own, &D.id32, dsrc.size());
+  pack.add(&D.rc, rc.data(), rc.size());
+  pack.add(&D.col, col.data(), col.size());
+  pack.add(&D.src, src.data(), src.size());
+  pack.add(&D.dsrc, dsrc.data(), dsrc.size());
+  pack.add(&D.ccol, ccol.data(), ccol.size());
+  pack.add(&D.csrc, csrc.data(), csrc.size());
+  pack.add(&D.cval, csrc.size());
+  pack.add(&D.cval32, csrc.size());
+  pack.add(&D.val, src.size());
+  pack.add(&D.val32, src.size());
+  pack.add(&D.id, dsrc.size());
+  pack.add(&D.id32, dsrc.size());
 }
 
 static void sub_fill(cudaStream_t st, SubDev& D, const double* l_val, const double* inv_diag) {
@@ -516,13 +553,14 @@ static gpcg_status alloc_tail(gpcg_ctx* c, MatDev& M, int which, int cap) {
   {
     std::vector<int32_t> pos(P.L.nnz());  // position in U -> position in L
     for (int k = 0; k < P.L.nnz(); ++k) pos[P.l_to_u[k]] = k;
-    CUDA_TRY(sub_upload(own, P.tblev_rows, P.tblev_ptr, P.n, P,
-                        [&](int i, std::vector<std::pair<int, int>>& e) {
-                          e.clear();
-                          for (int k = P.U.ptr[i] + 1; k < P.U.ptr[i + 1]; ++k)
-                            e.push_back({P.U.idx[k], pos[k]});
-                        },
-                        M.bwd));
+    Pack pack;
+    sub_pack(pack, P.tblev_rows, P.tblev_ptr, P.n, P,
+             [&](int i, std::vector<std::pair<int, int>>& e) {
+               e.clear();
+               for (int k = P.U.ptr[i] + 1; k < P.U.ptr[i + 1]; ++k)
+                 e.push_back({P.U.idx[k], pos[k]});
+             },
+             M.bwd);
     std::vector<int32_t> tp(1, 0), tc, ts;
     for (int i = P.tail_row0; i < P.n; ++i) {
       for (int k = P.L.ptr[i]; k < P.L.ptr[i + 1]; ++k)
@@ -533,11 +571,12 @@ static gpcg_status alloc_tail(gpcg_ctx* c, MatDev& M, int which, int cap) {
       tp.push_back((int32_t)tc.size());
     }
     M.n_th = (int)tc.size();
-    CUDA_TRY(upload(own, &M.th_ptr, tp.data(), tp.size()));
-    CUDA_TRY(upload(own, &M.th_col, tc.data(), tc.size()));
-    CUDA_TRY(upload(own, &M.th_src, ts.data(), ts.size()));
-    CUDA_TRY(dalloc(own, &M.th_val, tc.size()));
-    CUDA_TRY(dalloc(own, &M.th_val32, tc.size()));
+    pack.add(&M.th_ptr, tp.data(), tp.size());
+    pack.add(&M.th_col, tc.data(), tc.size());
+    pack.add(&M.th_src, ts.data(), ts.size());
+    pack.add(&M.th_val, tc.size());
+    pack.add(&M.th_val32, tc.size());
+    CUDA_TRY(pack.commit(own));
   }
   const size_t nt = (size_t)(P.n - P.tail_row0);
   CUDA_TRY(dalloc(own, &M.xc, nt * nt));
@@ -728,8 +767,10 @@ static gpcg_status build_matrix(gpcg_ctx* c, MatDev& M, int which,
     CUDA_TRY(ell_upload(own, ell_from_rows(ru, KU, P.n), M.U));
     std::vector<int32_t> rows(P.n);
     for (int i = 0; i < P.n; ++i) rows[i] = i;
-    CUDA_TRY(sub_upload(own, rows, P.lev_ptr, P.n, P,
-                        [&](int i, std::vector<std::pair<int, int>>& e) { e = rl[i]; }, M.fwd));
+    Pack pack;
+    sub_pack(pack, rows, P.lev_ptr, P.n, P,
+             [&](int i, std::vector<std::pair<int, int>>& e) { e = rl[i]; }, M.fwd);
+    CUDA_TRY(pack.commit(own));
     for (EllDev* E : {&M.L, &M.U}) {
       CUDA_TRY(dalloc(own, &E->valh, E->nslot));
       CUDA_TRY(dalloc(own, &E->ovalh, E->nover));
@@ -815,8 +856,12 @@ static gpcg_status build_matrices(gpcg_ctx* c) {
     CUDA_TRY(cudaDeviceSynchronize());
   }
   {
-    // the half-steps' bus tables
+    // the half-steps' bus tables and the DC screen's output maps
     auto& own = c->mat_owned;
+    Pack pack;
+    int4* d_md[2];
+    int32_t *d_nbr[2], *d_br[2];
+    double2 *d_gb[2], *d_yd[2], *d_pq[2];
     for (int which = 0; which < 2; ++which) {
       const MatrixPlan& P = which ? c->MQ.plan : c->MP.plan;
       const int n = P.n;
@@ -844,27 +889,27 @@ static gpcg_status build_matrices(gpcg_ctx* c) {
         }
         pq[k] = c->pq[b];
       }
-      BusTab& tab = which ? c->tabQ : c->tabP;
-      int4* d_md;
-      int32_t *d_nbr, *d_br;
-      double2 *d_gb, *d_yd, *d_pq;
-      CUDA_TRY(upload(own, &d_md, md.data(), md.size()));
-      CUDA_TRY(upload(own, &d_nbr, nbr.data(), nbr.size()));
-      CUDA_TRY(upload(own, &d_br, br.data(), br.size()));
-      CUDA_TRY(upload(own, &d_pq, pq.data(), pq.size()));
-      CUDA_TRY(dalloc(own, &d_gb, nbr.size()));
-      CUDA_TRY(dalloc(own, &d_yd, (size_t)n));
-      launch_adj_values(0, (int)br.size(), d_br, c->G.cf, c->G.g, c->G.by, d_gb, nullptr, nullptr);
-      launch_gather_pair(0, n, d_md, c->G.ydiag, d_yd);
-      CUDA_TRY(cudaGetLastError());
-      tab = BusTab{d_md, d_nbr, d_gb, d_yd, d_pq, n};
+      pack.add(&d_md[which], md.data(), md.size());
+      pack.add(&d_nbr[which], nbr.data(), nbr.size());
+      pack.add(&d_br[which], br.data(), br.size());
+      pack.add(&d_pq[which], pq.data(), pq.size());
+      pack.add(&d_gb[which], nbr.size());
+      pack.add(&d_yd[which], (size_t)n);
     }
     std::vector<int2> rp(c->n), ends(c->m);
     const std::vector<int32_t>& row = c->MP.plan.row_of_bus;
     for (int b = 0; b < c->n; ++b) rp[c->user_of[b]] = make_int2(row[b], c->pre[b]);
     for (int k = 0; k < c->m; ++k) ends[k] = make_int2(row[c->f[k]], row[c->t[k]]);
-    CUDA_TRY(upload(own, &c->row_pre, rp.data(), rp.size()));
-    CUDA_TRY(upload(own, &c->br_rows, ends.data(), ends.size()));
+    pack.add(&c->row_pre, rp.data(), rp.size());
+    pack.add(&c->br_rows, ends.data(), ends.size());
+    CUDA_TRY(pack.commit(own));
+    for (int k = 0; k < 2; ++k) {
+      const int n = k ? c->MQ.plan.n : c->MP.plan.n;
+      launch_adj_values(0, n * KG, d_br[k], c->G.cf, c->G.g, c->G.by, d_gb[k], nullptr, nullptr);
+      launch_gather_pair(0, n, d_md[k], c->G.ydiag, d_yd[k]);
+      (k ? c->tabQ : c->tabP) = BusTab{d_md[k], d_nbr[k], d_gb[k], d_yd[k], d_pq[k], n};
+    }
+    CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaDeviceSynchronize());
   }
   c->planned_precond = c->opt.precond;

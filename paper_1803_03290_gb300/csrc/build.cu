@@ -389,7 +389,8 @@ void launch_inv_diag(cudaStream_t st, int n, const int32_t* pos, const double* l
 }
 // X = inverse of the factor's tail block L_tt (rows and columns
 // [t0, t0 + nt) of L, lower triangular): column c of X by forward
-// substitution of L_tt x = e_c, one thread per column, in FP64.  Written
+// substitution of L_tt x = e_c, one thread per column (as many CTAs as leave no
+// thread two of the serial chains), in FP64.  Written
 // column-major (xc[c nt + i] = X_ic) and row-major (xr[i nt + c] = X_ic),
 // zeros above the diagonal, in FP64 (xr optional) and FP32.
 // With lsc (the scaled factor Ls = L D^-1) the block inverted is the one
@@ -399,7 +400,8 @@ __global__ void tail_inverse_kernel(int t0, int nt, const int32_t* __restrict__ 
                                     const double* __restrict__ l_val,
                                     const double* __restrict__ lsc, double* xc, double* xr,
                                     float* xc32, float* xr32) {
-  for (int c = threadIdx.x; c < nt; c += blockDim.x) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < nt) {
     // xc holds the column in FP64 while it is built (its earlier entries
     // are the unknowns solved before)
     for (int i = 0; i < nt; ++i) {
@@ -426,8 +428,8 @@ __global__ void tail_inverse_kernel(int t0, int nt, const int32_t* __restrict__ 
 }
 
 // The same for the adjoint (see ic_narrow_kernel): a warp per column, the row's
-// terms spread over its threads (a thread per column in one CTA takes 1 ms for 232
-// rows: each term waits for its own loads).
+// terms spread over its threads (a thread per column waits for the loads of each
+// term: about 1 ms for 232 rows).
 constexpr int TI_WARPS = 4;
 __global__ void __launch_bounds__(32 * TI_WARPS)
     tail_inverse_warp_kernel(int t0, int nt, const int32_t* __restrict__ l_ptr,
@@ -466,7 +468,8 @@ void launch_tail_inverse(cudaStream_t st, int t0, int nt, const int32_t* l_ptr,
                          const int32_t* l_idx, const double* l_val, const double* lsc, double* xc,
                          double* xr, float* xc32, float* xr32) {
   if (nt > 0)
-    tail_inverse_kernel<<<1, 128, 0, st>>>(t0, nt, l_ptr, l_idx, l_val, lsc, xc, xr, xc32, xr32);
+    tail_inverse_kernel<<<(nt + 127) / 128, 128, 0, st>>>(t0, nt, l_ptr, l_idx, l_val, lsc, xc, xr,
+                                                       xc32, xr32);
 }
 void launch_tail_inverse_warp(cudaStream_t st, int t0, int nt, const int32_t* l_ptr,
                               const int32_t* l_idx, const double* l_val, double* xc, double* xr,
