@@ -195,7 +195,9 @@ typedef struct {
  * precision, preconditioner, kernel kind, CTA width and the power of two of the
  * scenario count; a context whose key is cached takes the cached choice
  * without probing.  Every choice gives the same results up to the rounding
- * of the inner solve. */
+ * of the inner solve.  A list split into parts gives the bits of one call when
+ * tile and tail_rows are fixed by the options: left to the library, a part may
+ * be tuned to other knobs or small enough for the wider CTAs. */
 
 /* Sizes of the structures built by gpcg_create. */
 typedef struct {
@@ -282,6 +284,12 @@ GPCG_API gpcg_status gpcg_base_solve(gpcg_ctx *ctx, double *theta, double *vm,
  *   overload[n_out][GPCG_MASK_WORDS(n_branch)] the same branches as a bit
  *                                             mask: bit k % 32 of word
  *                                             k / 32 is set for branch k
+ * A scenario with status GPCG_SCEN_MAXITER or GPCG_SCEN_DIVERGED has no
+ * solution to report: its theta, vm, flow, max_loading, n_overload and overload
+ * are those of the last iterate, which the iteration's growing errors have
+ * brought there -- the rounding of the inner solve decides them, and for a few
+ * outages which of the two statuses it is.  They are the same for every call of
+ * one kernel and one set of knobs, and say nothing about the outage.
  * n_out may be 0.  An outage index outside [0, n_branch) is INVALID_ARG.
  * Requires a successful gpcg_base_solve (else NOT_READY).  A scenario that
  * fails to converge never fails the call: see status[].

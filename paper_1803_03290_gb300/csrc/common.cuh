@@ -62,8 +62,7 @@ struct Ell {
 };
 
 // The branches' columns in the complete Cholesky factor M = L L^T of a
-// base-case matrix, built once per factor (reduced_cg in fdpf_ops.cuh says
-// what for).  For branch l with v = c e_from - e_to on the matrix's rows, and
+// base-case matrix, built once per factor (reduced.cuh says what for).  For branch l with v = c e_from - e_to on the matrix's rows, and
 // v_m its part on the main island (v itself unless l is a bridge), the rows
 // where L^-1 v can be nonzero are the ancestors of its ends in the
 // elimination tree: positions [ptr[l], ptr[l + 1]) of row (ascending), with

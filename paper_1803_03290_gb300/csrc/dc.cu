@@ -183,12 +183,14 @@ __global__ void __launch_bounds__(NTHREADS, FDPF_MIN_BLOCKS)
 // coef pg over the generators), so L^-1 of it is f = f0 + coef fg with f0 =
 // L^-1 P and fg = L^-1 pg the same for every scenario of the call; the outage
 // adds a multiple of a column that is sparse and kept per branch (BranchCols):
-//   B_s^-1 rhs = L^-T (f + t L^-1 v),       t = w u / (1 - w v.M^-1 v),
-// u = v.M^-1 rhs = (L^-1 v).f.  For a bridge, injections of the island that
-// sum to zero leave the main island's angles alone (no flow over the bridge),
-// so instead of masking P the island's total is withdrawn at its end of the
-// bridge: that is f + t (L^-1 v_m - L^-1 v) with the same t, which makes the
-// bridge's flow zero.
+//   B_s^-1 rhs = L^-T (f + t L^-1 v),       t = w u / (1 - w v.M^-1 v_m),
+// u = v.M^-1 rhs = (L^-1 v).f, v_m = v unless the branch is a bridge.  For a
+// bridge v_m is v without the island's end and v.M^-1 v_m = 0, so that t = w u,
+// the flow over the bridge (v.M^-1 v is 1 / w there: not the term to divide by).
+// Injections of the island that sum to zero leave the main island's angles alone
+// (no flow over the bridge), so instead of masking P the island's total is
+// withdrawn at its end of the bridge: that is f + t (L^-1 v_m - L^-1 v), which
+// makes the bridge's flow zero.
 // Bound by the loads and stores of one pass over the rows and one over the
 // branches: 13,500 outages of a 10,000-bus grid with every output 29.8 ms by
 // the PCG (1.85 iterations of three passes over five vectors), 4.6 ms here.
